@@ -24,6 +24,7 @@
 #include "gemm_kernel.cuh"
 #include "kcluster_kernel.cuh"
 #include "attention_kernel.cuh"
+#include "attention_decode_kernel.cuh"
 #include "norm_kernel.cuh"
 #include "tune_kernels.cuh"
 
@@ -2053,6 +2054,69 @@ fact_status_t encode_map_bthd(fact_handle_t h, CUtensorMap* map, const void* bas
   }
   return FACT_OK;
 }
+
+// Attention of few query rows (attention_decode_kernel.cuh).  `strides`: batch, token and head of Q, K, V, O.
+fact_status_t attention_decode(fact_handle_t h, int64_t batch, int64_t seq_q, int64_t seq_kv, int64_t heads_q, int64_t heads_kv,
+                               int64_t head_dim, const void* Q, const int64_t (&strides)[12], const void* K, const void* V,
+                               void* O, float scale, cudaStream_t stream) {
+  CUtensorMap tk, tv;
+  auto bs = [&](int64_t s, int64_t fallback) { return (batch > 1 && s > 0) ? s : std::max<int64_t>(fallback, 8); };
+  fact_status_t st = encode_map_bthd(h, &tk, K, head_dim, heads_kv, seq_kv, batch, strides[5], strides[4],
+                                     bs(strides[3], strides[4] * seq_kv), kDecBlockK);
+  if (st == FACT_OK)
+    st = encode_map_bthd(h, &tv, V, head_dim, heads_kv, seq_kv, batch, strides[8], strides[7],
+                         bs(strides[6], strides[7] * seq_kv), kDecBlockK);
+  if (st != FACT_OK) return st;
+  DecodeParams p;
+  memset(&p, 0, sizeof p);
+  p.Q = reinterpret_cast<const __nv_bfloat16*>(Q);
+  p.O = reinterpret_cast<__nv_bfloat16*>(O);
+  p.q_sb = strides[0];
+  p.q_st = strides[1];
+  p.q_sh = strides[2];
+  p.o_sb = strides[9];
+  p.o_st = strides[10];
+  p.o_sh = strides[11];
+  p.Tq = (int)seq_q;
+  p.Tk = (int)seq_kv;
+  p.Hkv = (int)heads_kv;
+  p.group = (int)(heads_q / heads_kv);
+  p.rows = p.Tq * p.group;
+  p.scale_log2 = (float)((scale > 0.f ? (double)scale : 1.0 / std::sqrt((double)head_dim)) * 1.4426950408889634);
+  p.status = h->d_status;
+  const long long pairs = (long long)batch * heads_kv;
+  const long long blocks = (seq_kv + kDecBlockK - 1) / kDecBlockK;
+  // CTAs per problem.  More of them only where they have SMs of their own, with the large ring: three quarters of the
+  // SMs is what clusters of 8 can fill at once (15 of them; at 16 the sixteenth is a second wave: 21.2 us instead of 14.1
+  // with clusters of 4 for 2 sequences x 8192 keys x 8 heads of 128).  The cluster's merge costs as much as about six
+  // blocks (1.2 us): 260 keys 3.6 us in one CTA, 4.3 in two; 1000 keys 6.3 / 5.6 / 4.7 / 4.5 in 1 / 2 / 4 / 8; 8192 keys
+  // 36.2 / 21.0 / 13.0 / 9.7.  A head alone on an SM streams 64 keys in 0.27 us with the large ring, 0.36 with the small.
+  p.splits = 1;
+  if (blocks >= 12)
+    while (p.splits < 8 && 2 * pairs * p.splits <= h->sm_count * 3 / 4) p.splits *= 2;
+  const uint32_t ring = pairs * p.splits <= h->sm_count ? 2 * kDecRingBytes : kDecRingBytes;
+  p.stages = (int)(ring / dec_stage_bytes((int)head_dim));
+  if (pairs * p.splits > 0x7fffffffLL) return FACT_ERR_UNSUPPORTED;
+  const int nt = p.rows <= 8 ? 1 : (p.rows <= 16 ? 2 : 4);
+  typedef void (*Kern)(CUtensorMap, CUtensorMap, DecodeParams);
+  static const Kern kerns[2][3] = {
+      {fact_attention_decode_kernel<64, 1>, fact_attention_decode_kernel<64, 2>, fact_attention_decode_kernel<64, 4>},
+      {fact_attention_decode_kernel<128, 1>, fact_attention_decode_kernel<128, 2>, fact_attention_decode_kernel<128, 4>}};
+  if (!h->configured_mask.test(31)) {
+    for (const auto& row : kerns)
+      for (Kern k : row) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(2 * kDecRingBytes + kDecCtrlBytes));
+        if (e != cudaSuccess) return cuda_fail(h, "cudaFuncSetAttribute(attention, few rows)", e);
+      }
+    h->configured_mask.set(31);
+  }
+  cudaError_t e = launch_pdl(h, kerns[head_dim == 128][nt == 4 ? 2 : nt - 1], (unsigned)(pairs * p.splits), (unsigned)kDecThreads,
+                             (size_t)(ring + kDecCtrlBytes), stream, p.splits, tk, tv, p);
+  if (e != cudaSuccess) return cuda_fail(h, "attention launch (few rows)", e);
+  h->launches++;
+  return FACT_OK;
+}
 }  // namespace
 
 fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int64_t seq_kv, int64_t heads_q,
@@ -2081,6 +2145,12 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return FACT_ERR_CUDA;
   if (dev != h->device && cudaSetDevice(h->device) != cudaSuccess) return FACT_ERR_CUDA;
+  // Few query rows per key/value head: the kernel that streams the keys once for all of them.
+  if ((!causal || seq_kv == 1) && seq_q * (heads_q / heads_kv) <= kDecMaxRows) {
+    const fact_status_t ds = attention_decode(h, batch, seq_q, seq_kv, heads_q, heads_kv, head_dim, Q, strides, K, V, O, scale, stream);
+    if (dev != h->device) cudaSetDevice(dev);
+    return ds;
+  }
   CUtensorMap tq, tk, tv, to;
   auto bs = [&](int64_t s, int64_t fallback) { return (batch > 1 && s > 0) ? s : std::max<int64_t>(fallback, 8); };
   // keys go in blocks of 128 at head_dim 64 and of 64 at head_dim 128 (the kernel's tensor-memory budget)
