@@ -1,4 +1,8 @@
-"""ctypes binding of libfact: argument marshalling only.
+"""Binding of libfact: argument marshalling only.
+
+An ordinary call (plain CUDA tensors, the library's own configuration, the current stream) is marshalled by the
+extension ``_fact_bind``; what it does not take -- a configuration or a stream of the caller's, a workspace that has to
+grow, arguments that are wrong -- goes through ctypes here, whose checks say what is wrong.
 
 Every step of the computation runs in the CUDA library; PyTorch is used for
 device memory (tensors, the split-K workspace) and for the current stream.
@@ -11,6 +15,8 @@ The raw C entry points are available under their C names on ``lib()``
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 from ctypes import POINTER, Structure, byref, c_char_p, c_double, c_float, c_int, c_int64, c_size_t, c_void_p
 from pathlib import Path
 from typing import Optional
@@ -29,6 +35,7 @@ EPILOGUES = {"NONE": 0, "BIAS": 1, "BIAS_RELU": 2, "BIAS_GELU_TANH": 3, "SILU_GA
              "BIAS_SOFTMAX": 6}
 LAYOUTS = {"KN": 0, "NK": 1}
 OUT_TYPES = {torch.bfloat16: 0, torch.float32: 1, "bf16": 0, "f32": 1}
+_OUT_CODES = {torch.bfloat16: 0, torch.float32: 1}
 OPS = {"gemm": 0, "gemm_batched": 1, "gemm_splitk": 2, "linear": 3, "linear_fp8": 4}
 
 # every symbol include/fact.h declares
@@ -182,6 +189,24 @@ def lib() -> ctypes.CDLL:
     return L
 
 
+_bind = None
+
+
+def bind():
+    """The extension that marshals ordinary calls (built in-tree with libfact.so)."""
+    global _bind
+    if _bind is None:
+        lib()
+        path = _PKG / "_fact_bind.so"
+        if not path.exists():
+            raise RuntimeError(f"{path} is missing: build it with `python -m paper_2604_26666_b200.build`")
+        loader = importlib.machinery.ExtensionFileLoader("_fact_bind", str(path))
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fact_bind", loader))
+        loader.exec_module(module)
+        _bind = module
+    return _bind
+
+
 def _check(code: int, where: str, handle=None):
     if code != OK:
         if code == 6 and handle is not None:
@@ -322,6 +347,8 @@ class Handle:
         self._ws: Optional[torch.Tensor] = None
         self._ws_streams: dict = {}
         self._ws_cache: dict = {}
+        self._hp = int(self._h.value or 0)
+        self._bind = bind()
         table = _PKG / "tuned_b200.txt"
         if load_table and table.exists():  # the tuner's table for the benchmark shapes, measured on a B200
             self.tune_cache_load(str(table))
@@ -330,6 +357,7 @@ class Handle:
         if self._h:
             lib().fact_destroy(self._h)
             self._h = c_void_p()
+            self._hp = 0
 
     def __del__(self):
         try:
@@ -443,6 +471,11 @@ class Handle:
     # -- compute ------------------------------------------------------------------------------
     def gemm(self, A, B, layout="KN", out=None, out_dtype=torch.bfloat16, cfg=None, stream=None):
         """C = A @ B  (fact_gemm).  layout "KN": B is [K, N]; "NK": B is [N, K]."""
+        if cfg is None and stream is None:
+            r = self._bind.matmul(self._hp, self.device, self._ws, self._ws_streams, 0, A, B, LAYOUTS.get(layout, -1), out,
+                                  _OUT_CODES.get(out_dtype, -1))
+            if r is not None:
+                return r
         _, M, N, K = _validate_matmul(A, B, out, layout)
         if out is None:
             out = torch.empty((M, N), dtype=out_dtype, device=A.device)
@@ -494,6 +527,11 @@ class Handle:
 
     def gemm_batched(self, A, B, layout="KN", out=None, out_dtype=torch.bfloat16, cfg=None, stream=None):
         """C[b] = A[b] @ B[b]  (fact_gemm_batched)."""
+        if cfg is None and stream is None:
+            r = self._bind.matmul(self._hp, self.device, self._ws, self._ws_streams, 1, A, B, LAYOUTS.get(layout, -1), out,
+                                  _OUT_CODES.get(out_dtype, -1))
+            if r is not None:
+                return r
         batch, M, N, K = _validate_matmul(A, B, out, layout, batched=True)
         if out is None:
             out = torch.empty((batch, M, N), dtype=out_dtype, device=A.device)
@@ -507,6 +545,11 @@ class Handle:
 
     def gemm_splitk(self, A, B, layout="KN", out=None, out_dtype=torch.float32, splits=0, cfg=None, stream=None):
         """C = A @ B with K cut into slices and a fixed-order reduction  (fact_gemm_splitk)."""
+        if cfg is None and stream is None and splits == 0:
+            r = self._bind.matmul(self._hp, self.device, self._ws, self._ws_streams, 2, A, B, LAYOUTS.get(layout, -1), out,
+                                  _OUT_CODES.get(out_dtype, -1))
+            if r is not None:
+                return r
         _, M, N, K = _validate_matmul(A, B, out, layout)
         if out is None:
             out = torch.empty((M, N), dtype=out_dtype, device=A.device)
@@ -524,6 +567,11 @@ class Handle:
         For SILU_GATE W carries 2*N_out columns (gate first, then up).
         stats_out (FP32 [ceil(N_out/64), M, 2]) receives partial row sums of Y; x_norm "layer" / "rms" with x_stats
         (and w_colsum for "layer") folds a normalisation of X's rows into the product (fact_linear_ex)."""
+        if cfg is None and stream is None and stats_out is None and x_norm is None and x_stats is None and w_colsum is None:
+            r = self._bind.linear(self._hp, self.device, self._ws, self._ws_streams, X, W, None, bias, residual,
+                                  EPILOGUES.get(epilogue, -1), LAYOUTS.get(layout, -1), out, _OUT_CODES.get(out_dtype, -1), None)
+            if r is not None:
+                return r
         _need(X, "X", torch.bfloat16, 2)
         _need(W, "W", torch.bfloat16, 2)
         M, K = X.shape
@@ -610,6 +658,11 @@ class Handle:
                        out_dtype=torch.bfloat16, cfg=None, stream=None):
         """Y[rows of group g] = epilogue(X[rows of group g] @ W[g])  (fact_linear_grouped).  X [M, K]; W [G, Nw, K]
         (layout "NK") or [G, K, Nw] ("KN"); group_rows: G row counts summing to M (host integers)."""
+        if cfg is None and stream is None:
+            r = self._bind.linear(self._hp, self.device, None, None, X, W, None, bias, residual, EPILOGUES.get(epilogue, -1),
+                                  LAYOUTS.get(layout, -1), out, _OUT_CODES.get(out_dtype, -1), group_rows)
+            if r is not None:
+                return r
         _need(X, "X", torch.bfloat16, 2)
         _need(W, "W", torch.bfloat16, 3)
         rows = [int(r) for r in group_rows]
@@ -639,6 +692,11 @@ class Handle:
     def linear_grouped_fp8(self, X, W, group_rows, scale=1.0, bias=None, epilogue="NONE", out=None,
                            out_dtype=torch.bfloat16, cfg=None, stream=None):
         """fact_linear_grouped_fp8: X [M, K] and W [G, Nw, K] are FP8 E4M3 (torch.float8_e4m3fn or uint8 codes)."""
+        if cfg is None and stream is None:
+            r = self._bind.linear(self._hp, self.device, None, None, X, W, scale, bias, None, EPILOGUES.get(epilogue, -1), 1,
+                                  out, _OUT_CODES.get(out_dtype, -1), group_rows)
+            if r is not None:
+                return r
         def codes(t, name, nd):
             if isinstance(t, torch.Tensor) and t.dtype == torch.float8_e4m3fn:
                 t = t.view(torch.uint8)
@@ -669,6 +727,11 @@ class Handle:
                    out_dtype=torch.bfloat16, cfg=None, stream=None):
         """Y = epilogue(scale * X @ W^T)  (fact_linear_fp8).  X [M, K] and W [Nw, K] are FP8 E4M3: torch.float8_e4m3fn
         tensors, or torch.uint8 tensors holding the codes."""
+        if cfg is None and stream is None:
+            r = self._bind.linear(self._hp, self.device, self._ws, self._ws_streams, X, W, scale, bias, residual,
+                                  EPILOGUES.get(epilogue, -1), 1, out, _OUT_CODES.get(out_dtype, -1), None)
+            if r is not None:
+                return r
         def codes(t, name):
             if isinstance(t, torch.Tensor) and t.dtype == torch.float8_e4m3fn:
                 t = t.view(torch.uint8)
@@ -708,6 +771,10 @@ class Handle:
         """O = softmax(scale * Q K^T + causal mask) V  (fact_attention).
         q: [B, Tq, Hq, D], k / v: [B, Tk, Hkv, D] BF16 CUDA tensors (any strides with contiguous head_dim, e.g.
         slices of a fused QKV projection); returns [B, Tq, Hq, D]."""
+        if stream is None:
+            r = self._bind.attention(self._hp, self.device, q, k, v, causal, scale, out)
+            if r is not None:
+                return r
         for name, t in (("q", q), ("k", k), ("v", v)):
             _need(t, name, torch.bfloat16, 4)
         B, Tq, Hq, D = q.shape
@@ -724,6 +791,10 @@ class Handle:
     def norm(self, x, gamma, beta=None, kind="layer", eps=1e-5, out=None, stream=None):
         """Row normalisation (fact_norm): LayerNorm (kind="layer", gamma and beta) or RMSNorm (kind="rms", gamma).
         x: [M, C] BF16 (rows may be strided); returns [M, C]."""
+        if stream is None:
+            r = self._bind.norm(self._hp, self.device, x, gamma, beta, NORMS.get(kind, -1), eps, out)
+            if r is not None:
+                return r
         _need(x, "x", torch.bfloat16, 2)
         M, C = x.shape
         if out is None:
@@ -750,6 +821,10 @@ class Handle:
 
     def block_forward(self, desc, x, out=None, workspace=None, stream=None):
         """One transformer block forward (fact_block_forward).  x: [batch * seq, hidden] BF16, contiguous."""
+        if stream is None and workspace is None:
+            r = self._bind.block_forward(self._hp, self.device, self._ws, self._ws_streams, ctypes.addressof(desc), x, out)
+            if r is not None:
+                return r
         _need(x, "x", torch.bfloat16, 2)
         if not x.is_contiguous():
             raise ValueError("x must be contiguous")

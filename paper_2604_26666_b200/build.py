@@ -1,4 +1,4 @@
-"""Build libfact.so in-tree with nvcc for sm_100a (no JIT cache, no pip install).
+"""Build libfact.so in-tree with nvcc for sm_100a, and the Python extension beside it (no JIT cache, no pip install).
 
     python -m paper_2604_26666_b200.build [--force] [--verbose]
 
@@ -12,6 +12,7 @@ import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
@@ -19,6 +20,9 @@ ROOT = PKG.parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libfact.so"
 STAMP = PKG / "libfact.so.srchash"
+BIND_SOURCE = CSRC / "bind.cpp"
+BIND_LIB = PKG / "_fact_bind.so"  # the ordinary call's marshalling (CPython extension, linked to libfact.so beside it)
+BIND_STAMP = PKG / "_fact_bind.so.srchash"
 
 SOURCES = ["fact_api.cu"]
 HEADERS = ["gemm_kernel.cuh", "kcluster_kernel.cuh", "attention_kernel.cuh", "attention_decode_kernel.cuh",
@@ -72,5 +76,38 @@ def build(force: bool = False, verbose: bool = False) -> Path:
     return LIB
 
 
+def bind_hash() -> str:
+    import torch
+
+    h = hashlib.sha1()
+    for f in (BIND_SOURCE, ROOT / "include" / "fact.h"):
+        h.update(f.read_bytes())
+    h.update(f"{torch.__version__} {sys.version}".encode())
+    return h.hexdigest()
+
+
+def build_bind(force: bool = False) -> Path:
+    """The extension that binding.py calls; needs libfact.so (which it links to) and torch's headers."""
+    if not force and BIND_LIB.exists() and BIND_STAMP.exists() and BIND_STAMP.read_text().strip() == bind_hash():
+        return BIND_LIB
+    import torch
+
+    t = Path(torch.__file__).resolve().parent
+    tmp = BIND_LIB.with_suffix(f".tmp{os.getpid()}.so")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-isystem", str(t / "include"), "-isystem", str(t / "include" / "torch" / "csrc" / "api" / "include"),
+           "-isystem", str(Path(_nvcc()).resolve().parent.parent / "include"), "-I", sysconfig.get_paths()["include"],
+           "-I", str(ROOT / "include"), str(BIND_SOURCE), "-o", str(tmp), f"-L{PKG}", "-l:libfact.so", f"-L{t / 'lib'}",
+           "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("the binding extension failed to build:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
+    os.replace(tmp, BIND_LIB)
+    BIND_STAMP.write_text(bind_hash() + "\n")
+    return BIND_LIB
+
+
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="--verbose" in sys.argv))
+    print(build_bind(force="--force" in sys.argv))

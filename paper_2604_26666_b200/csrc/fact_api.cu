@@ -17,6 +17,7 @@
 #include <queue>
 #include <string>
 #include <tuple>
+#include <unordered_map>
 #include <utility>
 #include <vector>
 
@@ -86,6 +87,30 @@ struct Problem {
   int op_align() const { return fp8 ? 16 : 8; }              // elements in 16 bytes of an operand
 };
 
+// What the library's own choice of configuration depends on besides the tuner's table: kept choices are looked up by it.
+struct ChoiceKey {
+  long long batch, M, N_out, K;
+  int kind;  // op, epilogue, layout, output type, row sums out, normalisation in
+  int splits;
+  bool operator==(const ChoiceKey& o) const {
+    return batch == o.batch && M == o.M && N_out == o.N_out && K == o.K && kind == o.kind && splits == o.splits;
+  }
+};
+struct ChoiceHash {
+  size_t operator()(const ChoiceKey& k) const {
+    uint64_t h = 0x9E3779B97F4A7C15ull;
+    for (uint64_t v : {(uint64_t)k.batch, (uint64_t)k.M, (uint64_t)k.N_out, (uint64_t)k.K, (uint64_t)k.kind, (uint64_t)k.splits})
+      h = (h ^ v ^ (h >> 29)) * 0xBF58476D1CE4E5B9ull;
+    return (size_t)(h ^ (h >> 32));
+  }
+};
+struct Choice {
+  fact_status_t status;
+  fact_config_t cfg;
+  bool from_table;
+};
+constexpr size_t kMaxChoices = 4096;  // (a program with more shapes than that starts over)
+
 struct Plan {
   fact_config_t cfg;
   bool from_table = false;  // cfg came from the tuner's table: its store mode and K slices are hints, not demands
@@ -108,6 +133,7 @@ struct fact_handle_s {
   EncodeTiledFn encode = nullptr;
   long long launches = 0;
   std::map<TuneKey, fact_config_t> table;
+  std::unordered_map<ChoiceKey, Choice, ChoiceHash> choices;  // cleared with every change of the table
   std::bitset<192> configured_mask;  // kernels whose dynamic shared-memory limit was raised
   std::unique_ptr<AttnDeal> attn_deal;         // the host's deal of the last causal attention shape (see fact_attention)
   std::array<long long, 6> attn_deal_key{};
@@ -313,7 +339,7 @@ int raster_model(fact_handle_t h, const Problem& q, const fact_config_t& c) {
 }
 
 // Fill every zero field of `cfg`.  Returns FACT_ERR_UNSUPPORTED for a combination the kernels cannot run.
-fact_status_t resolve_config(fact_handle_t h, const Problem& q, const fact_config_t* user, int splits_override,
+fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const fact_config_t* user, int splits_override,
                              fact_config_t* out, bool* from_table_out = nullptr) {
   fact_config_t c;
   memset(&c, 0, sizeof c);
@@ -491,6 +517,29 @@ fact_status_t resolve_config(fact_handle_t h, const Problem& q, const fact_confi
   *out = c;
   if (from_table_out) *from_table_out = from_table;
   return FACT_OK;
+}
+
+// The same, with the library's own choices kept: the cost and raster models take longer than the rest of a call.
+// (A grouped problem's choice depends on its row counts, which are new with every call.)
+fact_status_t resolve_config(fact_handle_t h, const Problem& q, const fact_config_t* user, int splits_override,
+                             fact_config_t* out, bool* from_table_out = nullptr) {
+  if (user != nullptr || q.groups > 0) return resolve_config_uncached(h, q, user, splits_override, out, from_table_out);
+  const ChoiceKey key = {q.batch, q.M, q.N_out, q.K,
+                         (int)q.op | (int)q.epi << 4 | (int)q.layout << 8 | (int)q.out << 9 | (q.stats_out ? 1 << 10 : 0) | q.norm << 11,
+                         splits_override};
+  auto it = h->choices.find(key);
+  if (it == h->choices.end()) {
+    Choice c;
+    memset(&c, 0, sizeof c);
+    c.status = resolve_config_uncached(h, q, nullptr, splits_override, &c.cfg, &c.from_table);
+    if (h->choices.size() >= kMaxChoices) h->choices.clear();
+    it = h->choices.emplace(key, c).first;
+  }
+  if (it->second.status == FACT_OK) {
+    *out = it->second.cfg;
+    if (from_table_out) *from_table_out = it->second.from_table;
+  }
+  return it->second.status;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -1837,7 +1886,7 @@ fact_status_t fact_tune_ex(fact_handle_t h, fact_op_t op, int64_t batch, int64_t
   {
     auto saved = h->table;
     h->table.erase(make_key(q));
-    const fact_status_t rs = resolve_config(h, q, nullptr, 0, &ref_c);
+    const fact_status_t rs = resolve_config_uncached(h, q, nullptr, 0, &ref_c);
     h->table = saved;
     if (rs != FACT_OK || workspace_for(h, q, ref_c) > ws_bytes) {
       cleanup();
@@ -1981,6 +2030,7 @@ fact_status_t fact_tune_ex(fact_handle_t h, fact_op_t op, int64_t batch, int64_t
   if (n_tried) *n_tried = tried;
   if (tried == 0) return FACT_ERR_UNSUPPORTED;
   h->table[make_key(q)] = best_c;
+  h->choices.clear();
   *best = best_c;
   if (best_ms) *best_ms = best_t;
   return FACT_OK;
@@ -2030,6 +2080,7 @@ fact_status_t fact_tune_cache_load(fact_handle_t h, const char* path) {
       continue;
     h->table[TuneKey(op, epi, lay, out, b, M, N, K)] = c;
   }
+  h->choices.clear();
   fclose(f);
   return FACT_OK;
 }
