@@ -160,7 +160,12 @@ typedef enum {
  *                workspace, no partial planes in global memory, no grid-wide barrier.  Column-wise epilogues on
  *                BF16 operands (not SILU_GATE, row softmax, 8-bit operands, groups, row sums or a folded
  *                normalisation: FACT_ERR_UNSUPPORTED).  An untuned fact_gemm / fact_linear may take this schedule
- *                on its own (see split_k). */
+ *                on its own (see split_k).
+ *                4 = few rows: at most 64 rows of A / X against a weight matrix (decode), which is streamed once --
+ *                tile_n (16, 32 or 64; 32 or 64 for FACT_B_KN) weight rows and all of K per CTA, tile_m the rows rounded
+ *                up to 8, 16, 32 or 64; no workspace.  BF16 operands of fact_gemm / fact_linear (not the row softmax,
+ *                row sums, a folded normalisation or SILU_GATE with FACT_B_KN: FACT_ERR_UNSUPPORTED).  An untuned call
+ *                of at most 64 rows takes it on its own. */
 typedef struct {
   int tile_m, tile_n, tile_k, stages, cta_group, raster_group, split_k, store_mode, schedule;
 } fact_config_t;

@@ -24,6 +24,7 @@
 #include "fact.h"
 #include "gemm_kernel.cuh"
 #include "kcluster_kernel.cuh"
+#include "skinny_kernel.cuh"
 #include "attention_kernel.cuh"
 #include "attention_decode_kernel.cuh"
 #include "norm_kernel.cuh"
@@ -115,6 +116,7 @@ struct Plan {
   fact_config_t cfg;
   bool from_table = false;  // cfg came from the tuner's table: its store mode and K slices are hints, not demands
   bool dynamic = false;     // tiles are handed out through cluster launch control (one cluster of the grid per tile)
+  bool skinny = false;      // few rows: the kernel that streams the weights (schedule 4)
   bool kcluster = false;    // the K slices of a tile run as one cluster and are added up through shared memory
   int smem_bytes;
   int grid;
@@ -338,6 +340,28 @@ int raster_model(fact_handle_t h, const Problem& q, const fact_config_t& c) {
   return best_g;
 }
 
+// Few rows against a weight matrix (skinny_kernel.cuh): whether the kernel can run the problem, and how many weight rows
+// a CTA takes.
+bool skinny_ok(const Problem& q) {
+  return (q.op == FACT_OP_GEMM || q.op == FACT_OP_LINEAR) && q.batch == 1 && q.M >= 1 && q.M <= kSkinnyMaxRows && q.K > 0 &&
+         q.groups == 0 && !q.fp8 && !q.stats_out && !q.norm && q.epi != FACT_EPI_BIAS_SOFTMAX &&
+         !(q.layout == FACT_B_KN && q.epi == FACT_EPI_SILU_GATE);
+}
+int skinny_rows(fact_handle_t h, const Problem& q) {
+  // 16 where that makes no more CTAs than SMs (64 x 768 -> 2304: 3.7 us, 4.4 with 32), 64 where 32 would mean several
+  // waves (one row, 4096 -> 2 x 14336: 42.3 us with 32, 37.2 with 64), 32 between (4096 -> 6144: 14.2 / 10.2 / 10.7)
+  const long long nw = q.Nw();
+  if (q.layout == FACT_B_NK && nw <= 16LL * h->sm_count) return 16;
+  return nw <= 64LL * h->sm_count ? 32 : 64;
+}
+int skinny_groups(const Problem& q) { return q.M <= 8 ? 1 : (q.M <= 16 ? 2 : (q.M <= 32 ? 4 : 8)); }
+uint32_t skinny_stage_bytes(int rows, int groups) {
+  return (uint32_t)(rows + 8 * groups <= 64 ? 4 : 2) * 128u * (uint32_t)(rows + 8 * groups);
+}
+uint32_t skinny_part_bytes(int rows, int groups) {
+  return (uint32_t)(kSkinnyWarps / (rows == 64 ? 2 : 1)) * 8u * (uint32_t)groups * (uint32_t)(rows + 4) * 4u;
+}
+
 // Fill every zero field of `cfg`.  Returns FACT_ERR_UNSUPPORTED for a combination the kernels cannot run.
 fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const fact_config_t* user, int splits_override,
                              fact_config_t* out, bool* from_table_out = nullptr) {
@@ -353,6 +377,24 @@ fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const f
     }
   }
   if (splits_override > 0) c.split_k = splits_override;
+  // At most 64 rows: the kernel that streams the weights.  Above 32 rows and several waves of CTAs the rows' own traffic
+  // from L2 costs more than the tile kernels' padding (64 rows, 4096 -> 2 x 14336: 55.0 us against 43.5).
+  if (c.schedule == 4 || (user == nullptr && !from_table && splits_override == 0 && skinny_ok(q) &&
+                          !(q.M > 32 && q.Nw() > 64LL * h->sm_count))) {
+    if (!skinny_ok(q) || c.split_k > 1 || c.split_k < 0 || (c.store_mode != 0 && c.store_mode != 1)) return FACT_ERR_UNSUPPORTED;
+    const int rows = c.tile_n ? c.tile_n : skinny_rows(h, q), groups = skinny_groups(q);
+    if ((rows != 16 && rows != 32 && rows != 64) || (rows == 16 && q.layout == FACT_B_KN)) return FACT_ERR_UNSUPPORTED;
+    const long long ctas = (q.Nw() + rows - 1) / rows;
+    // one CTA per SM has the ring to itself; where there are more CTAs two share an SM
+    const uint32_t ring = ctas <= h->sm_count ? 192 * 1024 : 96 * 1024;
+    const int smax = (int)std::min<uint32_t>(kSkinnyMaxStages, ring / skinny_stage_bytes(rows, groups));
+    const int stages = c.stages ? c.stages : smax;
+    if (stages < 2 || stages > smax) return FACT_ERR_UNSUPPORTED;
+    const fact_config_t sk = {8 * groups, rows, kTileK, stages, 1, 1, 1, 1, 4};
+    *out = sk;
+    if (from_table_out) *from_table_out = from_table;
+    return FACT_OK;
+  }
   if (c.tile_k != 0 && c.tile_k != q.k_elems()) return FACT_ERR_UNSUPPORTED;
   c.tile_k = q.k_elems();
   const long long Nw = q.Nw();
@@ -512,7 +554,7 @@ fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const f
   if (c.split_k < -2) return FACT_ERR_INVALID_ARG;
   if (c.split_k > 0) c.split_k = std::max(1, std::min(c.split_k, std::max(1, k_blocks)));
   if (c.store_mode < 0 || c.store_mode > 3) return FACT_ERR_INVALID_ARG;
-  if (c.schedule < 0 || c.schedule > 3) return FACT_ERR_INVALID_ARG;
+  if (c.schedule < 0 || c.schedule > 4) return FACT_ERR_INVALID_ARG;
   if (c.schedule == 0) c.schedule = 1;
   *out = c;
   if (from_table_out) *from_table_out = from_table;
@@ -614,7 +656,7 @@ int sk_tiles_for(fact_handle_t h, const Problem& q, const fact_config_t& c) {
 }
 
 size_t workspace_for(fact_handle_t h, const Problem& q, const fact_config_t& c) {
-  if (c.schedule == 3) return 0;  // K slices as a cluster: the partial sums never leave the SMs
+  if (c.schedule >= 3) return 0;  // K slices as a cluster: the partial sums never leave the SMs
   if (c.split_k < 0) {  // stream-K: one FP32 accumulator tile per CTA
     if (sk_tiles_for(h, q, c) == 0) return 0;
     const size_t ctas = (size_t)std::max(1, h->sm_count / c.cta_group) * (size_t)c.cta_group;
@@ -642,6 +684,14 @@ fact_status_t make_plan(fact_handle_t h, const Problem& q, const fact_config_t* 
   memset(&p, 0, sizeof p);
   const int cg = c.cta_group;
   const bool gate = q.epi == FACT_EPI_SILU_GATE;
+  if (c.schedule == 4) {
+    plan->skinny = true;
+    plan->ws_bytes = 0;
+    plan->smem_bytes = (int)(std::max((uint32_t)c.stages * skinny_stage_bytes(c.tile_n, skinny_groups(q)),
+                                      skinny_part_bytes(c.tile_n, skinny_groups(q))) + kSkinnyCtrlBytes);
+    plan->grid = (int)((q.N_out + (gate ? c.tile_n / 2 : c.tile_n) - 1) / (gate ? c.tile_n / 2 : c.tile_n));
+    return plan->smem_bytes <= h->max_smem ? FACT_OK : FACT_ERR_UNSUPPORTED;
+  }
   p.M = (int)q.M;
   p.N_out = (int)q.N_out;
   p.Nw = (int)q.Nw();
@@ -811,12 +861,12 @@ fact_status_t make_plan(fact_handle_t h, const Problem& q, const fact_config_t* 
   return FACT_OK;
 }
 
-// A rank-3 tensor map (inner, rows, batch) with a (box0 x box1 x 1) box and 128-byte swizzle.
+// A rank-3 tensor map (inner, rows, batch) with a (box0 x box1 x 1) box and 128-byte (or 64-byte) swizzle.
 fact_status_t encode_map(fact_handle_t h, CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2,
                          uint64_t stride1_elems, uint64_t stride2_elems, uint32_t box0, uint32_t box1,
-                         bool f32 = false, bool u8 = false) {
+                         bool f32 = false, bool u8 = false, bool swizzle64 = false) {
   const uint64_t esz = f32 ? 4 : (u8 ? 1 : 2);
-  fact_handle_s::MapKey key = {base, d0, d1, d2, stride1_elems, stride2_elems, box0, box1, (uint32_t)(f32 ? 1 : (u8 ? 2 : 0))};
+  fact_handle_s::MapKey key = {base, d0, d1, d2, stride1_elems, stride2_elems, box0, box1, (uint32_t)(f32 ? 1 : (u8 ? 2 : 0)) + (swizzle64 ? 4u : 0u)};
   uint64_t hsh = reinterpret_cast<uintptr_t>(base) * 0x9E3779B97F4A7C15ull;
   for (uint64_t v : {d0, d1, d2, stride1_elems, stride2_elems, (uint64_t)box0 << 32 | box1, (uint64_t)key.kind})
     hsh = (hsh ^ v) * 0x9E3779B97F4A7C15ull;
@@ -831,7 +881,7 @@ fact_status_t encode_map(fact_handle_t h, CUtensorMap* map, const void* base, ui
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = h->encode(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : (u8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16), 3,
                          const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r == CUDA_SUCCESS) {
     slot.used = true;
@@ -993,6 +1043,60 @@ fact_status_t launch_reduce(fact_handle_t h, const Problem& q, const Plan& plan,
   return FACT_OK;
 }
 
+fact_status_t launch_skinny(fact_handle_t h, const Problem& q, const Plan& plan, cudaStream_t stream) {
+  const int rows = plan.cfg.tile_n, groups = skinny_groups(q);
+  const bool kn = q.layout == FACT_B_KN, gate = q.epi == FACT_EPI_SILU_GATE;
+  CUtensorMap tx, tw;
+  fact_status_t st = encode_map(h, &tx, q.A, (uint64_t)q.K, (uint64_t)q.M, 1, (uint64_t)q.lda,
+                                std::max<uint64_t>((uint64_t)q.lda * (uint64_t)q.M, 8), 64, (uint32_t)(8 * groups));
+  if (st != FACT_OK) return st;
+  if (kn)
+    st = encode_map(h, &tw, q.B, (uint64_t)q.Nw(), (uint64_t)q.K, 1, (uint64_t)q.ldb,
+                    std::max<uint64_t>((uint64_t)q.ldb * (uint64_t)q.K, 8), (uint32_t)rows, 64, false, false, rows == 32);
+  else
+    st = encode_map(h, &tw, q.B, (uint64_t)q.K, (uint64_t)q.Nw(), 1, (uint64_t)q.ldb,
+                    std::max<uint64_t>((uint64_t)q.ldb * (uint64_t)q.Nw(), 8), 64, (uint32_t)(gate ? rows / 2 : rows));
+  if (st != FACT_OK) return st;
+  SkinnyParams p;
+  memset(&p, 0, sizeof p);
+  p.M = (int)q.M;
+  p.N = (int)q.N_out;
+  p.K = (int)q.K;
+  p.gate = gate;
+  p.b_kn = kn;
+  p.stages = plan.cfg.stages;
+  p.epi = (int)q.epi;
+  p.out_f32 = q.out == FACT_OUT_F32;
+  p.C = q.C;
+  p.ldc = q.ldc;
+  p.c_vec = (reinterpret_cast<uintptr_t>(q.C) & (p.out_f32 ? 15u : 7u)) == 0 && q.ldc % 4 == 0;
+  p.bias = reinterpret_cast<const __nv_bfloat16*>(q.bias);
+  p.R = reinterpret_cast<const __nv_bfloat16*>(q.R);
+  p.ldr = q.ldr;
+  p.status = h->d_status;
+  typedef void (*Kern)(CUtensorMap, CUtensorMap, SkinnyParams);
+  static const Kern kerns[5][4] = {
+#define FACT_SKINNY_ROW(R, KN) \
+  {fact_linear_skinny_kernel<R, 1, KN>, fact_linear_skinny_kernel<R, 2, KN>, fact_linear_skinny_kernel<R, 4, KN>, \
+   fact_linear_skinny_kernel<R, 8, KN>}
+      FACT_SKINNY_ROW(16, false), FACT_SKINNY_ROW(32, false), FACT_SKINNY_ROW(64, false), FACT_SKINNY_ROW(32, true),
+      FACT_SKINNY_ROW(64, true)};
+#undef FACT_SKINNY_ROW
+  if (!h->configured_mask.test(165)) {
+    for (const auto& row : kerns)
+      for (Kern k : row) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        if (e != cudaSuccess) return cuda_fail(h, "cudaFuncSetAttribute(few rows)", e);
+      }
+    h->configured_mask.set(165);
+  }
+  const Kern kern = kerns[(rows == 16 ? 0 : (rows == 32 ? 1 : 2)) + (kn ? 2 : 0)][groups == 8 ? 3 : groups / 2];
+  cudaError_t e = launch_pdl(h, kern, (unsigned)plan.grid, (unsigned)kSkinnyThreads, (size_t)plan.smem_bytes, stream, 1, tx, tw, p);
+  if (e != cudaSuccess) return cuda_fail(h, "cudaLaunchKernelEx (few rows)", e);
+  h->launches++;
+  return FACT_OK;
+}
+
 fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, int splits_override, void* ws,
                   size_t ws_bytes, void* stream_v) {
   if (!h) return FACT_ERR_INVALID_ARG;
@@ -1002,9 +1106,9 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_v);
   Plan plan;
   st = make_plan(h, q, user, splits_override, &plan);
-  if (st == FACT_ERR_UNSUPPORTED && plan.from_table && plan.cfg.schedule == 3) {
-    // a table entry with K slices as a cluster, tuned on a plain call of this shape: this call (row sums, a folded
-    // normalisation) takes the library's own choice instead
+  if (st == FACT_ERR_UNSUPPORTED && plan.from_table) {
+    // a table entry with K slices as a cluster or the few-rows kernel, tuned on a plain call of this shape: this call
+    // (row sums, a folded normalisation) takes the library's own choice instead
     fact_config_t none;
     memset(&none, 0, sizeof none);
     none.split_k = 1;
@@ -1015,6 +1119,11 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
   if (cudaGetDevice(&dev) != cudaSuccess) return FACT_ERR_CUDA;
   if (dev != h->device && cudaSetDevice(h->device) != cudaSuccess) return FACT_ERR_CUDA;
 
+  if (plan.skinny) {
+    st = launch_skinny(h, q, plan, stream);
+    if (dev != h->device) cudaSetDevice(dev);
+    return st;
+  }
   std::vector<int> group_table;
   if (q.groups > 0) {
     // Grouped: tiles never cross a group boundary (a group's last m-tile is ragged), every tile is data-parallel and
@@ -1843,6 +1952,11 @@ fact_status_t fact_tune_ex(fact_handle_t h, fact_op_t op, int64_t batch, int64_t
         fact_config_t c = {128 * cg, tn, q.k_elems(), smax, cg, 0, sl, 0, 3};
         cands.push_back(c);
       }
+  // few rows: the kernel that streams the weights (refused for more rows, or where it cannot run)
+  for (int rows = 16; rows <= 64; rows *= 2) {
+    fact_config_t c = {0, rows, 0, 0, 0, 0, 0, 0, 4};
+    if (M <= kSkinnyMaxRows) cands.push_back(c);
+  }
   // Time `c` over `n` launches (per launch, ms); a negative result means the candidate failed.  Warm L2: the launches
   // run back to back between one event pair.  Cold L2: a buffer twice the size of L2 is overwritten before each
   // launch and every launch has an event pair of its own (what a benchmark that flushes L2 between launches sees).

@@ -1,0 +1,271 @@
+// Linear layers of a few rows (decode: at most 64 tokens against a weight matrix): Y = epilogue(X W).
+//
+// Bound: HBM.  The weights are read once and meet a few rows, so the kernel is a stream of the weights with a small
+// product attached.  (The tile kernels multiply 128-row tiles of which 112 rows are padding here; with so few tiles
+// they have to cut K over CTAs to fill the SMs, and adding the slices up -- through the workspace or a cluster's shared
+// memory -- costs about 5 us, as long as the whole stream of a 4096 x 4096 layer.)  Here
+//   - a CTA owns R = 16, 32 or 64 weight rows (output columns; half gate, half up rows for a gated layer) and ALL of K,
+//     so nothing is exchanged between CTAs; R is chosen so that the CTAs cover the SMs (see skinny_rows in the host
+//     code), and X, which every CTA reads, costs no more of an SM's 70-80 bytes a clock from L2 than the weights do;
+//   - one warp streams W and X through a TMA ring (128-byte swizzled boxes of 64 k);
+//   - eight warps take 16 k of a stage at a time with mma.sync.m16n8k16, the weights as the 16-row operand and the
+//     tokens, in groups of 8, as the other: 64 tokens are 4 % of the tensor rate a tile kernel needs, and no
+//     accumulator has to travel through tensor memory;
+//   - the warps' sums are added up in a fixed order through shared memory, then the epilogue and the store.
+// Measured, weights rotating through HBM, the tile kernels' choice -> this: 16 x 4096 -> 4096 14.1 -> 7.8 us (HBM alone
+// 5.1), 1 x 4096 -> 6144 23.3 -> 10.1, 1 x 4096 -> 2 x 14336 gated 54.9 -> 37.2 (6.3 TB/s), 16 x 14336 -> 4096 28.7 ->
+// 20.3, 16 x 768 -> 2304 6.9 -> 3.1.  (Sets of warps that take stages in turn, four steps each, were no faster.)
+#pragma once
+#include "gemm_kernel.cuh"
+
+namespace fact {
+
+constexpr int kSkinnyWarps = 8;
+constexpr int kSkinnyThreads = 32 * (kSkinnyWarps + 1);  // the last warp loads
+constexpr int kSkinnyMaxRows = 64;
+constexpr int kSkinnyMaxStages = 16;
+constexpr uint32_t kSkinnyCtrlBytes = 2 * kSkinnyMaxStages * 8 + 16;
+
+// Geometry of one (R weight rows, NT groups of 8 tokens) variant.
+template <int R, int NT>
+struct SkinnyShape {
+  static constexpr int kRowGroups = R == 64 ? 2 : 1;               // warps side by side along the weight rows
+  static constexpr int kKWarps = kSkinnyWarps / kRowGroups;         // ... and along k
+  static constexpr int kFrags = R / kRowGroups / 16;                // 16-row fragments per warp
+  static constexpr int kBoxes = R + 8 * NT <= 64 ? 4 : 2;           // 64-wide boxes of k per stage
+  static constexpr int kSteps = kBoxes * 4 / kKWarps;               // 16-wide steps of k per warp and stage: 1 or 2
+  static constexpr uint32_t kBoxW = R * 128u, kBoxX = 8u * NT * 128u;
+  static constexpr uint32_t kStage = kBoxes * (kBoxW + kBoxX);
+  static constexpr int kPartLd = R + 4;                             // floats per token of a warp's partial sums
+  static constexpr uint32_t kPartBytes = (uint32_t)kKWarps * 8u * NT * kPartLd * 4u;
+};
+
+struct SkinnyParams {
+  int M, N, K;        // N output columns
+  int gate, b_kn;
+  int stages;
+  int epi, out_f32;
+  void* C;
+  long long ldc;
+  int c_vec;          // four output columns can be stored at once
+  const __nv_bfloat16* bias;
+  const __nv_bfloat16* R;
+  long long ldr;
+  int* status;
+};
+
+template <int R, int NT, bool KN>
+__global__ void __launch_bounds__(kSkinnyThreads, 2)
+    fact_linear_skinny_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
+                              const SkinnyParams p) {
+  using S = SkinnyShape<R, NT>;
+  static_assert((S::kSteps == 1 || S::kSteps == 2) && S::kFrags >= 1, "every warp has work in every stage");
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31;
+  const uint32_t smem_base = ptx::smem_u32(smem_raw);
+  const int NS = p.stages;
+  const uint32_t ring_bytes = max((uint32_t)NS * S::kStage, S::kPartBytes);
+  if ((smem_base & 1023u) || NS < 2 || NS > kSkinnyMaxStages) {
+    if (threadIdx.x == 0) atomicExch(p.status, kDeviceTimeoutCode);
+    return;
+  }
+  const uint32_t bar_base = smem_base + ring_bytes;
+  auto full_bar = [&](int s) { return bar_base + 8u * (uint32_t)s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (uint32_t)(kSkinnyMaxStages + s); };
+  volatile int* abort_p = reinterpret_cast<volatile int*>(smem_raw + ring_bytes + 2 * kSkinnyMaxStages * 8);
+  if (threadIdx.x < 2 * kSkinnyMaxStages) {
+    ptx::mbar_init(bar_base + 8u * threadIdx.x, (int)threadIdx.x < kSkinnyMaxStages ? 1 : kSkinnyWarps);
+    if (threadIdx.x == 0) *abort_p = 0;
+    ptx::fence_mbar_init();
+  }
+  if (warp == kSkinnyWarps && lane == 0) {
+    ptx::prefetch_tensormap(&tmX);
+    ptx::prefetch_tensormap(&tmW);
+  }
+  __syncthreads();
+  ptx::grid_dependency_wait();
+
+  constexpr int kStageK = S::kBoxes * 64;
+  const int n_stages = (p.K + kStageK - 1) / kStageK;
+  const int cols = p.gate ? R / 2 : R;          // output columns of this CTA
+  const int n0 = (int)blockIdx.x * cols;
+  auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
+    return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_p, p.status)) != 0;
+  };
+  const int rg = warp % S::kRowGroups, kw = warp / S::kRowGroups;  // this warp's rows and its turn along k
+  float acc[S::kFrags][NT][4];
+#pragma unroll
+  for (int f = 0; f < S::kFrags; ++f)
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[f][t][i] = 0.f;
+
+  if (warp == kSkinnyWarps) {
+    // ------------------------------------------------------------ TMA producer
+    const uint64_t keep = ptx::l2_policy(2), normal = ptx::l2_policy(0);  // X is read by every CTA, W once
+    // Each CTA starts at a k of its own and wraps around: CTAs in step ask L2 for the same lines of X at the same time
+    // (4096 -> 2 x 14336 for one row 39.2 us in step, 37.1 apart; 4096 -> 6144 10.7 and 10.1).  Not for [K, N] weights,
+    // whose neighbouring CTAs share DRAM pages while in step (14336 -> 4096 20.6 and 22.4 us), nor for more than 32 rows.
+    int s = 0, jk = (!KN && NT <= 4) ? (int)(blockIdx.x % (unsigned)n_stages) : 0;
+    uint32_t phase = 0;
+    for (int j = 0; j < n_stages; ++j) {
+      if (!wait_all(empty_bar(s), phase ^ 1u)) break;
+      if (ptx::elect_one()) {
+        const uint32_t dst = smem_base + (uint32_t)s * S::kStage;
+        ptx::mbar_arrive_expect_tx(full_bar(s), S::kStage);
+#pragma unroll
+        for (int b = 0; b < S::kBoxes; ++b) {  // (boxes wholly past K arrive as zeros)
+          const int k = jk * kStageK + b * 64;
+          const uint32_t w = dst + (uint32_t)b * S::kBoxW;
+          if constexpr (KN) {
+            ptx::tma_load_3d_hint(w, &tmW, full_bar(s), n0, k, 0, normal);
+          } else if (p.gate) {
+            ptx::tma_load_3d_hint(w, &tmW, full_bar(s), k, n0, 0, normal);
+            ptx::tma_load_3d_hint(w + S::kBoxW / 2, &tmW, full_bar(s), k, p.N + n0, 0, normal);
+          } else {
+            ptx::tma_load_3d_hint(w, &tmW, full_bar(s), k, n0, 0, normal);
+          }
+          ptx::tma_load_3d_hint(dst + S::kBoxes * S::kBoxW + (uint32_t)b * S::kBoxX, &tmX, full_bar(s), k, 0, 0, keep);
+        }
+      }
+      __syncwarp();
+      if (++jk == n_stages) jk = 0;
+      if (++s == NS) {
+        s = 0;
+        phase ^= 1u;
+      }
+    }
+  } else {
+    // ------------------------------------------------------------ 16 k of a stage at a time per warp
+    // ldmatrix addresses of this lane.  W, [row][k] storage: row lane % 16, 16-byte piece lane / 16 of the step's two;
+    // [k][row] storage (read transposed): k row lane % 8 + 8 (lane / 16), piece (lane / 8) % 2 of 8 rows.
+    // X: token lane % 8 + 8 (lane / 16), piece (lane / 8) % 2.
+    const uint32_t w_row = (uint32_t)(rg * 16 * S::kFrags + (lane & 15)), w_piece = (uint32_t)(lane >> 4);
+    const uint32_t t_row = (uint32_t)((lane & 7) + ((lane >> 4) << 3)), t_piece = (uint32_t)((lane >> 3) & 1);
+    int s = 0;
+    uint32_t phase = 0;
+    for (int j = 0; j < n_stages; ++j) {
+      if (!wait_all(full_bar(s), phase)) break;
+      const uint32_t w0 = smem_base + (uint32_t)s * S::kStage;
+      const uint32_t x0 = w0 + S::kBoxes * S::kBoxW;
+      uint32_t xf[S::kSteps][NT][2], wf[S::kSteps][S::kFrags][4];
+#pragma unroll
+      for (int u = 0; u < S::kSteps; ++u) {
+        const uint32_t step = (uint32_t)(kw * S::kSteps + u);  // 16-wide step of the stage
+        const uint32_t box = step >> 2, in = step & 3u;
+#pragma unroll
+        for (int t = 0; t < NT; t += 2) {
+          const uint32_t base = x0 + box * S::kBoxX + (uint32_t)(8 * t) * 128u;
+          if (t + 1 < NT) {
+            uint32_t v[4];
+            ptx::ldmatrix_x4(base + t_row * 128u + (((2u * in + t_piece) ^ (t_row & 7u)) << 4), v);
+            xf[u][t][0] = v[0];
+            xf[u][t][1] = v[1];
+            xf[u][t + 1][0] = v[2];
+            xf[u][t + 1][1] = v[3];
+          } else {
+            const uint32_t r = (uint32_t)(lane & 7);
+            ptx::ldmatrix_x2(base + r * 128u + (((2u * in + t_piece) ^ r) << 4), xf[u][t]);
+          }
+        }
+#pragma unroll
+        for (int f = 0; f < S::kFrags; ++f) {
+          if constexpr (KN) {
+            // rows of 2 R bytes (64 or 128); the swizzle XORs address bits 4.. with bits 7.. (two bits, or three)
+            const uint32_t off = (16u * in + t_row) * (2u * R) + (((uint32_t)(rg * 2 * S::kFrags + 2 * f) + t_piece) << 4);
+            ptx::ldmatrix_x4_trans(w0 + box * S::kBoxW + (off ^ (((off >> 7) & (R / 8u - 1u)) << 4)), wf[u][f]);
+          } else {
+            const uint32_t row = w_row + 16u * (uint32_t)f;
+            ptx::ldmatrix_x4(w0 + box * S::kBoxW + row * 128u + (((2u * in + w_piece) ^ (row & 7u)) << 4), wf[u][f]);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < S::kSteps; ++u)
+#pragma unroll
+        for (int f = 0; f < S::kFrags; ++f)
+#pragma unroll
+          for (int t = 0; t < NT; ++t) ptx::mma_m16n8k16_bf16(acc[f][t], wf[u][f], xf[u][t]);
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(empty_bar(s));
+      if (++s == NS) {
+        s = 0;
+        phase ^= 1u;
+      }
+    }
+  }
+  __syncthreads();  // every load has landed and been read: the ring becomes the partial sums' place
+  ptx::grid_launch_dependents();
+  float* const part = reinterpret_cast<float*>(smem_raw);  // [warp along k][token][kPartLd]
+  if (warp < kSkinnyWarps) {
+#pragma unroll
+    for (int f = 0; f < S::kFrags; ++f)
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int token = 8 * t + 2 * (lane & 3) + (i & 1);
+          const int row = (rg * S::kFrags + f) * 16 + (lane >> 2) + (i >> 1) * 8;
+          part[(kw * 8 * NT + token) * S::kPartLd + row] = acc[f][t][i];
+        }
+  }
+  __syncthreads();
+  auto sum4 = [&](int token, int row) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < S::kKWarps; ++w) {
+      const float4 u = *reinterpret_cast<const float4*>(part + (w * 8 * NT + token) * S::kPartLd + row);
+      v.x += u.x;
+      v.y += u.y;
+      v.z += u.z;
+      v.w += u.w;
+    }
+    return v;
+  };
+  const int quads = cols / 4;
+  for (int i = (int)threadIdx.x; i < p.M * quads; i += kSkinnyThreads) {
+    const int token = i / quads, c = 4 * (i - token * quads), n = n0 + c;
+    const int nvalid = min(4, p.N - n);
+    if (nvalid <= 0) continue;
+    const float4 a = sum4(token, c);
+    const float av[4] = {a.x, a.y, a.z, a.w};
+    float uv[4] = {0.f, 0.f, 0.f, 0.f};
+    if (p.gate) {
+      const float4 u = sum4(token, R / 2 + c);
+      uv[0] = u.x; uv[1] = u.y; uv[2] = u.z; uv[3] = u.w;
+    }
+    float y[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool ok = j < nvalid;
+      const float bias = (ok && p.bias != nullptr) ? __bfloat162float(p.bias[n + j]) : 0.f;
+      const float res = (ok && p.epi == kEpiBiasResidual) ? __bfloat162float(p.R[(long long)token * p.ldr + n + j]) : 0.f;
+      y[j] = reduce_epilogue(p.epi, av[j], uv[j], bias, res);
+    }
+    const long long off = (long long)token * p.ldc + n;
+    if (p.out_f32) {
+      float* dst = reinterpret_cast<float*>(p.C) + off;
+      if (p.c_vec && nvalid == 4) {
+        *reinterpret_cast<float4*>(dst) = make_float4(y[0], y[1], y[2], y[3]);
+      } else {
+        for (int j = 0; j < nvalid; ++j) dst[j] = y[j];
+      }
+    } else {
+      __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.C) + off;
+      if (p.c_vec && nvalid == 4) {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]));
+      } else {
+        for (int j = 0; j < nvalid; ++j) dst[j] = __float2bfloat16_rn(y[j]);
+      }
+    }
+  }
+  if (*abort_p) {  // a wait expired: give copies that may still be in flight time to land
+    const unsigned long long t0 = ptx::globaltimer_ns();
+    while (ptx::globaltimer_ns() - t0 < 200000ull) {
+    }
+  }
+}
+
+}  // namespace fact
