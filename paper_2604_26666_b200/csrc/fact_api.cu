@@ -771,14 +771,20 @@ fact_status_t make_plan(fact_handle_t h, const Problem& q, const fact_config_t* 
   p.r_vec = q.R && aligned16(q.R) && (q.ldr % 8 == 0) && (q.batch <= 1 || q.strideR % 8 == 0);
   p.ws_ld = ws_ld_for(q);
   p.ws_planes = ws_planes_for(q);
-  // Staged TMA stores need a 16-byte aligned output whose rows are 16-byte multiples, whole 128-byte chunks per
-  // tile, and (for a residual) a BF16 output; anything else is stored directly from registers.
+  // The staged epilogue needs whole 128-byte chunks per tile and (for a residual) a BF16 output; its tensor stores also a
+  // 16-byte aligned output whose rows are 16-byte multiples apart AND hold whole 16-byte pieces (a tensor store writes the
+  // piece that the last column lies in as a whole, zeros into the columns behind it).
   const int chunk_cols = p.out_f32 ? 32 : 64;
-  const bool can_stage = p.c_vec && (p.out_cols % chunk_cols == 0) &&
-                         !(p.out_f32 && q.epi == FACT_EPI_BIAS_RESIDUAL);
+  const long long esz_c = p.out_f32 ? 4 : 2;
+  const bool chunks = (p.out_cols % chunk_cols == 0) && !(p.out_f32 && q.epi == FACT_EPI_BIAS_RESIDUAL);
+  const bool can_stage = p.c_vec && chunks;
+  const bool tensor_stores = can_stage && (q.N_out * esz_c) % 16 == 0;
+  // Rows of any alignment: staged all the same and written out by the warps, where the staged epilogue runs at all (whole,
+  // unsliced, ungrouped, statically dealt tiles); otherwise each thread stores its own row from registers.
+  const bool any_rows = chunks && !tensor_stores && c.store_mode != 1 && c.store_mode != 3 && c.split_k <= 1 && c.schedule == 1 &&
+                        q.groups == 0 && q.epi != FACT_EPI_BIAS_SOFTMAX && (can_stage || (!q.stats_out && !q.norm));
   // The table is keyed on the shape alone, so what it says about the store path is a hint: this call's output may
   // be less aligned than the one the entry was tuned on.  Only a caller's own configuration is refused.
-  const long long esz_c = p.out_f32 ? 4 : 2;
   const bool rows32 = (reinterpret_cast<uintptr_t>(q.C) & 31u) == 0 && (q.ldc * esz_c) % 32 == 0 &&
                       (q.N_out * esz_c) % 32 == 0 && (q.batch <= 1 || (q.strideC * esz_c) % 32 == 0);
   const bool can_rows32 = can_stage && rows32 && c.split_k == 1 && q.groups == 0 && !q.stats_out && !q.norm &&
@@ -787,9 +793,10 @@ fact_status_t make_plan(fact_handle_t h, const Problem& q, const fact_config_t* 
     plan->cfg.store_mode = 0;
   if (c.store_mode == 2 && !can_stage) return FACT_ERR_UNSUPPORTED;
   const int asked_store = c.store_mode;  // (c aliases plan->cfg, which is rewritten below)
-  p.store_tma = (c.store_mode == 1) ? 0 : (can_stage ? 1 : 0);
+  p.store_tma = (c.store_mode == 1) ? 0 : ((tensor_stores || any_rows) ? 1 : 0);
   p.r_tma = p.store_tma && q.epi == FACT_EPI_BIAS_RESIDUAL && p.r_vec;
-  plan->cfg.store_mode = p.store_tma ? 2 : 1;
+  plan->cfg.store_mode = p.store_tma ? (any_rows ? asked_store : 2) : 1;
+  if (any_rows && p.store_tma) p.row_stores = 2;
   if (asked_store == 3) {
     // the staged epilogue's arithmetic with each row stored from registers in 32-byte pieces: whole, unsliced,
     // ungrouped tiles whose output rows are 32-byte aligned multiples of 32 bytes
@@ -844,7 +851,7 @@ fact_status_t make_plan(fact_handle_t h, const Problem& q, const fact_config_t* 
   }
   if (c.split_k < 0) {
     // Stream-K: the staged epilogue parks and finishes the pieces, so an output it cannot store is data-parallel.
-    const int sk = p.store_tma ? sk_tiles_for(h, q, c) : 0;
+    const int sk = p.store_tma && !p.row_stores ? sk_tiles_for(h, q, c) : 0;
     if (sk == 0) {
       plan->cfg.split_k = 1;
       plan->ws_bytes = 0;
@@ -968,11 +975,11 @@ fact_status_t launch_epi(fact_handle_t h, int epi, const Plan& plan, const CUten
 }
 
 // The instantiations with row sums out (EXT 1), a folded row normalisation in, with or without row sums out
-// (EXT 2), or rows stored from registers in 32-byte pieces (EXT 3): staged epilogue, data-parallel tiles.  Two sets, because the consumer's code slows the producer's
+// (EXT 2), rows stored from registers in 32-byte pieces (EXT 3) or rows of any alignment (EXT 4): staged epilogue, data-parallel tiles.  Two sets, because the consumer's code slows the producer's
 // epilogue down even when it does not run.
 template <int CG, int EXT>
 fact_status_t launch_epi_ext(fact_handle_t h, int epi, const Plan& plan, const CUtensorMap* tm, cudaStream_t stream) {
-  const int base = 32 + (EXT - 1) * 16 + (CG - 1) * 8;
+  const int base = (EXT == 4 ? 166 : 32 + (EXT - 1) * 16) + (CG - 1) * 8;
   switch (epi) {
     case kEpiNone: return launch_instance<CG, kEpiNone, false, false, EXT>(h, base + 0, plan, tm, stream);
     case kEpiBias: return launch_instance<CG, kEpiBias, false, false, EXT>(h, base + 1, plan, tm, stream);
@@ -1259,7 +1266,8 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
     } else if (plan.p.store_tma && !plan.kcluster) {
       const bool f32 = q.out == FACT_OUT_F32;
       const uint64_t sC = q.batch > 1 ? (uint64_t)q.strideC : (uint64_t)q.ldc * (uint64_t)q.M;
-      st = encode_map(h, &tm[2], q.C, (uint64_t)q.N_out, (uint64_t)q.M, batch_dim, (uint64_t)q.ldc,
+      if (plan.p.row_stores != 2)
+        st = encode_map(h, &tm[2], q.C, (uint64_t)q.N_out, (uint64_t)q.M, batch_dim, (uint64_t)q.ldc,
                       std::max<uint64_t>(sC, 8), f32 ? 32 : 64, 32, f32);
       if (st != FACT_OK) return st;
       if (plan.p.r_tma) {
@@ -1278,7 +1286,9 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
                                     : launch_epi_dp<1, true, false>(h, epi, plan, tm, stream);
     else if (plan.dynamic) st = two ? launch_epi_dp<2, false, true>(h, epi, plan, tm, stream)
                                     : launch_epi_dp<1, false, true>(h, epi, plan, tm, stream);
-    else if (plan.p.row_stores && !split) st = plan.cfg.cta_group == 2 ? launch_epi_ext<2, 3>(h, epi, plan, tm, stream)
+    else if (plan.p.row_stores == 2 && !split && !q.norm && !q.stats_out) st = two ? launch_epi_ext<2, 4>(h, epi, plan, tm, stream)
+                                                       : launch_epi_ext<1, 4>(h, epi, plan, tm, stream);
+    else if (plan.p.row_stores == 1 && !split) st = plan.cfg.cta_group == 2 ? launch_epi_ext<2, 3>(h, epi, plan, tm, stream)
                                                                        : launch_epi_ext<1, 3>(h, epi, plan, tm, stream);
     else if (q.norm) st = plan.cfg.cta_group == 2 ? launch_epi_ext<2, 2>(h, epi, plan, tm, stream)
                                                   : launch_epi_ext<1, 2>(h, epi, plan, tm, stream);

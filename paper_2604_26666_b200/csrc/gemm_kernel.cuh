@@ -157,8 +157,10 @@ struct GemmParams {
   const float* colsum;     // [N_out]: sum over k of the folded W[n][k] (LayerNorm only)
   int norm_mode;
   float norm_eps;
-  // EXT = 3 instantiations: the staged epilogue's arithmetic, but every thread stores its own row's 128 bytes of a
+  // 1 (EXT = 3 instantiations): the staged epilogue's arithmetic, but every thread stores its own row's 128 bytes of a
   // chunk straight from registers as four 32-byte stores (no staging traffic through shared memory)
+  // 2 (EXT = 4 instantiations; 1 and 2 as well): the staged epilogue, but the warp writes a chunk's rows out itself in
+  // element-aligned words, for outputs that tensor stores cannot address (write_rows_any)
   int row_stores;
   // bit 256: the first CTA counts where its cycles go (fact_last_kernel_profile).  In a -DFACT_EXPERIMENTS build
   // also the work-skipping switches: 1 = no loads, MMA on stale shared memory; 2 = loads only, no MMA; 4 = the
@@ -795,6 +797,46 @@ __device__ __forceinline__ uint64_t epilogue_pair(uint64_t acc, uint64_t up, uin
   }
 }
 
+// One warp writes a staged chunk (32 rows of 128 bytes, 128-byte swizzle) to rows of any alignment: a row at a time,
+// 32 consecutive 4-byte words per instruction.  FP32 elements are such words; BF16 pairs are where the row starts on a
+// 4-byte boundary, and otherwise pairs shifted by one element, put together from neighbouring lanes, with the first and
+// the last element by themselves.  (A thread storing its own row writes 2 bytes to 32 sectors per instruction:
+// 283 x 6642 x 4232 to BF16 59.3 us that way, 33.0 this way; 8000 x 8001 x 512 685 and 106; 1962 x 5451 x 4808 to FP32 163
+// and 108.)
+__device__ __forceinline__ void write_rows_any(uint8_t* dst, long long ldc, bool f32, uint32_t buf, int rows, int cols, int lane) {
+  const long long row_bytes = ldc * (f32 ? 4 : 2);
+  for (int r0 = 0; r0 < rows; r0 += 8) {  // (rows may be <= 0; warp-uniform)
+    uint32_t v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t r = (uint32_t)(r0 + i);
+      asm volatile("ld.shared.b32 %0, [%1];"
+                   : "=r"(v[i])
+                   : "r"(buf + r * 128u + ((((uint32_t)lane >> 2) ^ (r & 7u)) << 4) + ((uint32_t)lane & 3u) * 4u)
+                   : "memory");
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (r0 + i >= rows) break;
+      uint8_t* const row = dst + (long long)(r0 + i) * row_bytes;
+      if (f32) {
+        if (lane < cols) reinterpret_cast<uint32_t*>(row)[lane] = v[i];
+      } else if ((reinterpret_cast<uintptr_t>(row) & 2u) == 0) {
+        if (2 * lane + 1 < cols) reinterpret_cast<uint32_t*>(row)[lane] = v[i];
+        else if (2 * lane < cols) reinterpret_cast<uint16_t*>(row)[2 * lane] = (uint16_t)v[i];
+      } else {
+        uint16_t* const e = reinterpret_cast<uint16_t*>(row);  // lane l: elements 2 l + 1 and 2 l + 2; lane 0: element 0 too
+        const uint32_t next = __shfl_down_sync(0xffffffffu, v[i], 1);
+        if (lane == 0 && cols > 0) e[0] = (uint16_t)v[i];
+        if (lane < 31 && 2 * lane + 2 < cols)
+          *reinterpret_cast<uint32_t*>(e + 2 * lane + 1) = __byte_perm(v[i], next, 0x5432);
+        else if (2 * lane + 1 < cols)
+          e[2 * lane + 1] = (uint16_t)(v[i] >> 16);
+      }
+    }
+  }
+}
+
 template <int CG, int EPI, bool SK = false, bool GROUPED = false, int EXT = 0, bool DYN = false>
 __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
     fact_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -822,12 +864,12 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
       return;
     }
   }
-  if constexpr (EXT != 0) {  // 1: row sums out; 2: a folded normalisation in (and row sums out); 3: rows stored
-                             // from registers -- all in the staged epilogue of a whole, ungrouped tile
+  if constexpr (EXT != 0) {  // 1: row sums out; 2: a folded normalisation in (and row sums out); 3: rows stored from
+                             // registers; 4: rows of any alignment -- all in the staged epilogue of a whole, ungrouped tile
     static_assert(!SK && !GROUPED && EPI != kEpiPartial && EPI != kEpiBiasSoftmax, "extras: plain data-parallel tiles");
     if (!p.store_tma || (EXT != 2 && p.norm_mode != 0) || (p.norm_mode != 0 && p.stats_in == nullptr) ||
-        (p.norm_mode == 1 && p.colsum == nullptr) || (EXT == 3) != (p.row_stores != 0) ||
-        (EXT == 3 && p.stats_out != nullptr)) {
+        (p.norm_mode == 1 && p.colsum == nullptr) || (EXT >= 3 ? p.row_stores != EXT - 2 : p.row_stores == 1) ||
+        (EXT >= 3 && p.stats_out != nullptr)) {
       if (threadIdx.x == 0) atomicExch(p.status, kDeviceTimeoutCode);
       return;
     }
@@ -1581,6 +1623,13 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
               const uint4 v = ptx::ld_shared_v4(buf + (uint32_t)r * 128u + ((uint32_t)(piece ^ (r & 7)) << 4));
               if (r < rows_left && col_ok && !FACT_SKIP(p, 4)) *reinterpret_cast<uint4*>(out_b + r * row_bytes) = v;
             }
+            ptx::fence_proxy_async_smem();  // (a residual tile may be loaded into this buffer next, by TMA)
+            __syncwarp();
+          } else if (EXT == 4 || ((EXT == 1 || EXT == 2) && p.row_stores == 2)) {
+            if (!FACT_SKIP(p, 4))
+              write_rows_any(reinterpret_cast<uint8_t*>(p.C) + ((long long)z * p.strideC + (long long)row0 * p.ldc + n_chunk) *
+                                                                    (long long)(f32 ? 4 : 2),
+                             p.ldc, f32, buf, min(32, p.M - row0), min(chunk_cols, p.N_out - n_chunk), lane);
             ptx::fence_proxy_async_smem();  // (a residual tile may be loaded into this buffer next, by TMA)
             __syncwarp();
           } else {
