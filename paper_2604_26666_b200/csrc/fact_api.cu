@@ -2435,7 +2435,7 @@ fact_status_t fact_norm(fact_handle_t h, fact_norm_t kind, int64_t M, int64_t C,
   if (C < 8 || C > 8192 || C % 8) return FACT_ERR_UNSUPPORTED;
   if (M == 0) return FACT_OK;
   if (!X || !Y || !gamma || (kind == FACT_NORM_RMS && beta) || !(eps >= 0.f)) return FACT_ERR_INVALID_ARG;
-  if (ldx < C || ldy < C || M > 0x7fffffffLL * kNormWarps) return FACT_ERR_INVALID_ARG;
+  if (ldx < C || ldy < C || M > (C <= 1024 ? 0x7fffffffLL * kNormWarps : 0x7fffffffLL)) return FACT_ERR_INVALID_ARG;
   if (!aligned16(X) || !aligned16(Y) || !aligned16(gamma) || (beta && !aligned16(beta)) || ldx % 8 || ldy % 8)
     return FACT_ERR_BAD_ALIGNMENT;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_v);
@@ -2455,17 +2455,26 @@ fact_status_t fact_norm(fact_handle_t h, fact_norm_t kind, int64_t M, int64_t C,
   const unsigned grid = (unsigned)((M + kNormWarps - 1) / kNormWarps);
   const int threads = kNormWarps * 32;
   const bool rms = kind == FACT_NORM_RMS;
-  // a lane keeps ceil(C / 256) 16-byte chunks of its row in registers
+  // Up to 1024 values a warp keeps a row in registers (four 16-byte chunks a lane); longer rows get a CTA each, and so do
+  // rows of more than 256 values where there are few of them (LayerNorm, 768 values: 1000 rows 2.5 us by warps, 1.9 by CTAs;
+  // 4096 rows 3.3 and 3.9: there the CTAs' launches are what takes the time).
   cudaError_t e;
-  if (C <= 1024) {
+  const unsigned rows = (unsigned)M;
+  if (C > 256 && C <= 1024 && M <= 2048) {
+    e = rms ? launch_pdl(h, fact_norm_long_kernel<128, 1, true>, rows, 128u, 0, stream, 1, p)
+            : launch_pdl(h, fact_norm_long_kernel<128, 1, false>, rows, 128u, 0, stream, 1, p);
+  } else if (C <= 1024) {
     e = rms ? launch_pdl(h, fact_norm_kernel<4, true>, grid, (unsigned)threads, 0, stream, 1, p)
             : launch_pdl(h, fact_norm_kernel<4, false>, grid, (unsigned)threads, 0, stream, 1, p);
+  } else if (C <= 2048) {
+    e = rms ? launch_pdl(h, fact_norm_long_kernel<256, 1, true>, rows, (unsigned)threads, 0, stream, 1, p)
+            : launch_pdl(h, fact_norm_long_kernel<256, 1, false>, rows, (unsigned)threads, 0, stream, 1, p);
   } else if (C <= 4096) {
-    e = rms ? launch_pdl(h, fact_norm_kernel<16, true>, grid, (unsigned)threads, 0, stream, 1, p)
-            : launch_pdl(h, fact_norm_kernel<16, false>, grid, (unsigned)threads, 0, stream, 1, p);
+    e = rms ? launch_pdl(h, fact_norm_long_kernel<256, 2, true>, rows, (unsigned)threads, 0, stream, 1, p)
+            : launch_pdl(h, fact_norm_long_kernel<256, 2, false>, rows, (unsigned)threads, 0, stream, 1, p);
   } else {
-    e = rms ? launch_pdl(h, fact_norm_kernel<32, true>, grid, (unsigned)threads, 0, stream, 1, p)
-            : launch_pdl(h, fact_norm_kernel<32, false>, grid, (unsigned)threads, 0, stream, 1, p);
+    e = rms ? launch_pdl(h, fact_norm_long_kernel<256, 4, true>, rows, (unsigned)threads, 0, stream, 1, p)
+            : launch_pdl(h, fact_norm_long_kernel<256, 4, false>, rows, (unsigned)threads, 0, stream, 1, p);
   }
   fact_status_t st = FACT_OK;
   if (e != cudaSuccess) st = cuda_fail(h, "norm launch", e);
