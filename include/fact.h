@@ -27,7 +27,7 @@
  *     never allocates or frees device memory on a call path; split-K scratch
  *     is a caller-provided workspace sized by fact_workspace_bytes.  The handle
  *     owns a small device status area (status word, counters, stream-K flags),
- *     a 32 KB device table for grouped calls and the tuner's table.
+ *     a 32 KB device table for calls of more than 256 groups and the tuner's table.
  *   - Calls only enqueue work on `cuda_stream` (a cudaStream_t passed as
  *     void*; NULL = the legacy default stream) and return; results are valid
  *     in stream order.
@@ -313,9 +313,10 @@ fact_status_t fact_linear(fact_handle_t handle, int64_t M, int64_t N_out, int64_
  * fact_linear.  One launch: tiles never cross a group boundary (the last tile of a group is ragged), all tiles are
  * data-parallel, the output is stored by row-predicated 16-byte stores -- staged through shared memory so that
  * they are whole 128-byte rows when Y is 16-byte aligned with ldy and N_out multiples of 16 bytes, straight from
- * registers otherwise or with cfg->store_mode == 1 (the group table travels to a buffer of
- * the handle in stream order, so grouped calls through one handle must be stream-ordered with respect to each
- * other, and not inside a stream capture: the table is copied from pageable host memory).  cfg: tile shape, pair
+ * registers otherwise or with cfg->store_mode == 1 (up to 256 groups the group
+ * table is a parameter of the kernel, and calls are free to overlap and to be captured; a table of more groups travels
+ * to a buffer of the handle in stream order, so such calls through one handle must be stream-ordered with respect to
+ * each other, and not inside a stream capture: the table is copied from pageable host memory).  cfg: tile shape, pair
  * size, stages and store mode only (K slices, stream-K and the row softmax are refused with
  * FACT_ERR_UNSUPPORTED).  groups == 0 or M == 0 is a successful no-op. */
 fact_status_t fact_linear_grouped(fact_handle_t handle, int groups, const int64_t* group_rows, int64_t N_out, int64_t K,

@@ -121,6 +121,7 @@ struct Plan {
   int smem_bytes;
   int grid;
   size_t ws_bytes;
+  const GroupTable* groups = nullptr;  // grouped: the row groups of the call in flight
   GemmParams p;
 };
 
@@ -914,8 +915,13 @@ fact_status_t launch_instance(fact_handle_t h, int slot, const Plan& plan, const
     if (e != cudaSuccess) return cuda_fail(h, "cudaFuncSetAttribute(MaxDynamicSharedMemorySize)", e);
     h->configured_mask.set((size_t)slot);
   }
-  cudaError_t e = launch_pdl(h, kern, (unsigned)plan.grid, (unsigned)(kThreads + (DYN ? 32 : 0)),
-                             (size_t)plan.smem_bytes, stream, CG, tm[0], tm[1], tm[2], tm[3], plan.p);
+  cudaError_t e;
+  if constexpr (GROUPED)
+    e = launch_pdl(h, kern, (unsigned)plan.grid, (unsigned)(kThreads + (DYN ? 32 : 0)), (size_t)plan.smem_bytes, stream, CG,
+                   tm[0], tm[1], tm[2], tm[3], plan.p, *plan.groups);
+  else
+    e = launch_pdl(h, kern, (unsigned)plan.grid, (unsigned)(kThreads + (DYN ? 32 : 0)), (size_t)plan.smem_bytes, stream, CG,
+                   tm[0], tm[1], tm[2], tm[3], plan.p, NoGroups{0});
   if (e != cudaSuccess) return cuda_fail(h, "cudaLaunchKernelEx", e);
   h->launches++;
   return FACT_OK;
@@ -1131,11 +1137,12 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
     if (dev != h->device) cudaSetDevice(dev);
     return st;
   }
-  std::vector<int> group_table;
+  std::vector<int> group_table;  // more than kParamGroups groups: goes to the handle's device buffer in stream order
+  GroupTable group_param;
   if (q.groups > 0) {
     // Grouped: tiles never cross a group boundary (a group's last m-tile is ragged), every tile is data-parallel and
-    // stored by the row-predicated direct path.  The table -- m-tiles before each group, first row of each group --
-    // goes to the handle's device buffer in stream order.
+    // stored by the row-predicated path.  The table -- m-tiles before each group, first row of each group -- is a kernel
+    // parameter.
     fact_config_t gc = plan.cfg;
     gc.split_k = 1;
     // staged through shared memory (then the warp's own row-predicated 16-byte stores) when the output's rows are
@@ -1148,24 +1155,28 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
     st = make_plan(h, q, &gc, 0, &plan);
     if (st != FACT_OK) return st;
     const int G = q.groups;
-    group_table.resize(2 * (size_t)(G + 1));
+    const bool in_param = G <= kParamGroups;
+    if (!in_param) group_table.resize(2 * (size_t)(G + 1));
+    int* const tab_tiles = in_param ? group_param.tiles : group_table.data();
+    int* const tab_rows = in_param ? group_param.rows : group_table.data() + G + 1;
     long long tiles = 0, rows = 0;
     for (int g = 0; g < G; ++g) {
-      group_table[g] = (int)tiles;
-      group_table[G + 1 + g] = (int)rows;
+      tab_tiles[g] = (int)tiles;
+      tab_rows[g] = (int)rows;
       tiles += (q.group_rows[g] + plan.cfg.tile_m - 1) / plan.cfg.tile_m;
       rows += q.group_rows[g];
     }
-    group_table[G] = (int)tiles;
-    group_table[2 * G + 1] = (int)rows;
+    tab_tiles[G] = (int)tiles;
+    tab_rows[G] = (int)rows;
     const long long units = tiles * plan.p.tiles_n;
     if (units > 0x7fffffffLL) return FACT_ERR_UNSUPPORTED;
     // slabs of m-tiles whose rows of A fit a 32 MB share of L2
     plan.p.raster_group = (int)std::max<long long>(
         1, (32LL << 20) / ((long long)plan.cfg.tile_m * std::max<long long>(q.K, 1) * (q.fp8 ? 1 : 2)));
     plan.p.groups = G;
-    plan.p.grp_tiles = h->d_groups;
-    plan.p.grp_rows = h->d_groups + (G + 1);
+    plan.groups = &group_param;
+    plan.p.grp_tiles = in_param ? nullptr : h->d_groups;
+    plan.p.grp_rows = in_param ? nullptr : h->d_groups + (G + 1);
     plan.p.total_units = (int)units;
     plan.p.strideC = 0;
     plan.p.strideR = 0;
@@ -1237,7 +1248,7 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
     const uint64_t batch_dim = (uint64_t)q.batch;
     const uint64_t b_batch_dim = q.groups > 0 ? (uint64_t)q.groups : batch_dim;  // grouped: B is W[group]
     const bool b_strided = q.batch > 1 || q.groups > 0;
-    if (q.groups > 0) {
+    if (!group_table.empty()) {
       cudaError_t e = cudaMemcpyAsync(h->d_groups, group_table.data(), group_table.size() * sizeof(int),
                                       cudaMemcpyHostToDevice, stream);  // pageable source: staged before it returns
       if (e != cudaSuccess) return cuda_fail(h, "cudaMemcpyAsync(group table)", e);

@@ -130,7 +130,8 @@ struct GemmParams {
   int reduce_epi;     // the epilogue the reduction applies
   int* status;        // [0] error word, [2..17] clock / profile counters, [24], [25] grid-barrier counters
   // grouped GEMM (the GROUPED instantiations only): the rows of A and C are cut into `groups` consecutive row
-  // groups, group g multiplies W[g]; see decode_grouped
+  // groups, group g multiplies W[g]; see decode_grouped.  Up to kParamGroups groups the two tables below are a kernel
+  // parameter of their own (GroupTable) and these pointers are null.
   int groups;
   const int* grp_tiles;   // [groups + 1] m-tiles (of tile_m rows) before each group
   const int* grp_rows;    // [groups + 1] first row of each group; grp_rows[groups] = M
@@ -166,6 +167,25 @@ struct GemmParams {
   // also the work-skipping switches: 1 = no loads, MMA on stale shared memory; 2 = loads only, no MMA; 4 = the
   // epilogue skips its global stores (they isolate the feed, issue and store ceilings; results are garbage).
   int debug;
+};
+
+// The row groups of a grouped GEMM as a kernel parameter: nothing to copy to the device ahead of the launch (a copy from
+// pageable memory in stream order costs the stream 4 us and the next launch its overlap), nothing shared between calls.
+constexpr int kParamGroups = 256;
+struct GroupTable {
+  int tiles[kParamGroups + 1];  // m-tiles before each group
+  int rows[kParamGroups + 1];   // first row of each group; the last entry is M
+};
+struct NoGroups {
+  int unused;
+};
+template <bool GROUPED>
+struct GroupArg {
+  using type = NoGroups;
+};
+template <>
+struct GroupArg<true> {
+  using type = GroupTable;
 };
 
 struct WorkUnit {
@@ -221,17 +241,20 @@ __device__ __forceinline__ WorkUnit decode_unit(const GemmParams& p, int u) {
 // the prefix table of m-tiles.  Inside a group the walk takes slabs of `raster_group` m-tiles (their rows of A stay
 // in L2) and, within a slab, the m-tiles fastest: CTAs that run at the same time then share the group's weight
 // columns, which are streamed once per slab.
-__device__ __forceinline__ WorkUnit decode_grouped(const GemmParams& p, int u) {
+__device__ __forceinline__ WorkUnit decode_grouped(const GemmParams& p, const GroupTable& tab, int u) {
+  const bool in_param = p.grp_tiles == nullptr;
+  auto tiles_before = [&](int g) { return in_param ? tab.tiles[g] : __ldg(p.grp_tiles + g); };
+  auto first_row = [&](int g) { return in_param ? tab.rows[g] : __ldg(p.grp_rows + g); };
   WorkUnit w;
   const int mt = u / p.tiles_n;
   int lo = 0, hi = p.groups;  // invariant: grp_tiles[lo] <= mt < grp_tiles[hi]
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if (__ldg(p.grp_tiles + mid) <= mt) lo = mid;
+    if (tiles_before(mid) <= mt) lo = mid;
     else hi = mid;
   }
-  const int first = __ldg(p.grp_tiles + lo);
-  const int mtiles = __ldg(p.grp_tiles + lo + 1) - first;  // m-tiles of this group (> 0: empty groups own no unit)
+  const int first = tiles_before(lo);
+  const int mtiles = tiles_before(lo + 1) - first;  // m-tiles of this group (> 0: empty groups own no unit)
   const int local = u - first * p.tiles_n;
   const int per_slab = p.raster_group * p.tiles_n;
   const int slab = local / per_slab;
@@ -240,8 +263,8 @@ __device__ __forceinline__ WorkUnit decode_grouped(const GemmParams& p, int u) {
   w.tn = rem / height;
   w.tm = slab * p.raster_group + (rem - w.tn * height);
   w.b = lo;
-  w.m_base = __ldg(p.grp_rows + lo);
-  w.m_end = __ldg(p.grp_rows + lo + 1);
+  w.m_base = first_row(lo);
+  w.m_end = first_row(lo + 1);
   w.split = 0;
   w.kb_begin = 0;
   w.kb_end = p.k_blocks;
@@ -307,8 +330,10 @@ struct UnitWalk {
   int slot;
   uint32_t phase;
   const SchedCtx* sc;
-  __device__ __forceinline__ UnitWalk(const GemmParams& p, int unit0, int unit_stride, const SchedCtx* sched = nullptr)
-      : u(unit0), stride(unit_stride), wave(0), sk_pos(0), sk_end(0), group(unit0), slot(0), phase(0), sc(sched) {
+  const typename GroupArg<GROUPED>::type& grp;
+  __device__ __forceinline__ UnitWalk(const GemmParams& p, int unit0, int unit_stride, const SchedCtx* sched,
+                                      const typename GroupArg<GROUPED>::type& grp_)
+      : u(unit0), stride(unit_stride), wave(0), sk_pos(0), sk_end(0), group(unit0), slot(0), phase(0), sc(sched), grp(grp_) {
     if constexpr (SK) {
       sk_pos = sk_group_begin(p.sk_len, p.sk_rem, unit0);
       sk_end = sk_group_begin(p.sk_len, p.sk_rem, unit0 + 1);
@@ -365,7 +390,7 @@ struct UnitWalk {
       if (u >= p.total_units) return false;
     }
     if constexpr (GROUPED) {
-      w = decode_grouped(p, u);
+      w = decode_grouped(p, grp, u);
     } else {
       w = decode_unit(p, u);
       w.m_base = 0;
@@ -841,7 +866,7 @@ template <int CG, int EPI, bool SK = false, bool GROUPED = false, int EXT = 0, b
 __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
     fact_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmR,
-                     const GemmParams p) {
+                     const GemmParams p, const __grid_constant__ typename GroupArg<GROUPED>::type grp) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
 
   // The warp index is made provably warp-uniform (a shuffle result), and the producer / MMA roles
@@ -859,7 +884,7 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
   }
   if constexpr (GROUPED) {  // (group boundaries are kept by row-predicated stores, staged or direct)
     static_assert(!SK && EPI != kEpiPartial, "grouped tiles are data-parallel");
-    if (p.grp_tiles == nullptr || p.grp_rows == nullptr) {
+    if ((p.grp_tiles == nullptr) != (p.grp_rows == nullptr) || (p.grp_tiles == nullptr && p.groups > kParamGroups)) {
       if (threadIdx.x == 0) atomicExch(p.status, kDeviceTimeoutCode);
       return;
     }
@@ -993,7 +1018,7 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      UnitWalk<SK, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched);
+      UnitWalk<SK, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched, grp);
       WorkUnit w;
       while (ok && walk.next(p, w)) {
         // Odd waves walk K downwards: the wave before ended at the top of K, so the operand slabs both waves
@@ -1083,7 +1108,7 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
       uint32_t acc_phase = 0;
       bool ok = true;
       long long prof_acc_wait = 0, prof_full_wait = 0, prof_first_full = 0;
-      UnitWalk<SK, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched);
+      UnitWalk<SK, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched, grp);
       WorkUnit w;
       while (ok && walk.next(p, w)) {
         long long t0 = prof ? clock64() : 0;
@@ -1151,7 +1176,7 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
       else issue_all(FactFalse{});
     } else if constexpr (DYN) {
       // the peer's MMA warp issues nothing, but it is one of the warps the scheduler counts: it walks the list
-      UnitWalk<SK, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched);
+      UnitWalk<SK, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched, grp);
       WorkUnit w;
       while (walk.next(p, w)) {
       }
@@ -1226,7 +1251,7 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
       long long prof_epi_busy = 0, prof_epi_wait = 0, prof_tiles = 0;
       uint32_t gc = 0;      // chunks this warp has stored so far: buffer = gc % bufs
       uint32_t r_next = 0;  // residual loads have been issued for every chunk counter below this
-      UnitWalk<SK, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched);
+      UnitWalk<SK, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched, grp);
       WorkUnit w;
       // hand the accumulator back to the MMA issuer (of the leader CTA) and move on to the other one
       // (a relaxed arrival: the barrier orders tensor-memory reads only, which the tcgen05 fences take care of; a
@@ -1674,7 +1699,7 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
       // ---- direct: each thread stores its own row from registers (any alignment, any leading dimension)
       const bool c_vec = p.c_vec != 0;
       uint32_t xch_count = 0;  // exchanges with the other warp of the lane quarter so far (row softmax only)
-      UnitWalk<false, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched);  // (stream-K always stores through the staged path)
+      UnitWalk<false, GROUPED, DYN, CG> walk(p, unit0, unit_stride, sched, grp);  // (stream-K always stores through the staged path)
       WorkUnit w;
       while (ok && walk.next(p, w)) {
         if (!wait_all(accf_bar(acc), acc_phase)) {  // (a warp-uniform verdict: what follows is warp-wide)

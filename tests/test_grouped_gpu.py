@@ -191,3 +191,43 @@ def test_grouped_benchmark_shape_sampled_rows(h):
         c, t = gates(ref, to_f64(out[idx]), "bf16", case.epilogue)
         worst_c, worst_t = max(worst_c, c), max(worst_t, t)
     assert worst_c <= 1.0 and worst_t <= 1.0, (worst_c, worst_t)
+
+
+@pytest.mark.parametrize("groups", [255, 256, 257])
+def test_group_tables_as_a_parameter_and_in_device_memory(h, groups):
+    """Up to 256 groups the table is a kernel parameter, beyond that it is copied to the device: the same sums (exact on
+    integers) either way, some groups empty, the sizes different in consecutive calls on two streams."""
+    g = torch.Generator().manual_seed(groups)
+    K, N = 72, 64
+    W = torch.randint(-2, 3, (groups, N, K), generator=g).to(torch.bfloat16)
+    sides = [torch.cuda.Stream(), torch.cuda.Stream()] if groups <= 256 else [torch.cuda.current_stream()] * 2
+    Wd = W.cuda()
+    for turn in range(4):
+        rows = torch.randint(0, 9, (groups,), generator=g).tolist()
+        M = sum(rows)
+        X = torch.randint(-2, 3, (M, K), generator=g).to(torch.bfloat16)
+        Xd = X.cuda()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(sides[turn % 2]):
+            y = h.linear_grouped(Xd, Wd, rows)
+        ref = torch.cat([x.double() @ W[i].double().t() for i, x in enumerate(X.split(rows))])
+        torch.cuda.synchronize()
+        assert torch.equal(y.cpu().double(), ref.to(torch.bfloat16).double())
+    assert h.device_status() == 0
+
+
+def test_grouped_call_in_a_cuda_graph(h):
+    g = torch.Generator().manual_seed(3)
+    rows, K, N = [100, 0, 157, 30], 128, 192
+    X = torch.randint(-2, 3, (sum(rows), K), generator=g).to(torch.bfloat16).cuda()
+    W = torch.randint(-2, 3, (len(rows), N, K), generator=g).to(torch.bfloat16).cuda()
+    want = h.linear_grouped(X, W, rows).clone()
+    out = torch.zeros_like(want)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        h.linear_grouped(X, W, rows, out=out)
+    for _ in range(2):
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
