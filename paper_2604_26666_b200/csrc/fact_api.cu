@@ -443,9 +443,14 @@ fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const f
     // at 128 columns and 420 at 64 -- 0.57 and 0.45 -- which is what the comparison with the cluster schedule uses)
     const double eff = tn >= 256 ? 1.0 : (tn >= 192 ? 0.85 : (!calibrated ? 0.65 : (tn >= 128 ? 0.57 : 0.45)));
     auto per_tile = [&](double kb) {
-      return kb * 512.0 * std::max(tn, 96) / 256.0 / eff + 1500.0 + (cg == 1 ? 60.0 * kb : 0.0);
+      return kb * 512.0 * std::max(tn, 96) / 256.0 / eff + 1500.0 + (cg == 1 ? (tn >= 192 ? 120.0 : (tn >= 128 ? 100.0 : 30.0)) * kb : 0.0);
     };
-    double best_cost = (double)((tiles + slots - 1) / slots) * per_tile(k_blocks_all);
+    // (a pair's launch costs about 1 us more -- cluster placement, the pair's barriers: 744 x 768 -> 2304 takes 7.3 us as
+    // pairs of 128-column tiles and 6.6 as single CTAs, 2000 rows 9.7 and 8.8 with 256 columns -- which its cheaper k-blocks
+    // earn back from about fifteen on, as a single CTA's tile is bound by what an SM takes in from L2: 5811 x 1304 -> 376
+    // 12.6 us as single CTAs, 11.7 as pairs; tiles of 64 columns from sixty on)
+    const double best_launch = cg == 2 ? 1800.0 : 0.0;
+    double best_cost = (double)((tiles + slots - 1) / slots) * per_tile(k_blocks_all) + best_launch;
     int best_s = 1;
     if (may_slice) {
       const double plane_bytes = (double)q.M * (double)round_up((int)q.N_out, 4) * 4.0 * ws_planes_for(q);
