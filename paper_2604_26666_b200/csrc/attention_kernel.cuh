@@ -25,6 +25,7 @@
 // came from, as tensor memory forces at BK = 128 and head_dim 128, every block is a serial chain softmax ->
 // O += P V -> next S -> softmax, and a tile-block takes 1900 cycles instead of the 1100 the exponentials need.)
 // In a causal problem tile 0 may see one key block fewer than tile 1; its issuer releases that block's slots unused.
+// Sequences of at most 128 queries have items of another kind (MODE).
 // Every mbarrier wait is bounded, as in the GEMM kernel.
 #pragma once
 #include <cuda.h>
@@ -107,9 +108,11 @@ __device__ __forceinline__ uint64_t attn_exp2_poly(uint64_t x2) {
 }
 
 struct AttnItem {
-  int b, h, kvh, t0;
-  int nb0, nb1;  // key blocks tile 0 / tile 1 see
-  int nbi;       // key blocks the item loads
+  int b, h, kvh, t0;   // of tile 0 (tile 1: the same head 128 rows on, or, with two heads per item, b1, h1, kvh1 at row 0)
+  int b1, h1, kvh1;
+  int nb0, nb1;        // key blocks tile 0 / tile 1 see
+  int nbi;             // key blocks the item loads
+  bool store1;
 };
 
 // Which items a CTA works through, decided on the host for causal problems of few rounds: the items in order of
@@ -133,7 +136,17 @@ struct AttnDealArg<true> {
   using type = AttnDeal;
 };
 
-template <int HD, bool DEAL = false>  // head_dim: 64 or 128; DEAL: the items come from the host's list
+// HD: head_dim, 64 or 128.  DEAL: the items come from the host's list.  MODE: what an item is --
+//   kAttnRows   256 query rows of one head, as two tiles;
+//   kAttnPair   sequences of at most 128 queries, which fill one tile: two query heads, tile t the whole sequence of head
+//               2 i + t; the two tiles' key blocks alternate in the rings, each released by the one issuer that uses it;
+//   kAttnHalf   the same sequences where there are no more heads than SMs: one head, tile 0 only; tile 1 passes its
+//               hand-overs on and releases the blocks unused.
+// (As 256-row items such sequences computed a second tile of padding: 106 x 97 x 12 heads of 64 34.0 -> 19.3 us,
+// 256 x 64 x 12 73.2 -> 35.5, 60 x 128 x 32 heads of 128 50.5 -> 34.4 in pairs; 7 x 84 x 32 heads of 128 11.1 -> 8.4 as
+// halves.)
+enum : int { kAttnRows = 0, kAttnPair = 1, kAttnHalf = 2 };
+template <int HD, bool DEAL = false, int MODE = kAttnRows>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     fact_attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
@@ -149,6 +162,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   const bool prof = (p.debug & 256) && blockIdx.x == 0;
   const long long t_entry = prof ? clock64() : 0;
   const unsigned long long ns_entry = prof ? ptx::globaltimer_ns() : 0ull;
+  constexpr bool PAIR = MODE == kAttnPair, HALF = MODE == kAttnHalf;
+  static_assert(MODE == kAttnRows || !DEAL, "short sequences' items weigh the same");
   constexpr int BK = attn_block_k(HD);              // keys per block
   constexpr uint32_t tile_bytes = attn_tile_bytes(HD);   // a 128-row tile (Q, O)
   constexpr uint32_t kv_bytes = attn_kv_bytes(HD);  // a BK-row tile (K, V)
@@ -190,7 +205,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     const int i = (int)threadIdx.x;
     uint32_t count = 1;
     if ((i >= S_READ && i < P_FULL + 2) || (i >= O_FREE && i < O_STAGED + 2)) count = 4;  // one arrival per softmax warp
-    if (i >= K_EMPTY) count = 2;                                                          // one per issuer
+    if (i >= K_EMPTY) count = PAIR ? 1 : 2;                                               // one per issuer that uses it
     ptx::mbar_init(bar(i), count);
     if (i == 0) *abort_p = 0;
     ptx::fence_mbar_init();
@@ -233,18 +248,37 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   auto item_of = [&](int n) -> AttnItem {
     int idx = n * G + pos_in_round(n);
     if constexpr (DEAL) idx = deal.list[deal_first + n];
-    const int qr = idx / bh_count;
-    const int bh = idx - qr * bh_count;
-    const int qp = p.causal ? (p.q_pairs - 1 - qr) : qr;
     AttnItem it;
-    it.h = bh % p.Hq;
-    it.b = bh / p.Hq;
-    it.kvh = it.h / (p.Hq / p.Hkv);
-    it.t0 = qp * 2 * kAttnBlockQ;
-    // causal: a tile whose last row is r sees keys 0 .. r
-    it.nb0 = p.causal ? min(kv_blocks_all, (it.t0 + kAttnBlockQ - 1) / BK + 1) : kv_blocks_all;
-    it.nb1 = p.causal ? min(kv_blocks_all, (it.t0 + 2 * kAttnBlockQ - 1) / BK + 1) : kv_blocks_all;
-    it.nbi = it.nb1;
+    if constexpr (PAIR) {
+      const int bh0 = 2 * idx, bh1 = min(2 * idx + 1, bh_count - 1);  // (an odd count: the last head twice, stored once)
+      it.h = bh0 % p.Hq;
+      it.b = bh0 / p.Hq;
+      it.kvh = it.h / (p.Hq / p.Hkv);
+      it.h1 = bh1 % p.Hq;
+      it.b1 = bh1 / p.Hq;
+      it.kvh1 = it.h1 / (p.Hq / p.Hkv);
+      it.t0 = 0;
+      it.nb0 = it.nb1 = kv_blocks_all;  // (causal: as many keys as queries, so every block holds a visible key)
+      it.nbi = 2 * kv_blocks_all;
+      it.store1 = bh0 + 1 < bh_count;
+    } else {
+      const int qr = idx / bh_count;
+      const int bh = idx - qr * bh_count;
+      const int qp = p.causal ? (p.q_pairs - 1 - qr) : qr;
+      it.h = it.h1 = bh % p.Hq;
+      it.b = it.b1 = bh / p.Hq;
+      it.kvh = it.kvh1 = it.h / (p.Hq / p.Hkv);
+      it.t0 = qp * 2 * kAttnBlockQ;
+      // causal: a tile whose last row is r sees keys 0 .. r
+      it.nb0 = p.causal ? min(kv_blocks_all, (it.t0 + kAttnBlockQ - 1) / BK + 1) : kv_blocks_all;
+      it.nb1 = p.causal ? min(kv_blocks_all, (it.t0 + 2 * kAttnBlockQ - 1) / BK + 1) : kv_blocks_all;
+      it.nbi = it.nb1;
+      if constexpr (HALF) {
+        it.nbi = it.nb0;
+        it.nb1 = 0;
+      }
+      it.store1 = it.t0 + kAttnBlockQ < p.Tq;
+    }
     return it;
   };
   auto wait_all = [&](uint32_t br, uint32_t parity) -> bool {
@@ -276,11 +310,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (ok && ptx::elect_one()) {
             ptx::mbar_arrive_expect_tx(bar(Q_FULL + t), tile_bytes);
             for (int c = 0; c < chunks; ++c)
-              ptx::tma_load_4d(q_s0 + (uint32_t)t * tile_bytes + c * kAttnChunkBytes, &tmQ, bar(Q_FULL + t), c * 64, it.h,
-                               it.t0 + t * kAttnBlockQ, it.b);
+              ptx::tma_load_4d(q_s0 + (uint32_t)t * tile_bytes + c * kAttnChunkBytes, &tmQ, bar(Q_FULL + t), c * 64,
+                               t ? it.h1 : it.h, PAIR ? 0 : it.t0 + t * kAttnBlockQ, t ? it.b1 : it.b);
           }
         }
-        for (int j = 0; ok && j < it.nbi; ++j, ++g) {
+        for (int r = 0; ok && r < it.nbi; ++r, ++g) {
+          const int j = PAIR ? r >> 1 : r;                        // key block ...
+          const int kvh = (PAIR && (r & 1)) ? it.kvh1 : it.kvh;   // ... of the head of tile r % 2 (of both tiles' one head)
+          const int kb = (PAIR && (r & 1)) ? it.b1 : it.b;
           const int s = slot_of(g);
           const uint32_t par = pass_of(g) ^ 1u;  // an empty slot's first wait passes
           ok = wait_all(bar(K_EMPTY + s), par);
@@ -288,7 +325,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (ptx::elect_one()) {
             ptx::mbar_arrive_expect_tx(bar(K_FULL + s), kv_bytes);
             for (int c = 0; c < chunks; ++c)
-              ptx::tma_load_4d_hint(k_s0 + s * kv_bytes + c * kv_chunk, &tmK, bar(K_FULL + s), c * 64, it.kvh, j * BK, it.b,
+              ptx::tma_load_4d_hint(k_s0 + s * kv_bytes + c * kv_chunk, &tmK, bar(K_FULL + s), c * 64, kvh, j * BK, kb,
                                     keep);
           }
           ok = wait_all(bar(V_EMPTY + s), par);
@@ -296,7 +333,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (ptx::elect_one()) {
             ptx::mbar_arrive_expect_tx(bar(V_FULL + s), kv_bytes);
             for (int c = 0; c < chunks; ++c)
-              ptx::tma_load_4d_hint(v_s0 + s * kv_bytes + c * kv_chunk, &tmV, bar(V_FULL + s), c * 64, it.kvh, j * BK, it.b,
+              ptx::tma_load_4d_hint(v_s0 + s * kv_bytes + c * kv_chunk, &tmV, bar(V_FULL + s), c * 64, kvh, j * BK, kb,
                                     keep);
           }
         }
@@ -335,36 +372,44 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       };
       for (int n = 0; ok && n < n_items; ++n) {
         const AttnItem it = item_of(n);
-        const int nbt = (t ? it.nb1 : it.nb0);
+        const int nbt = t ? it.nb1 : it.nb0;
+        auto ring = [&](int j) { return g + (PAIR ? 2 * j + t : j); };  // where the tile's j-th block is in the rings
         ok = wait_all(bar(Q_FULL + t), (uint32_t)n & 1u);
-        // the scores of the previous item's last block have been read (every other block's S_READ is waited for below)
-        if (ok && gt > 0) ok = wait_all(bar(S_READ + t), (uint32_t)(gt - 1) & 1u);
-        if (ok) ok = wait_all(bar(K_FULL + slot_of(g)), pass_of(g));
-        if (!ok) break;
-        issue_s(slot_of(g), nbt == 1);
-        for (int j = 0; ok && j < it.nbi; ++j) {
+        if (HALF && t == 1) {  // no rows: the tile's Q buffer is free again, and its blocks are released unused
+          if (ok && ptx::elect_one()) ptx::mbar_arrive(bar(Q_EMPTY + t));
+          if (ok) ok = wait_all(bar(K_FULL + slot_of(g)), pass_of(g));
+          if (!ok) break;
+          if (ptx::elect_one()) ptx::mbar_arrive(bar(K_EMPTY + slot_of(g)));
+        } else {
+          // the scores of the previous item's last block have been read (every other block's S_READ is waited for below)
+          if (ok && gt > 0) ok = wait_all(bar(S_READ + t), (uint32_t)(gt - 1) & 1u);
+          if (ok) ok = wait_all(bar(K_FULL + slot_of(ring(0))), pass_of(ring(0)));
+          if (!ok) break;
+          issue_s(slot_of(ring(0)), nbt == 1);
+        }
+        for (int j = 0; ok && j < (PAIR ? nbt : it.nbi); ++j) {
           // ---- the next block's scores, as soon as this block's have been read
-          if (j + 1 < it.nbi) {
-            const int s1 = slot_of(g + j + 1);
+          if (j + 1 < (PAIR ? nbt : it.nbi)) {
+            const int s1 = slot_of(ring(j + 1));
             if (j + 1 < nbt) {
               ok = wait_all(bar(S_READ + t), (uint32_t)gt & 1u);
-              if (ok) ok = wait_all(bar(K_FULL + s1), pass_of(g + j + 1));
+              if (ok) ok = wait_all(bar(K_FULL + s1), pass_of(ring(j + 1)));
               if (!ok) break;
               issue_s(s1, j + 1 == nbt - 1);
             } else {
               // a block this tile does not see (causal, tile 0): release its K slot unused, once it has been filled
-              ok = wait_all(bar(K_FULL + s1), pass_of(g + j + 1));
+              ok = wait_all(bar(K_FULL + s1), pass_of(ring(j + 1)));
               if (!ok) break;
               if (ptx::elect_one()) ptx::mbar_arrive(bar(K_EMPTY + s1));
             }
           }
           // ---- this block's second product
-          const int s = slot_of(g + j);
+          const int s = slot_of(ring(j));
           if (j < nbt) {
             ok = wait_all(bar(P_FULL + t), (uint32_t)gt & 1u);
             // the first block of an item overwrites O_t: the previous item's epilogue must have read it
             if (ok && j == 0 && n > 0) ok = wait_all(bar(O_FREE + t), (uint32_t)(n - 1) & 1u);
-            if (ok) ok = wait_all(bar(V_FULL + s), pass_of(g + j));
+            if (ok) ok = wait_all(bar(V_FULL + s), pass_of(ring(j)));
             if (!ok) break;
             ptx::tc_fence_after();
             if (ptx::elect_one()) {
@@ -380,7 +425,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             }
             ++gt;
           } else {
-            ok = wait_all(bar(V_FULL + s), pass_of(g + j));
+            ok = wait_all(bar(V_FULL + s), pass_of(ring(j)));
             if (!ok) break;
             if (ptx::elect_one()) ptx::mbar_arrive(bar(V_EMPTY + s));
           }
@@ -397,9 +442,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           ok = wait_all(bar(O_STAGED + t), (uint32_t)n & 1u);
           if (!ok) break;
           if (lane == 0) {  // bulk groups belong to the issuing thread
-            const int t0 = it.t0 + t * kAttnBlockQ;
-            if (t0 < p.Tq) {  // (a second tile wholly past the end of the sequence computed on zero-filled Q)
-              for (int c = 0; c < chunks; ++c) ptx::tma_store_4d(&tmO, o_stage + c * kAttnChunkBytes, c * 64, it.h, t0, it.b);
+            if (t == 0 || it.store1) {
+              for (int c = 0; c < chunks; ++c)
+                ptx::tma_store_4d(&tmO, o_stage + c * kAttnChunkBytes, c * 64, t ? it.h1 : it.h,
+                                  PAIR ? 0 : it.t0 + t * kAttnBlockQ, t ? it.b1 : it.b);
               ptx::bulk_commit_group();
               ptx::bulk_wait_group_read<0>();  // the staging buffer may be rewritten
             }
@@ -426,8 +472,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     int gt = 0;
     for (int n = 0; ok && n < n_items; ++n) {
       const AttnItem it = item_of(n);
-      const int nbt = (t ? it.nb1 : it.nb0);
-      const int t_row = it.t0 + t * kAttnBlockQ + row;
+      const int nbt = t ? it.nb1 : it.nb0;
+      const int t_row = PAIR ? row : it.t0 + t * kAttnBlockQ + row;
       float m = -INFINITY;  // reference maximum of scale_log2 * score the exponentials are taken against
       float l = 0.f;        // running sum of 2^(scale_log2 * score - m)
       for (int j = 0; ok && j < nbt; ++j, ++gt) {
@@ -551,6 +597,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (lane == 0) ptx::mbar_arrive(bar(P_FULL + t));
       }
       if (!ok) break;
+      if constexpr (HALF) {
+        if (t == 1) {
+          // No rows: the hand-overs only, no sooner than the store warp has come to them -- an arrival ahead of its turn
+          // could overrun the one-bit phase.
+          ok = wait_all(bar(OS_DONE + 0), (uint32_t)n & 1u);
+          if (!ok) break;
+          __syncwarp();
+          if (lane == 0) {
+            ptx::mbar_arrive(bar(O_FREE + t));
+            ptx::mbar_arrive(bar(O_STAGED + t));
+          }
+          continue;
+        }
+      }
       // ---- the tile's output: O_t / l as BF16 into the staging tile (128-byte rows of 64 columns, 16-byte pieces
       // swizzled by the row like every other tile here), which tiles 0 and 1 of every item use in turn
       const long long te0 = prof ? clock64() : 0;

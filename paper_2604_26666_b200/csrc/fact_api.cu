@@ -1053,7 +1053,9 @@ fact_status_t launch_reduce(fact_handle_t h, const Problem& q, const Plan& plan,
   r.ldr = q.ldr;
   r.strideR = q.strideR;
   r.alpha = q.fp8 ? q.alpha : 1.f;
-  const long long total = 4LL * r.batch * r.M * ((r.N_out + 3) / 4);  // four threads per group of 4 columns
+  const long long groups = (long long)r.batch * r.M * ((r.N_out + 3) / 4);
+  r.lanes_log2 = reduce_lanes_log2(groups, (long long)h->sm_count * 16 * 128, splits, r.epi == kEpiSiluGate);
+  const long long total = groups << r.lanes_log2;  // threads that share a group of 4 columns
   const int blocks = (int)std::min<long long>((total + 127) / 128, (long long)h->sm_count * 16);
   cudaError_t e = launch_pdl(h, fact_splitk_reduce_kernel, (unsigned)std::max(1, blocks), 128u, 0, stream, 1, r);
   if (e != cudaSuccess) return cuda_fail(h, "split-K reduce launch", e);
@@ -1241,6 +1243,9 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
       plan.p.fused_reduce = !(plan.cfg.split_k <= kReduceWideSlices && q.epi != FACT_EPI_SILU_GATE &&
                               (plan.p.ws_ld & 7) == 0);
       plan.p.reduce_epi = (int)q.epi;
+      plan.p.reduce_lanes_log2 =
+          reduce_lanes_log2((long long)q.batch * q.M * ((q.N_out + 3) / 4), (long long)plan.grid * kThreads,
+                            plan.cfg.split_k, q.epi == FACT_EPI_SILU_GATE);
     }
     if (h->debug_flags & 256) {  // the all-CTA span stamps start from "no start yet" / "no end yet"
       cudaMemsetAsync(h->d_status + 40, 0xff, 2 * sizeof(int), stream);
@@ -2372,7 +2377,10 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     p.status = h->d_status;
     p.debug = h->debug_flags;
     p.q_pairs = (int)((seq_q + 2 * kAttnBlockQ - 1) / (2 * kAttnBlockQ));  // an item is two tiles of 128 query rows
-    const long long items = (long long)p.q_pairs * heads_q * batch;
+    // ... or, for sequences that fit one tile, two heads' tiles once there are more heads than SMs, one head's before that
+    const bool one_tile = seq_q <= kAttnBlockQ;
+    const bool pair = one_tile && batch * heads_q > h->sm_count;
+    const long long items = pair ? (batch * heads_q + 1) / 2 : (long long)p.q_pairs * heads_q * batch;
     if (items > 0x7fffffffLL) {
       if (dev != h->device) cudaSetDevice(dev);
       return FACT_ERR_UNSUPPORTED;
@@ -2380,27 +2388,31 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     p.items = (int)items;
     const long long ctas = std::min<long long>(p.items, h->sm_count);  // persistent: one CTA per SM
     const int smem = std::max((int)attn_smem_bytes(p.D), kMinSmemRequest);
+    typedef void (*Plain)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams, AttnNoDeal);
+    typedef void (*Dealt)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams, AttnDeal);
+    static const Plain plain[2][3] = {{fact_attention_kernel<64, false, kAttnRows>, fact_attention_kernel<64, false, kAttnPair>,
+                                       fact_attention_kernel<64, false, kAttnHalf>},
+                                      {fact_attention_kernel<128, false, kAttnRows>, fact_attention_kernel<128, false, kAttnPair>,
+                                       fact_attention_kernel<128, false, kAttnHalf>}};
+    static const Dealt dealt[2] = {fact_attention_kernel<64, true>, fact_attention_kernel<128, true>};
     if (!h->configured_mask.test(30)) {
-      cudaError_t e = cudaFuncSetAttribute(fact_attention_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fact_attention_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fact_attention_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fact_attention_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-      cudaFuncAttributes fa, fb;
-      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fact_attention_kernel<64, false>);
-      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fb, fact_attention_kernel<128, false>);
-      if (e == cudaSuccess) fa.numRegs = std::min(fa.numRegs, fb.numRegs);
-      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fb, fact_attention_kernel<64, true>);
-      if (e == cudaSuccess) fa.numRegs = std::min(fa.numRegs, fb.numRegs);
-      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fb, fact_attention_kernel<128, true>);
-      if (e == cudaSuccess) fa.numRegs = std::min(fa.numRegs, fb.numRegs);
+      cudaError_t e = cudaSuccess;
+      int regs = 1 << 30;
+      auto configure = [&](const void* kern) {
+        cudaFuncAttributes fa;
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+        if (e == cudaSuccess) regs = std::min(regs, fa.numRegs);
+      };
+      for (int d = 0; d < 2; ++d) {
+        for (Plain k : plain[d]) configure(reinterpret_cast<const void*>(k));
+        configure(reinterpret_cast<const void*>(dealt[d]));
+      }
       if (e != cudaSuccess) {
         st = cuda_fail(h, "cudaFuncSetAttribute(attention)", e);
-      } else if (fa.numRegs < kAttnRegsAtLaunch) {
+      } else if (regs < kAttnRegsAtLaunch) {
         // the kernel's register rebalancing would wait forever for registers the CTA does not own
-        h->last_error = "attention kernel compiled with " + std::to_string(fa.numRegs) + " registers per thread, needs " +
+        h->last_error = "attention kernel compiled with " + std::to_string(regs) + " registers per thread, needs " +
                         std::to_string(kAttnRegsAtLaunch);
         st = FACT_ERR_UNSUPPORTED;
       } else {
@@ -2413,7 +2425,7 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
       // the host deals the items out itself -- heaviest first, each to the CTA with the least so far -- and hands the
       // list to the kernel as a parameter.  The list is kept for the next call of the same shape.
       const int bk = head_dim == 64 ? 128 : 64;
-      const bool deal = causal != 0 && p.items > ctas && p.items <= kAttnDealItems && ctas <= kAttnDealCtas &&
+      const bool deal = causal != 0 && !one_tile && p.items > ctas && p.items <= kAttnDealItems && ctas <= kAttnDealCtas &&
                         p.items < 16 * ctas;
       if (deal) {
         const std::array<long long, 6> key = {(long long)batch * heads_q, (long long)p.q_pairs, (long long)bk, (long long)seq_kv, (long long)ctas, (long long)seq_q};
@@ -2425,16 +2437,13 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
       }
       const AttnNoDeal none = {0};
       cudaError_t e;
+      const int d = head_dim == 128;
       if (deal)
-        e = head_dim == 64 ? launch_pdl(h, fact_attention_kernel<64, true>, (unsigned)ctas, (unsigned)kAttnThreads,
-                                        (size_t)smem, stream, 1, tq, tk, tv, to, p, *h->attn_deal)
-                           : launch_pdl(h, fact_attention_kernel<128, true>, (unsigned)ctas, (unsigned)kAttnThreads,
-                                        (size_t)smem, stream, 1, tq, tk, tv, to, p, *h->attn_deal);
+        e = launch_pdl(h, dealt[d], (unsigned)ctas, (unsigned)kAttnThreads, (size_t)smem, stream, 1, tq, tk, tv, to, p,
+                       *h->attn_deal);
       else
-        e = head_dim == 64 ? launch_pdl(h, fact_attention_kernel<64, false>, (unsigned)ctas, (unsigned)kAttnThreads,
-                                        (size_t)smem, stream, 1, tq, tk, tv, to, p, none)
-                           : launch_pdl(h, fact_attention_kernel<128, false>, (unsigned)ctas, (unsigned)kAttnThreads,
-                                        (size_t)smem, stream, 1, tq, tk, tv, to, p, none);
+        e = launch_pdl(h, plain[d][pair ? kAttnPair : (one_tile ? kAttnHalf : kAttnRows)], (unsigned)ctas, (unsigned)kAttnThreads,
+                       (size_t)smem, stream, 1, tq, tk, tv, to, p, none);
       if (e != cudaSuccess) st = cuda_fail(h, "attention launch", e);
       else h->launches++;
     }

@@ -128,6 +128,7 @@ struct GemmParams {
   const float* ws;    // the partial planes, for the reduction in the kernel's tail
   int fused_reduce;   // 1: after a grid-wide barrier every CTA reduces its share of the output (split-K only)
   int reduce_epi;     // the epilogue the reduction applies
+  int reduce_lanes_log2;  // lanes that share a group of 4 columns in it
   int* status;        // [0] error word, [2..17] clock / profile counters, [24], [25] grid-barrier counters
   // grouped GEMM (the GROUPED instantiations only): the rows of A and C are cut into `groups` consecutive row
   // groups, group g multiplies W[g]; see decode_grouped.  Up to kParamGroups groups the two tables below are a kernel
@@ -558,8 +559,7 @@ __device__ __forceinline__ void apply_epilogue8(const uint32_t* acc, const uint3
 }
 
 // ---------------------------------------------------------------------------------------------
-// Split-K reduction: adds the S partials of every output element in ascending slice order,
-// applies the epilogue and stores.  One thread per 4 consecutive output columns.  The same routine
+// Split-K reduction: adds the S partials of every output element in a fixed order, applies the epilogue and stores.  The same routine
 // serves the tail of the GEMM kernel (all CTAs, after a grid-wide barrier) and a stand-alone kernel.
 struct ReduceParams {
   const float* ws;  // ws[(split * batch + b) * planes + plane][M][ws_ld]
@@ -575,6 +575,7 @@ struct ReduceParams {
   const __nv_bfloat16* R;
   long long ldr, strideR;
   float alpha;  // the summed accumulator is multiplied by this first (1 unless the operands carry scales)
+  int lanes_log2;  // reduce_groups: lanes that share a group of 4 columns (reduce_lanes_log2)
 };
 
 __device__ __forceinline__ float reduce_epilogue(int epi, float a, float up, float bias, float res) {
@@ -588,23 +589,45 @@ __device__ __forceinline__ float reduce_epilogue(int epi, float a, float up, flo
   }
 }
 
-constexpr int kReduceBatch = 10;  // loads in flight per thread and round trip: 40 slices (the 37 of a 148-SM part in one trip)
-
-// Four adjacent lanes share one group of 4 output columns: lane q of the quad adds slices q, q+4, q+8, ...
-// in ascending order, then the four sums are combined as (s0 + s1) + (s2 + s3).  The order of every
-// addition depends only on the number of slices, so the result is reproducible bit for bit.
+// 2^lanes_log2 adjacent lanes share one group of 4 output columns: lane q of them adds slices q, q + L, q + 2 L, ... in
+// ascending order, then the L sums are combined pairwise -- (s0 + s1), (s2 + s3), ... and so on -- by a butterfly.  The
+// order of every addition depends only on the number of slices and L, so the result is reproducible bit for bit.
+// Every lane keeps up to kReduceBatch loads (of each plane of a gated accumulator) in flight.
 // `first` and `stride` count threads and must be multiples of 32 (whole warps walk the loop together).
+constexpr int kReduceBatch = 10;
+
+// How many lanes share a group, for `threads` threads and `groups` groups of columns: as few passes of the threads over
+// the groups, and as few trips to L2 per pass, as possible.  (Four lanes always: 80 x 128 x 209992, 148 slices, kept 29 of
+// 148 CTAs busy for four trips; sixteen share it out in one: 25.8 -> 24.2 us, 79 x 160 x 83512 18.6 -> 16.6.)  Up to 8 slices
+// four lanes, the association of the wide walk below.
+__host__ __device__ inline int reduce_lanes_log2(long long groups, long long threads, int splits, bool gate) {
+  if (splits <= 8) return 2;
+  int best = 2;
+  long long best_cost = -1;
+  for (int l = 0; l <= 5; ++l) {
+    const long long passes = ((groups << l) + threads - 1) / threads;
+    const int loads = (splits + (1 << l) - 1) >> l;
+    const long long cost = passes * (1200LL * ((loads + kReduceBatch - 1) / kReduceBatch) + 60LL * loads * (gate ? 2 : 1) + 60LL * l);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = l;
+    }
+  }
+  return best;
+}
+
 __device__ __forceinline__ void reduce_groups(const ReduceParams& p, long long first, long long stride) {
+  const bool gate = p.epi == kEpiSiluGate;
+  const int ll = p.lanes_log2, L = 1 << ll;
   const long long groups_per_row = (p.N_out + 3) / 4;
   const long long total = (long long)p.batch * p.M * groups_per_row;
   const long long plane_stride = (long long)p.M * p.ws_ld;
   const long long slice_stride = (long long)p.batch * p.planes * plane_stride;
-  const bool gate = p.epi == kEpiSiluGate;
   const long long warp_first = first & ~31LL;
   const int lane = (int)(first & 31);
-  const int sub = lane & 3;
-  for (long long t0 = warp_first; t0 < total * 4; t0 += stride) {  // uniform trip count within a warp
-    const long long i = (t0 + lane) >> 2;                           // the quad's group
+  const int sub = lane & (L - 1);
+  for (long long t0 = warp_first; t0 < (total << ll); t0 += stride) {  // uniform trip count within a warp
+    const long long i = (t0 + lane) >> ll;                              // these lanes' group
     const bool valid = i < total;
     const long long ii = valid ? i : 0;
     int gcol, m, b;
@@ -625,54 +648,51 @@ __device__ __forceinline__ void reduce_groups(const ReduceParams& p, long long f
     float a[4] = {0.f, 0.f, 0.f, 0.f}, up[4] = {0.f, 0.f, 0.f, 0.f};
     const float* base = p.ws + ((long long)b * p.planes) * plane_stride + (long long)m * p.ws_ld + n;
     if (valid) {
-      for (int s0 = sub; s0 < p.splits; s0 += 4 * kReduceBatch) {  // this lane's slices, a batch of loads at a time
+      for (int s0 = sub; s0 < p.splits; s0 += L * kReduceBatch) {  // this lane's slices, a batch of loads at a time
         float4 v[kReduceBatch], t[kReduceBatch];
 #pragma unroll
-        for (int i8 = 0; i8 < kReduceBatch; ++i8) {
-          const int sl = s0 + 4 * i8;
+        for (int k = 0; k < kReduceBatch; ++k) {
+          const int sl = s0 + L * k;
           if (sl < p.splits) {
             const float* ps = base + (long long)sl * slice_stride;
-            v[i8] = __ldcg(reinterpret_cast<const float4*>(ps));  // ws_ld is a multiple of 4: padding is in bounds
-            if (gate) t[i8] = __ldcg(reinterpret_cast<const float4*>(ps + plane_stride));
+            v[k] = __ldcg(reinterpret_cast<const float4*>(ps));  // ws_ld is a multiple of 4: padding is in bounds
+            if (gate) t[k] = __ldcg(reinterpret_cast<const float4*>(ps + plane_stride));
           }
         }
 #pragma unroll
-        for (int i8 = 0; i8 < kReduceBatch; ++i8) {
-          if (s0 + 4 * i8 < p.splits) {
-            a[0] += v[i8].x; a[1] += v[i8].y; a[2] += v[i8].z; a[3] += v[i8].w;
+        for (int k = 0; k < kReduceBatch; ++k) {
+          if (s0 + L * k < p.splits) {
+            a[0] += v[k].x; a[1] += v[k].y; a[2] += v[k].z; a[3] += v[k].w;
             if (gate) {
-              up[0] += t[i8].x; up[1] += t[i8].y; up[2] += t[i8].z; up[3] += t[i8].w;
+              up[0] += t[k].x; up[1] += t[k].y; up[2] += t[k].z; up[3] += t[k].w;
             }
           }
         }
       }
     }
-    // (s0 + s1) + (s2 + s3): every lane of the quad ends with the same total
+    for (int o = 1; o < L; o <<= 1) {  // every lane of the group ends with the same total
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      a[j] += __shfl_xor_sync(0xffffffffu, a[j], 1);
-      a[j] += __shfl_xor_sync(0xffffffffu, a[j], 2);
-      if (gate) {
-        up[j] += __shfl_xor_sync(0xffffffffu, up[j], 1);
-        up[j] += __shfl_xor_sync(0xffffffffu, up[j], 2);
+      for (int j = 0; j < 4; ++j) {
+        a[j] += __shfl_xor_sync(0xffffffffu, a[j], o);
+        if (gate) up[j] += __shfl_xor_sync(0xffffffffu, up[j], o);
       }
     }
-    // lane `sub` of the quad finishes column n + sub
-    if (valid && sub < nvalid) {
-      const int j = sub;
-      const float av = sub == 0 ? a[0] : sub == 1 ? a[1] : sub == 2 ? a[2] : a[3];
-      const float uv = sub == 0 ? up[0] : sub == 1 ? up[1] : sub == 2 ? up[2] : up[3];
-      const float bias = p.bias ? __bfloat162float(p.bias[n + j]) : 0.f;
-      const float res =
-          (p.epi == kEpiBiasResidual) ? __bfloat162float(p.R[(long long)b * p.strideR + (long long)m * p.ldr + n + j]) : 0.f;
-      const float y = reduce_epilogue(p.epi, av * p.alpha, uv * p.alpha, bias, res);
-      const long long off = (long long)b * p.strideC + (long long)m * p.ldc + n + j;
-      if (p.out_f32) reinterpret_cast<float*>(p.C)[off] = y;
-      else reinterpret_cast<__nv_bfloat16*>(p.C)[off] = __float2bfloat16_rn(y);
+    // lanes 0-3 of the group finish columns n .. n + 3 (or however many lanes there are, several columns each)
+    if (valid) {
+      for (int j = sub; j < nvalid; j += L) {
+        const float av = j == 0 ? a[0] : j == 1 ? a[1] : j == 2 ? a[2] : a[3];
+        const float uv = j == 0 ? up[0] : j == 1 ? up[1] : j == 2 ? up[2] : up[3];
+        const float bias = p.bias ? __bfloat162float(p.bias[n + j]) : 0.f;
+        const float res =
+            (p.epi == kEpiBiasResidual) ? __bfloat162float(p.R[(long long)b * p.strideR + (long long)m * p.ldr + n + j]) : 0.f;
+        const float y = reduce_epilogue(p.epi, av * p.alpha, uv * p.alpha, bias, res);
+        const long long off = (long long)b * p.strideC + (long long)m * p.ldc + n + j;
+        if (p.out_f32) reinterpret_cast<float*>(p.C)[off] = y;
+        else reinterpret_cast<__nv_bfloat16*>(p.C)[off] = __float2bfloat16_rn(y);
+      }
     }
   }
 }
-
 // The same sums for a few slices of a large output: one thread adds every slice of 8 adjacent columns of a row,
 // with all its loads in flight at once, and stores 16 (BF16) or 32 (FP32) bytes.  (The quads above keep one round
 // trip to L2 per 32 outputs of a warp, which a 16384 x 768 output with two slices pays 400 000 times over: 445 us.)
@@ -1850,18 +1870,24 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
       __syncthreads();
       volatile int* arrived = p.status + 24;
       int* leaving = p.status + 25;
+      int left = 0;
       if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(p.status + 24, 1);
-        const unsigned long long t0 = ptx::globaltimer_ns();
-        while (*arrived < (int)gridDim.x) {
-          if (ptx::globaltimer_ns() - t0 > kWaitLimitNs) {  // bounded: give up, flag, skip the reduction
+        unsigned long long t0 = 0;
+        for (uint32_t it = 1; ptx::ld_acquire_gpu(p.status + 24) < (int)gridDim.x; ++it) {
+          if ((it & 63u) != 0) continue;  // (the timer is slow to read: only now and then)
+          const unsigned long long now = ptx::globaltimer_ns();
+          if (t0 == 0) {
+            t0 = now;
+          } else if (now - t0 > kWaitLimitNs) {  // bounded: give up, flag, skip the reduction
             *abort_p = 1;
             atomicExch(p.status, kDeviceTimeoutCode);
             break;
           }
         }
         __threadfence();
+        left = atomicAdd(leaving, 1);  // (this CTA is past the barrier: the answer is looked at after the reduction)
       }
       __syncthreads();
       if (prof && threadIdx.x == 0) reinterpret_cast<long long*>(p.status + 2)[7] = clock64() - t_clk0;
@@ -1884,14 +1910,14 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
         r.ldr = p.ldr;
         r.strideR = p.strideR;
         r.alpha = p.use_alpha ? p.alpha : 1.f;
+        r.lanes_log2 = p.reduce_lanes_log2;
         // (the quads only: the host sends a product of few slices, which the wide walk serves better, to the
         // stand-alone reduction kernel, and this kernel's tail stays short -- cold, every extra line of code on the
         // way to the reduction is a trip to DRAM: 41 against 37 us for the 256 x 256 x 131072 product)
         reduce_groups(r, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
       }
-      __syncthreads();
-      // the last CTA to leave resets both counters for the next launch
-      if (threadIdx.x == 0 && atomicAdd(leaving, 1) == (int)gridDim.x - 1) {
+      // the last CTA past the barrier resets both counters for the next launch
+      if (threadIdx.x == 0 && left == (int)gridDim.x - 1) {
         *arrived = 0;
         *leaving = 0;
         __threadfence();
