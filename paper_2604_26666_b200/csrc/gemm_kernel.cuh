@@ -491,6 +491,15 @@ __device__ __forceinline__ void load_bf16x8(const __nv_bfloat16* ptr, int nvalid
   }
 }
 
+// The same as the BF16 words themselves (to hold many of them while something else is waited for).
+__device__ __forceinline__ uint4 load_bf16x8_raw(const __nv_bfloat16* ptr, int nvalid, bool vec) {
+  if (vec && nvalid >= 8) return __ldg(reinterpret_cast<const uint4*>(ptr));
+  uint32_t h[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) h[j] = (j < nvalid) ? (uint32_t)*reinterpret_cast<const uint16_t*>(ptr + j) : 0u;
+  return make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
@@ -1866,7 +1875,7 @@ __global__ void __launch_bounds__(kThreads + (DYN ? 32 : 0), 1)
     if (p.fused_reduce) {
       // Every CTA's partial stores are complete (the epilogue warps waited for their bulk groups).  A
       // grid-wide barrier -- all CTAs are resident: at most one per SM and never more CTAs than SMs --
-      // then every thread of the grid reduces its share of the output in ascending slice order.
+      // then every thread of the grid reduces its share of the output in a fixed order of the slices.
       __syncthreads();
       volatile int* arrived = p.status + 24;
       int* leaving = p.status + 25;
