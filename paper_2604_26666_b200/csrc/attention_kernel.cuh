@@ -55,7 +55,11 @@ struct AttnParams {
   int causal;
   float scale_log2;           // softmax scale * log2(e)
   int q_pairs;                // ceil(Tq / 256)
-  int items;                  // B * Hq * q_pairs work items, ordered heaviest first
+  int q_tiles;                // ceil(Tq / 128) (independent tiles, like the four below)
+  int items;                  // work items, ordered heaviest first
+  __nv_bfloat16* O;           // rows are stored from registers: batch, token and head strides in elements
+  long long o_sb, o_st, o_sh;
+  int o_vec32;                // rows of O start on 32 bytes
   uint64_t kmajor_desc;       // UMMA descriptor template, K-major 128B-swizzled tiles (Q, K)
   uint64_t v_desc;            // UMMA descriptor template, V as an N-major operand
   uint32_t idesc_s, idesc_pv;

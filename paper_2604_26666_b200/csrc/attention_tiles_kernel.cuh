@@ -1,0 +1,435 @@
+// Fused multi-head attention forward at head_dim 64 for sm_100a: independent query tiles, three or two per CTA.
+//
+// What bounds this head size is the softmax: an SM partition takes four exponentials a cycle, 1024 cycles for the 32 x 128
+// scores a warp has of a 128-key block, twice what the two products take.  attention_kernel.cuh works on 256 query rows of a
+// head at a time, as two tiles that share the key blocks; a causal problem then wastes the blocks that only the second of
+// them sees, a ragged one up to 255 rows, and a small one half of the SMs.  Here a tile of 128 rows is a pipeline of its own
+// with its own list of items, its own query buffer and key and value rings: one warp that issues its loads and its
+// products, and a warpgroup with one thread per query row.  Nothing is shared between a CTA's pipelines, so they fill each
+// other's gaps.  Two shapes:
+//   three tiles, blocks of 64 keys (480 of the 512 tensor-memory columns: 32 of probabilities, 64 of scores and 64 of
+//   output each): three softmax warps per SM partition hide more of each other's latencies (score loads, maxima, hand-overs),
+//   and half of a causal tile's warps have nothing to do in its last block;
+//   two tiles, blocks of 128 keys: half the hand-overs per key, for problems too small to have three tiles on every SM.
+// Causal, 12 heads, microseconds, pairs -> this kernel: 16 x 1000 53.4 -> 45.5, 128 x 512 128 -> 113, 40 x 384 42.1 -> 27.6,
+// 16 x 300 19.9 -> 12.7, 8 x 4096 285 -> 266; two tiles: 1 x 1500 23.0 -> 17.5.  Which call takes what is in
+// attention_tiles_choice (fact_api.cu).  What is left: 12 of 16 exponentials a cycle and SM within a block; about 2500
+// cycles per tile for its last product and its output, under which only the other pipelines run.
+// Tried and slower: two tiles in blocks of 64 keys with scores and probabilities double-buffered and the next block's
+// scores loaded under the exponentials (16 x 1024 full 99 us against 85, the loop is no longer one straight block).
+//
+// Per block j (online softmax with a reference maximum that moves only when a block exceeds it by more than 8, as in
+// attention_kernel.cuh):
+//   issuer    S(j + 1) = Q K^T as soon as S(j) has been read; the slot of K(j) is then known to be free (S(j) is complete),
+//             so the next key block is loaded into it; O += P(j) V(j) when P(j) has been stored -- which the softmax threads
+//             do only after O += P(j - 1) V(j - 1), so the next value block is loaded into the slot of V(j - 1): the rings
+//             need no "empty" barriers
+//   softmax   scores to registers, mask, maximum, exponentials, row sum, probabilities to tensor memory; after the last
+//             block O / l straight to global memory, 128 contiguous bytes a row
+// Every barrier has one event per block (or per item) that its waiter waits for every time, and whose next event needs the
+// waiter's own next step, so a one-bit phase is enough.  Every wait is bounded, as in the GEMM kernel.
+#pragma once
+#include "attention_kernel.cuh"
+
+namespace fact {
+
+// The two shapes: three tiles in blocks of 64 keys, two in blocks of 128.
+template <int TILES>
+struct AttnTiles {
+  static_assert(TILES == 2 || TILES == 3, "");
+  static constexpr int kThreads = 128 * TILES + 128;  // softmax warpgroups, then a warpgroup of issuers (the rest of it idle)
+  static constexpr int kBlockK = TILES == 3 ? 64 : 128;
+  static constexpr int kKStages = TILES == 3 ? 4 : 3, kVStages = 3;
+  static constexpr uint32_t kTileBytes = kAttnChunkBytes;   // 128 query rows
+  static constexpr uint32_t kKvBytes = kBlockK * 128u;      // a block of keys or values
+  static constexpr uint32_t kPipeBytes = kTileBytes + (kKStages + kVStages) * kKvBytes;
+  static constexpr uint32_t kCols = kBlockK / 2 + kBlockK + 64;  // tensor-memory columns of a pipeline: P, S, O
+  static_assert(kCols * TILES <= 512 && kCols % 32 == 0, "tensor memory");
+  // Registers per thread after the warpgroups rebalance; the host checks kRegsAtLaunch before the first launch.
+  static constexpr int kRegsSoftmax = TILES == 3 ? 144 : 208, kRegsOther = 80, kRegsAtLaunch = TILES == 3 ? 128 : 168;
+  static_assert(4 * TILES * kRegsSoftmax + 4 * kRegsOther <= kThreads / 32 * kRegsAtLaunch, "setmaxnreg requests exceed the pool");
+  // barriers of a pipeline
+  static constexpr int kQFull = 0;  // the tile's Q has landed
+  static constexpr int kSFull = 1;  // a block's scores are complete
+  static constexpr int kSRead = 2;  // the four softmax warps hold them in registers
+  static constexpr int kPFull = 3;  // the four softmax warps have stored the block's probabilities
+  static constexpr int kPvDone = 4; // a block's second product has completed
+  static constexpr int kOFree = 5;  // the softmax warps have read the finished O
+  static constexpr int kKFull = 6, kVFull = kKFull + kKStages, kBars = kVFull + kVStages;
+  static constexpr uint32_t kSmemBytes = TILES * (kPipeBytes + kBars * 8u) + 16u;
+};
+
+// Which items a pipeline works through (see AttnDeal): pipeline t of CTA c is worker t * CTAs + c.
+struct AttnTilesDeal {
+  uint16_t off[3 * kAttnDealCtas + 1];
+  uint16_t list[kAttnDealItems];
+};
+template <bool DEAL>
+struct AttnTilesDealArg {
+  using type = AttnNoDeal;
+};
+template <>
+struct AttnTilesDealArg<true> {
+  using type = AttnTilesDeal;
+};
+
+struct AttnTile {
+  int b, h, kvh, t0;
+  int nb;  // key blocks the tile sees
+};
+
+template <int TILES, bool DEAL>
+__global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
+    fact_attention_tiles_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                                const __grid_constant__ CUtensorMap tmV, const AttnParams p,
+                                const __grid_constant__ typename AttnTilesDealArg<DEAL>::type deal) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31;
+  const uint32_t smem_base = ptx::smem_u32(smem_raw);
+  if (smem_base & 1023u) {
+    if (threadIdx.x == 0) atomicExch(p.status, kDeviceTimeoutCode);
+    return;
+  }
+  using L = AttnTiles<TILES>;
+  constexpr int BK = L::kBlockK;
+  constexpr uint32_t ctrl_off = TILES * (L::kPipeBytes + L::kBars * 8u);
+  volatile uint32_t* tmem_holder_p = reinterpret_cast<volatile uint32_t*>(smem_raw + ctrl_off);
+  volatile int* abort_p = reinterpret_cast<volatile int*>(smem_raw + ctrl_off + 4);
+  const int t = warp < 4 * TILES ? warp >> 2 : warp - 4 * TILES;  // the pipeline this warp serves (TILES on: none)
+  const uint32_t bar_base = smem_base + TILES * L::kPipeBytes + (uint32_t)t * (L::kBars * 8u);
+  auto bar = [&](int i) { return bar_base + 8u * (uint32_t)i; };
+
+  if (threadIdx.x < TILES * L::kBars) {
+    const int i = (int)threadIdx.x % L::kBars;
+    const bool by_warps = i == L::kSRead || i == L::kPFull || i == L::kOFree;  // one arrival per softmax warp
+    ptx::mbar_init(smem_base + TILES * L::kPipeBytes + 8u * threadIdx.x, by_warps ? 4 : 1);
+    if (threadIdx.x == 0) *abort_p = 0;
+    ptx::fence_mbar_init();
+  }
+  if (warp == 4 * TILES) {
+    if (lane == 0) {
+      ptx::prefetch_tensormap(&tmQ);
+      ptx::prefetch_tensormap(&tmK);
+      ptx::prefetch_tensormap(&tmV);
+    }
+    __syncwarp();
+    ptx::tmem_alloc<1>(smem_base + ctrl_off, 512);
+    ptx::tmem_relinquish<1>();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = *tmem_holder_p;
+  // the set-up above may overlap the tail of the previous kernel in the stream; global memory only from here on
+  ptx::grid_dependency_wait();
+
+  // Items are numbered with the query position as the slow index, heaviest first (the late rows of a causal problem), and
+  // dealt to the pipelines round by round, every second round in the opposite direction, or by the host's list.
+  const int G = (int)gridDim.x, W = TILES * G;
+  const int worker = t * G + (int)blockIdx.x;
+  const int full_rounds = p.items / W, tail = p.items - full_rounds * W;
+  auto pos_in_round = [&](int n) { return (n & 1) ? W - 1 - worker : worker; };
+  int n_items = 0, deal_first = 0;
+  if (t < TILES) {
+    if constexpr (DEAL) {
+      deal_first = deal.off[worker];
+      n_items = (int)deal.off[worker + 1] - deal_first;
+    } else {
+      n_items = full_rounds + (pos_in_round(full_rounds) < tail ? 1 : 0);
+    }
+  }
+  const int kv_blocks_all = (p.Tk + BK - 1) / BK;
+  const int bh_count = p.B * p.Hq;
+  auto item_of = [&](int n) -> AttnTile {
+    int idx = n * W + pos_in_round(n);
+    if constexpr (DEAL) idx = deal.list[deal_first + n];
+    const int qr = idx / bh_count;
+    const int bh = idx - qr * bh_count;
+    AttnTile it;
+    it.h = bh % p.Hq;
+    it.b = bh / p.Hq;
+    it.kvh = it.h / (p.Hq / p.Hkv);
+    it.t0 = (p.causal ? (p.q_tiles - 1 - qr) : qr) * kAttnBlockQ;
+    // causal: a tile whose last row is r sees keys 0 .. r
+    it.nb = p.causal ? min(kv_blocks_all, (it.t0 + kAttnBlockQ - 1) / BK + 1) : kv_blocks_all;
+    return it;
+  };
+  auto wait_all = [&](uint32_t br, uint32_t parity) -> bool {
+    if (__all_sync(0xffffffffu, ptx::mbar_try_wait(br, parity))) return true;
+    return __all_sync(0xffffffffu, wait_bar(br, parity, abort_p, p.status)) != 0;
+  };
+  const uint32_t q_s = smem_base + (uint32_t)t * L::kPipeBytes;
+  const uint32_t k_s = q_s + L::kTileBytes;
+  const uint32_t v_s = k_s + L::kKStages * L::kKvBytes;
+  const uint32_t tmem_p = tmem_base + (uint32_t)t * L::kCols;
+  const uint32_t tmem_s = tmem_p + BK / 2;
+  const uint32_t tmem_o = tmem_s + BK;
+
+  if (warp >= 4 * TILES) {
+    ptx::setmaxnreg_dec<L::kRegsOther>();
+    if (t < TILES && n_items > 0) {
+      // ------------------------------------------------------------ loads and products of pipeline t
+      const uint64_t keep = ptx::l2_policy(2);  // keys and values are read again by every query tile of their head
+      struct Cursor {  // the next block to load
+        int n, j, slot;
+        AttnTile it;
+      };
+      Cursor kc{0, 0, 0, item_of(0)}, vc{0, 0, 0, kc.it};
+      auto load_kv = [&](Cursor& c, const CUtensorMap* map, uint32_t ring, int full, int stages) {
+        if (c.n >= n_items) return;
+        if (ptx::elect_one()) {
+          ptx::mbar_arrive_expect_tx(bar(full + c.slot), L::kKvBytes);
+          ptx::tma_load_4d_hint(ring + (uint32_t)c.slot * L::kKvBytes, map, bar(full + c.slot), 0, c.it.kvh, c.j * BK, c.it.b, keep);
+        }
+        __syncwarp();
+        if (++c.slot == stages) c.slot = 0;
+        if (++c.j == c.it.nb) {
+          c.j = 0;
+          if (++c.n < n_items) c.it = item_of(c.n);
+        }
+      };
+      auto load_q = [&](const AttnTile& it) {
+        if (ptx::elect_one()) {
+          ptx::mbar_arrive_expect_tx(bar(L::kQFull), L::kTileBytes);
+          ptx::tma_load_4d(q_s, &tmQ, bar(L::kQFull), 0, it.h, it.t0, it.b);
+        }
+        __syncwarp();
+      };
+      AttnTile it = kc.it;
+      load_q(it);
+#pragma unroll 1
+      for (int i = 0; i < L::kKStages; ++i) {
+        load_kv(kc, &tmK, k_s, L::kKFull, L::kKStages);
+        if (i < L::kVStages) load_kv(vc, &tmV, v_s, L::kVFull, L::kVStages);
+      }
+      const uint64_t qdesc0 = p.kmajor_desc | (uint64_t)((q_s >> 4) & 0x3fffu);
+      int ks = 0, vs = 0;         // ring slots of the next first and second product
+      uint32_t kpar = 0, vpar = 0;
+      bool ok = true;
+      auto issue_s = [&]() -> bool {
+        if (!wait_all(bar(L::kKFull + ks), kpar)) return false;
+        ptx::tc_fence_after();
+        if (ptx::elect_one()) {
+          const uint64_t kdesc0 = p.kmajor_desc | (uint64_t)(((k_s + (uint32_t)ks * L::kKvBytes) >> 4) & 0x3fffu);
+#pragma unroll
+          for (int kk = 0; kk < 64 / kUmmaK; ++kk)  // 16 elements of head_dim = 32 bytes of a row
+            ptx::umma_bf16<1>(tmem_s, qdesc0 + (uint64_t)(kk * 2), kdesc0 + (uint64_t)(kk * 2), p.idesc_s, kk > 0 ? 1u : 0u);
+          ptx::umma_commit<1>(bar(L::kSFull));
+        }
+        __syncwarp();
+        if (++ks == L::kKStages) {
+          ks = 0;
+          kpar ^= 1u;
+        }
+        return true;
+      };
+      int gt = 0;  // blocks so far
+      for (int n = 0; ok && n < n_items; ++n) {
+        const int nb = it.nb;
+        ok = wait_all(bar(L::kQFull), (uint32_t)n & 1u);
+        if (ok) ok = issue_s();
+        for (int j = 0; ok && j < nb; ++j, ++gt) {
+          ok = wait_all(bar(L::kSRead), (uint32_t)gt & 1u);
+          if (!ok) break;
+          if (j + 1 < nb) {
+            ok = issue_s();
+            if (!ok) break;
+          } else if (n + 1 < n_items) {  // the tile's last scores are complete: Q is free
+            it = item_of(n + 1);
+            load_q(it);
+          }
+          load_kv(kc, &tmK, k_s, L::kKFull, L::kKStages);  // ... into the slot of the block whose scores have been read
+          ok = wait_all(bar(L::kPFull), (uint32_t)gt & 1u);
+          // the first block of an item overwrites O: the previous item's must have been read
+          if (ok && j == 0 && n > 0) ok = wait_all(bar(L::kOFree), (uint32_t)(n - 1) & 1u);
+          if (ok) ok = wait_all(bar(L::kVFull + vs), vpar);
+          if (!ok) break;
+          ptx::tc_fence_after();
+          if (ptx::elect_one()) {
+            const uint64_t vdesc0 = p.v_desc | (uint64_t)(((v_s + (uint32_t)vs * L::kKvBytes) >> 4) & 0x3fffu);
+#pragma unroll
+            for (int kk = 0; kk < BK / kUmmaK; ++kk)  // 16 keys = 2048 bytes further on in V, 8 columns in P
+              ptx::umma_bf16_ts(tmem_o, tmem_p + (uint32_t)kk * 8u, vdesc0 + (uint64_t)(kk * 128), p.idesc_pv,
+                                (j > 0 || kk > 0) ? 1u : 0u);
+            ptx::umma_commit<1>(bar(L::kPvDone));
+          }
+          __syncwarp();
+          if (++vs == L::kVStages) {
+            vs = 0;
+            vpar ^= 1u;
+          }
+          // the probabilities were stored after the second product of the block before: its V slot is free
+          if (gt > 0) load_kv(vc, &tmV, v_s, L::kVFull, L::kVStages);
+        }
+      }
+      __syncwarp();
+    }
+  } else {
+    ptx::setmaxnreg_inc<L::kRegsSoftmax>();
+    // ------------------------------------------------------------ softmax warps: one thread per query row
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
+    const uint32_t p_addr = tmem_p + lane_addr, s_addr = tmem_s + lane_addr, o_addr = tmem_o + lane_addr;
+    const uint64_t scale2 = ptx::pack_f32x2(__float_as_uint(p.scale_log2), __float_as_uint(p.scale_log2));
+    bool ok = true;  // warp-uniform
+    int gt = 0;
+    for (int n = 0; ok && n < n_items; ++n) {
+      const AttnTile it = item_of(n);
+      const int t_row = it.t0 + row;
+      const int visible = min(p.Tk, p.causal ? t_row + 1 : p.Tk);  // keys this row sees
+      // blocks of which every row of this warp sees every key, and blocks any of its rows sees
+      const int first_row = it.t0 + (warp & 3) * 32;
+      const int full_blocks = min(p.Tk, p.causal ? first_row + 1 : p.Tk) / BK;
+      const int some_blocks = p.causal ? (first_row + 31) / BK + 1 : it.nb;
+      float m = -INFINITY;  // reference maximum of scale_log2 * score the exponentials are taken against
+      float l = 0.f;        // running sum of 2^(scale_log2 * score - m)
+      for (int j = 0; ok && j < it.nb; ++j, ++gt) {
+        ok = wait_all(bar(L::kSFull), (uint32_t)gt & 1u);
+        if (!ok) break;
+        const int key_limit = visible - j * BK;
+        uint32_t pw[BK / 2];
+        bool pv_waited = gt == 0;  // whether O += P(j-1) V(j-1) has completed (or there is none)
+        if (j >= some_blocks) {
+          // beyond the diagonal of all 32 rows: nothing to read and no exponentials, the probabilities are zero
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(bar(L::kSRead));
+#pragma unroll
+          for (int i = 0; i < BK / 2; ++i) pw[i] = 0u;
+        } else {
+          ptx::tc_fence_after();
+          uint32_t s64[BK / 64][64];
+#pragma unroll
+          for (int c = 0; c < BK / 64; ++c) ptx::tmem_ld_32x32b_x64(s_addr + (uint32_t)c * 64u, s64[c]);
+          uint32_t (&s)[BK] = *reinterpret_cast<uint32_t (*)[BK]>(&s64[0][0]);
+          ptx::tmem_wait_ld();
+          // the scores are in registers: the next block's may overwrite them
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(bar(L::kSRead));
+          // Only the block on the diagonal (or the ragged last one) needs the per-key mask.
+          if (j >= full_blocks) {
+#pragma unroll
+            for (int i = 0; i < BK; ++i)
+              if (i >= key_limit) s[i] = 0xff800000u;  // -inf
+          }
+          // four independent chains of three-input maxima
+          float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+          for (int i = 0; i < BK; i += 2)
+            mx4[(i >> 1) & 3] = ptx::max3(mx4[(i >> 1) & 3], __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
+          const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * p.scale_log2;  // scale > 0
+          // Move the reference maximum only when this block exceeds it by more than the threshold (always from -inf).
+          if (__any_sync(0xffffffffu, mx > m + kAttnRescaleThreshold)) {
+            const float m_new = fmaxf(m, mx);
+            const float alpha = ptx::ex2_approx(m - ((m_new == -INFINITY) ? 0.f : m_new));
+            l *= alpha;
+            m = m_new;
+            if (j > 0) {
+              // O is rescaled between O += P(j-1) V(j-1), which must have completed, and O += P(j) V(j), which waits for
+              // the probabilities announced below
+              ok = wait_all(bar(L::kPvDone), (uint32_t)(gt - 1) & 1u);
+              if (!ok) break;
+              pv_waited = true;
+              ptx::tc_fence_after();
+#pragma unroll 1
+              for (int c = 0; c < 64; c += 32) {
+                uint32_t o[32];
+                ptx::tmem_ld_32x32b_x32(o_addr + (uint32_t)c, o);
+                ptx::tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                ptx::tmem_st_32x32b_x32(o_addr + (uint32_t)c, o);
+              }
+            }
+          }
+          const float m_use = (m == -INFINITY) ? 0.f : m;  // a row with nothing visible yet
+          // 2^(scale_log2 * s - m) on pairs of keys with packed FP32 arithmetic; kAttnPolyOf8 of every eight pairs take
+          // the exponential on the FMA pipe (attn_exp2_poly), the others on the special-function unit
+          const uint64_t negm2 = ptx::pack_f32x2(__float_as_uint(-m_use), __float_as_uint(-m_use));
+          uint64_t sum2[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+          for (int pr = 0; pr < BK / 2; ++pr) {
+            const uint64_t x2 = ptx::fma_f32x2(ptx::pack_f32x2(s[2 * pr], s[2 * pr + 1]), scale2, negm2);
+            uint64_t p2;
+            if ((pr & 7) < kAttnPolyOf8) {
+              p2 = attn_exp2_poly(x2);
+            } else {
+              uint32_t x0, x1;
+              ptx::unpack_f32x2(x2, x0, x1);
+              p2 = ptx::pack_f32x2(__float_as_uint(ptx::ex2_approx(__uint_as_float(x0))),
+                                   __float_as_uint(ptx::ex2_approx(__uint_as_float(x1))));
+            }
+            sum2[pr & 3] = ptx::add_f32x2(sum2[pr & 3], p2);
+            uint32_t p0, p1;
+            ptx::unpack_f32x2(p2, p0, p1);
+            pw[pr] = pack_bf16x2(__uint_as_float(p0), __uint_as_float(p1));
+          }
+          const uint64_t st = ptx::add_f32x2(ptx::add_f32x2(sum2[0], sum2[1]), ptx::add_f32x2(sum2[2], sum2[3]));
+          uint32_t lo, hi;
+          ptx::unpack_f32x2(st, lo, hi);
+          l += __uint_as_float(lo) + __uint_as_float(hi);
+        }
+        // the probabilities of the block before must have been consumed before these overwrite them
+        if (!pv_waited) {
+          ok = wait_all(bar(L::kPvDone), (uint32_t)(gt - 1) & 1u);
+          if (!ok) break;
+          ptx::tc_fence_after();
+        }
+        // lane = row, column c holds keys 2c and 2c + 1
+        if constexpr (BK == 128) ptx::tmem_st_32x32b_x64(p_addr, pw);
+        else ptx::tmem_st_32x32b_x32(p_addr, pw);
+        ptx::tmem_wait_st();
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(bar(L::kPFull));
+      }
+      if (!ok) break;
+      // ---- the tile's output: a thread's row, 128 contiguous bytes
+      ok = wait_all(bar(L::kPvDone), (uint32_t)(gt - 1) & 1u);  // the tile's last product
+      if (!ok) break;
+      ptx::tc_fence_after();
+      uint32_t o[2][32];
+      ptx::tmem_ld_32x32b_x32(o_addr, o[0]);
+      ptx::tmem_ld_32x32b_x32(o_addr + 32u, o[1]);
+      ptx::tmem_wait_ld();
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(bar(L::kOFree));
+      if (t_row < p.Tq) {
+        const float inv = (l > 0.f) ? __fdividef(1.f, l) : 0.f;
+        __nv_bfloat16* dst = p.O + (long long)it.b * p.o_sb + (long long)t_row * p.o_st + (long long)it.h * p.o_sh;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t w[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            w[i] = pack_bf16x2(__uint_as_float(o[c >> 1][(c & 1) * 16 + 2 * i]) * inv,
+                               __uint_as_float(o[c >> 1][(c & 1) * 16 + 2 * i + 1]) * inv);
+          if (p.o_vec32) {
+            ptx::st_global_v8(dst + 16 * c, w);
+          } else {
+            *reinterpret_cast<uint4*>(dst + 16 * c) = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4*>(dst + 16 * c + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+          }
+        }
+      }
+    }
+  }
+
+  // ------------------------------------------------------------ teardown
+  ptx::grid_launch_dependents();  // this CTA's items are done: the next kernel of the stream may move in behind it
+  if (*abort_p) {
+    const unsigned long long tw = ptx::globaltimer_ns();
+    while (ptx::globaltimer_ns() - tw < 200000ull) {
+    }
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 4 * TILES) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc<1>(tmem_base, 512);
+  }
+}
+
+}  // namespace fact

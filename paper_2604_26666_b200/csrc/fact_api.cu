@@ -27,6 +27,7 @@
 #include "skinny_kernel.cuh"
 #include "attention_kernel.cuh"
 #include "attention_decode_kernel.cuh"
+#include "attention_tiles_kernel.cuh"
 #include "norm_kernel.cuh"
 #include "tune_kernels.cuh"
 
@@ -140,6 +141,8 @@ struct fact_handle_s {
   std::bitset<192> configured_mask;  // kernels whose dynamic shared-memory limit was raised
   std::unique_ptr<AttnDeal> attn_deal;         // the host's deal of the last causal attention shape (see fact_attention)
   std::array<long long, 6> attn_deal_key{};
+  std::unique_ptr<AttnTilesDeal> attn_tiles_deal;  // the same at head_dim 64
+  std::array<long long, 4> attn_tiles_deal_key{};
   int kc_clusters[6] = {0, 0, 0, 0, 0, 0};  // clusters of 2 / 4 / 8 CTAs of the K-slice kernel (single CTAs, pairs) the
                                             // device holds at once
   std::string last_error;        // text of the most recent CUDA failure
@@ -1354,6 +1357,104 @@ void build_attention_deal(int G, long long bh, int q_pairs, int bk, long long se
   d.off[G] = (uint16_t)pos;
 }
 
+// The same for the kernel of independent tiles (attention_tiles_kernel.cuh), whose items are tiles of 128 rows: each to the
+// CTA with the least so far, and there to the pipeline with the least.
+void build_attention_tiles_deal(int G, int pipes, int bk, long long bh, int q_tiles, AttnTilesDeal& d) {
+  const int items = (int)(bh * q_tiles);
+  std::vector<std::vector<uint16_t>> mine((size_t)G * pipes);
+  std::vector<int> load((size_t)G * pipes, 0);
+  using Slot = std::pair<int, int>;  // (load, CTA)
+  std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
+  for (int c = 0; c < G; ++c) heap.push({0, c});
+  for (int idx = 0; idx < items; ++idx) {
+    const int qt = q_tiles - 1 - (int)(idx / bh);
+    const int w = (qt * kAttnBlockQ + kAttnBlockQ - 1) / bk + 1 + 64 / bk;
+    const Slot s = heap.top();
+    heap.pop();
+    heap.push({s.first + w, s.second});
+    int best = s.second;
+    for (int t = 1; t < pipes; ++t)
+      if (load[(size_t)(t * G + s.second)] < load[(size_t)best]) best = t * G + s.second;
+    load[(size_t)best] += w;
+    mine[(size_t)best].push_back((uint16_t)idx);
+  }
+  int pos = 0;
+  for (int c = 0; c < G * pipes; ++c) {
+    d.off[c] = (uint16_t)pos;
+    for (uint16_t v : mine[(size_t)c]) d.list[pos++] = v;
+  }
+  d.off[G * pipes] = (uint16_t)pos;
+}
+
+// Which kernel an attention call at head_dim 64 takes: 3 or 2 independent tiles of 128 rows per SM
+// (attention_tiles_kernel.cuh), or 0, tiles in pairs that share their keys (attention_kernel.cuh).  Microseconds measured
+// as pairs / two / three (12 heads):
+//  - sequences of one tile: two while every head has an SM (4 x 100 6.1 / 5.3 / 6.7); three where one block of 64 keys is
+//    all there is, which the blocks of 128 compute twice over (256 x 64 36.4 / 43.3 / 29.4); pairs else (64 x 128 full
+//    13.6 / 14.9 / 15.6).
+//  - causal: a pair's first tile waits out the blocks that only its second sees.  Three from one and a half tiles an SM on
+//    for short sequences and three for long (16 x 1000 53.4 / 53.4 / 45.5, 128 x 512 128 / 133 / 113, 10 x 256 8.4 / 7.5 /
+//    7.2), two below that, where a tile is mostly alone on its SM and blocks of 128 keys get it done sooner (1 x 4096
+//    55.6 / 48.8 / 53.7, 1 x 1500 23.0 / 17.5 / 21.0).
+//  - full: pairs load their keys once for two tiles and are the best where both are busy (16 x 1024 81.9 / 87.1 / 85.4, 128
+//    x 512 151 / 186 / 189); tiles where items of 256 rows leave a sixth of the SMs' time or more empty (1 x 1000 18.4 /
+//    13.5 / 15.9, 40 x 384 45.0 / 38.3 / 41.3, 16 x 300 22.5 / 17.8 / 17.4; three a SM exactly: 1 x 4096 104 / 95.6 / 81.2).
+int attention_tiles_choice(long long q_tiles, long long bh, long long seq_kv, bool causal, long long sms) {
+  const long long items = q_tiles * bh;
+  if (items > 0x7fffffffLL) return 0;
+  if (q_tiles == 1) return items <= sms ? 2 : (seq_kv <= AttnTiles<3>::kBlockK ? 3 : 0);
+  if (causal) return items >= 3 * sms || (q_tiles <= 4 && 2 * items >= 3 * sms) ? 3 : 2;
+  const long long tiles_each = (items + sms - 1) / sms;
+  const long long as_pairs = 2 * (((q_tiles + 1) / 2 * bh + sms - 1) / sms);
+  if (5 * as_pairs < 6 * tiles_each) return 0;
+  return tiles_each == 3 ? 3 : 2;
+}
+
+// Attention at head_dim 64 by independent tiles (attention_tiles_kernel.cuh), items = (batch, head, 128 query rows).
+template <int TILES>
+fact_status_t attention_tiles(fact_handle_t h, AttnParams p, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                              cudaStream_t stream) {
+  using L = AttnTiles<TILES>;
+  const auto plain = fact_attention_tiles_kernel<TILES, false>;
+  const auto dealt = fact_attention_tiles_kernel<TILES, true>;
+  const int smem = std::max((int)L::kSmemBytes, kMinSmemRequest);
+  const size_t bit = TILES == 3 ? 29 : 28;
+  if (!h->configured_mask.test(bit)) {
+    for (const void* kern : {reinterpret_cast<const void*>(plain), reinterpret_cast<const void*>(dealt)}) {
+      cudaFuncAttributes fa;
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+      if (e != cudaSuccess) return cuda_fail(h, "cudaFuncSetAttribute(attention)", e);
+      if (fa.numRegs < L::kRegsAtLaunch) {  // (the register rebalancing would wait forever for registers it does not own)
+        h->last_error = "attention kernel compiled with " + std::to_string(fa.numRegs) + " registers per thread, needs " +
+                        std::to_string(L::kRegsAtLaunch);
+        return FACT_ERR_UNSUPPORTED;
+      }
+    }
+    h->configured_mask.set(bit);
+  }
+  const int ctas = (int)std::min<long long>(p.items, h->sm_count);
+  // Problems of few rounds are dealt out by the host, as in the kernel of paired tiles.
+  const bool deal = p.causal && p.q_tiles > 1 && p.items > ctas && p.items <= kAttnDealItems && ctas <= kAttnDealCtas &&
+                    p.items < 16LL * TILES * ctas;
+  cudaError_t e;
+  if (deal) {
+    const std::array<long long, 4> key = {(long long)p.B * p.Hq, p.q_tiles, TILES, ctas};
+    if (!h->attn_tiles_deal || h->attn_tiles_deal_key != key) {
+      if (!h->attn_tiles_deal) h->attn_tiles_deal.reset(new AttnTilesDeal());
+      build_attention_tiles_deal(ctas, TILES, L::kBlockK, (long long)p.B * p.Hq, p.q_tiles, *h->attn_tiles_deal);
+      h->attn_tiles_deal_key = key;
+    }
+    e = launch_pdl(h, dealt, (unsigned)ctas, (unsigned)L::kThreads, (size_t)smem, stream, 1, tq, tk, tv, p, *h->attn_tiles_deal);
+  } else {
+    const AttnNoDeal none = {0};
+    e = launch_pdl(h, plain, (unsigned)ctas, (unsigned)L::kThreads, (size_t)smem, stream, 1, tq, tk, tv, p, none);
+  }
+  if (e != cudaSuccess) return cuda_fail(h, "attention launch", e);
+  h->launches++;
+  return FACT_OK;
+}
+
 Problem make_problem(fact_op_t op, long long batch, long long M, long long N, long long K, const void* A,
                      long long lda, long long sA, const void* B, long long ldb, long long sB, fact_blayout_t layout,
                      const void* bias, const void* R, long long ldr, long long sR, void* C, long long ldc,
@@ -2349,14 +2450,18 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
   }
   CUtensorMap tq, tk, tv, to;
   auto bs = [&](int64_t s, int64_t fallback) { return (batch > 1 && s > 0) ? s : std::max<int64_t>(fallback, 8); };
-  // keys go in blocks of 128 at head_dim 64 and of 64 at head_dim 128 (the kernel's tensor-memory budget)
-  const int block_k = attn_block_k((int)head_dim);
+  const long long q_tiles = (seq_q + kAttnBlockQ - 1) / kAttnBlockQ;
+  const long long tile_items = q_tiles * heads_q * batch;
+  const int tiles = head_dim == 64 ? attention_tiles_choice(q_tiles, heads_q * batch, seq_kv, causal != 0, h->sm_count) : 0;
+  // keys go in blocks of 128 or 64, as the kernels' tensor-memory budgets have it
+  const int block_k = tiles == 3 ? AttnTiles<3>::kBlockK : (tiles == 2 ? AttnTiles<2>::kBlockK : attn_block_k((int)head_dim));
   fact_status_t st = encode_map_bthd(h, &tq, Q, head_dim, heads_q, seq_q, batch, q_sh, q_st, bs(q_sb, q_st * seq_q));
   if (st == FACT_OK)
     st = encode_map_bthd(h, &tk, K, head_dim, heads_kv, seq_kv, batch, k_sh, k_st, bs(k_sb, k_st * seq_kv), block_k);
   if (st == FACT_OK)
     st = encode_map_bthd(h, &tv, V, head_dim, heads_kv, seq_kv, batch, v_sh, v_st, bs(v_sb, v_st * seq_kv), block_k);
-  if (st == FACT_OK) st = encode_map_bthd(h, &to, O, head_dim, heads_q, seq_q, batch, o_sh, o_st, bs(o_sb, o_st * seq_q));
+  if (st == FACT_OK && tiles == 0)
+    st = encode_map_bthd(h, &to, O, head_dim, heads_q, seq_q, batch, o_sh, o_st, bs(o_sb, o_st * seq_q));
   if (st == FACT_OK) {
     AttnParams p;
     memset(&p, 0, sizeof p);
@@ -2376,6 +2481,18 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
                  ((uint32_t)(kAttnBlockQ >> 4) << 24);
     p.status = h->d_status;
     p.debug = h->debug_flags;
+    if (tiles != 0) {
+      p.q_tiles = (int)q_tiles;
+      p.items = (int)tile_items;
+      p.O = static_cast<__nv_bfloat16*>(O);
+      p.o_sb = bs(o_sb, o_st * seq_q);
+      p.o_st = o_st;
+      p.o_sh = o_sh;
+      p.o_vec32 = (reinterpret_cast<uintptr_t>(O) & 31u) == 0 && p.o_sb % 16 == 0 && o_st % 16 == 0 && o_sh % 16 == 0;
+      st = tiles == 3 ? attention_tiles<3>(h, p, tq, tk, tv, stream) : attention_tiles<2>(h, p, tq, tk, tv, stream);
+      if (dev != h->device) cudaSetDevice(dev);
+      return st;
+    }
     p.q_pairs = (int)((seq_q + 2 * kAttnBlockQ - 1) / (2 * kAttnBlockQ));  // an item is two tiles of 128 query rows
     // ... or, for sequences that fit one tile, two heads' tiles once there are more heads than SMs, one head's before that
     const bool one_tile = seq_q <= kAttnBlockQ;
@@ -2390,11 +2507,11 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     const int smem = std::max((int)attn_smem_bytes(p.D), kMinSmemRequest);
     typedef void (*Plain)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams, AttnNoDeal);
     typedef void (*Dealt)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams, AttnDeal);
-    static const Plain plain[2][3] = {{fact_attention_kernel<64, false, kAttnRows>, fact_attention_kernel<64, false, kAttnPair>,
-                                       fact_attention_kernel<64, false, kAttnHalf>},
+    // (head_dim 64: neither causal problems of more than a tile nor one head per item, see attention_tiles_choice)
+    static const Plain plain[2][3] = {{fact_attention_kernel<64, false, kAttnRows>, fact_attention_kernel<64, false, kAttnPair>, nullptr},
                                       {fact_attention_kernel<128, false, kAttnRows>, fact_attention_kernel<128, false, kAttnPair>,
                                        fact_attention_kernel<128, false, kAttnHalf>}};
-    static const Dealt dealt[2] = {fact_attention_kernel<64, true>, fact_attention_kernel<128, true>};
+    static const Dealt dealt = fact_attention_kernel<128, true>;
     if (!h->configured_mask.test(30)) {
       cudaError_t e = cudaSuccess;
       int regs = 1 << 30;
@@ -2405,9 +2522,10 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
         if (e == cudaSuccess) regs = std::min(regs, fa.numRegs);
       };
       for (int d = 0; d < 2; ++d) {
-        for (Plain k : plain[d]) configure(reinterpret_cast<const void*>(k));
-        configure(reinterpret_cast<const void*>(dealt[d]));
+        for (Plain k : plain[d])
+          if (k) configure(reinterpret_cast<const void*>(k));
       }
+      configure(reinterpret_cast<const void*>(dealt));
       if (e != cudaSuccess) {
         st = cuda_fail(h, "cudaFuncSetAttribute(attention)", e);
       } else if (regs < kAttnRegsAtLaunch) {
@@ -2424,8 +2542,8 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
       // CTAs up to 10 % more key blocks than the mean (16 x 12 heads x 1024 tokens: 28 block-times against 25.9), so
       // the host deals the items out itself -- heaviest first, each to the CTA with the least so far -- and hands the
       // list to the kernel as a parameter.  The list is kept for the next call of the same shape.
-      const int bk = head_dim == 64 ? 128 : 64;
-      const bool deal = causal != 0 && !one_tile && p.items > ctas && p.items <= kAttnDealItems && ctas <= kAttnDealCtas &&
+      const int bk = block_k;
+      const bool deal = causal != 0 && head_dim == 128 && !one_tile && p.items > ctas && p.items <= kAttnDealItems && ctas <= kAttnDealCtas &&
                         p.items < 16 * ctas;
       if (deal) {
         const std::array<long long, 6> key = {(long long)batch * heads_q, (long long)p.q_pairs, (long long)bk, (long long)seq_kv, (long long)ctas, (long long)seq_q};
@@ -2439,7 +2557,7 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
       cudaError_t e;
       const int d = head_dim == 128;
       if (deal)
-        e = launch_pdl(h, dealt[d], (unsigned)ctas, (unsigned)kAttnThreads, (size_t)smem, stream, 1, tq, tk, tv, to, p,
+        e = launch_pdl(h, dealt, (unsigned)ctas, (unsigned)kAttnThreads, (size_t)smem, stream, 1, tq, tk, tv, to, p,
                        *h->attn_deal);
       else
         e = launch_pdl(h, plain[d][pair ? kAttnPair : (one_tile ? kAttnHalf : kAttnRows)], (unsigned)ctas, (unsigned)kAttnThreads,

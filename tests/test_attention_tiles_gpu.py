@@ -1,0 +1,61 @@
+"""GPU parity of attention at head_dim 64 by independent tiles (three or two per SM), against the FP64 oracle under the
+gates of test_attention_gpu."""
+import numpy as np
+import pytest
+import torch
+
+from tests.test_attention_gpu import check, h, rnd  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def rows_of(T):
+    return np.array(sorted({0, 1, 31, 32, 63, 64, 95, 127, 128, T // 2, T - 2, T - 1} & set(range(T))), dtype=np.int64)
+
+
+# two tiles (fewer than three, or one and a half short ones, per SM) and three; one item per pipeline, the host's deal of
+# several, the closed form (more than 16 a pipeline); lengths at the edges of tiles and of 64- and 128-key blocks; grouped
+@pytest.mark.parametrize("B,T,Hq,Hkv", [(1, 129, 1, 1), (1, 192, 3, 3), (2, 257, 6, 2), (1, 1500, 12, 12), (1, 2049, 8, 8),
+                                        (10, 256, 12, 12), (20, 193, 12, 4), (7, 1000, 12, 12), (300, 130, 12, 12)])
+def test_causal_tiles(h, B, T, Hq, Hkv):  # noqa: F811
+    check(h, rnd((B, T, Hq, 64), 61), rnd((B, T, Hkv, 64), 62), rnd((B, T, Hkv, 64), 63), True, rows=rows_of(T))
+
+
+# without a mask: items of 256 rows would leave SMs idle (two tiles; exactly three a SM); keys ragged and of other lengths
+@pytest.mark.parametrize("B,Tq,Tk,H", [(1, 1000, 1000, 12), (2, 300, 77, 12), (4, 1300, 1, 10), (16, 300, 640, 12), (40, 384, 129, 12),
+                                       (1, 4090, 4090, 12)])
+def test_full_tiles(h, B, Tq, Tk, H):  # noqa: F811
+    check(h, rnd((B, Tq, H, 64), 64), rnd((B, Tk, H, 64), 65), rnd((B, Tk, H, 64), 66), False, rows=rows_of(Tq))
+
+
+# sequences of one tile: a head per pipeline (two), more heads than SMs with one 64-key block (three)
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("B,T", [(1, 1), (3, 63), (5, 128), (13, 64), (100, 33)])
+def test_one_tile_sequences(h, causal, B, T):  # noqa: F811
+    check(h, rnd((B, T, 12, 64), 67), rnd((B, T, 12, 64), 68), rnd((B, T, 12, 64), 69), causal, rows=rows_of(T))
+
+
+# reference maxima that move in the middle of a row (the output is rescaled), by two and by three tiles
+@pytest.mark.parametrize("B", [1, 8])
+def test_moving_maxima(h, B):  # noqa: F811
+    T = 900
+    q, k, v = rnd((B, T, 12, 64), 71, 4.0), rnd((B, T, 12, 64), 72, 4.0), rnd((B, T, 12, 64), 73)
+    k = (k.float() * torch.linspace(0.2, 2.0, T).view(1, T, 1, 1)).to(torch.bfloat16)  # later keys score higher
+    check(h, q, k, v, True, rows=rows_of(T))
+
+
+# rows of the output on 32 bytes and on 16 only (a slice of a wider buffer), whose other columns stay untouched
+@pytest.mark.parametrize("B", [1, 16])
+@pytest.mark.parametrize("pad,off", [(0, 0), (8, 0), (16, 8)])
+def test_output_rows(h, B, pad, off):  # noqa: F811
+    T, H = 300, 12
+    q, k, v = (rnd((B, T, H, 64), 74 + i).cuda() for i in range(3))
+    want = h.attention(q, k, v, causal=True)
+    buf = torch.full((B, T, H * 64 + pad), -7.0, dtype=torch.bfloat16, device="cuda")
+    out = buf[:, :, off: off + H * 64].unflatten(2, (H, 64))
+    h.attention(q, k, v, causal=True, out=out)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    assert torch.equal(out, want)
+    out.fill_(-7.0)
+    assert bool((buf == -7.0).all())
