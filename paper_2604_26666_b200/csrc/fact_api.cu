@@ -445,8 +445,12 @@ fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const f
     // taken as 0.85 at 192, rank the widths against each other; timed on untuned shapes a k-block costs 450 cycles
     // at 128 columns and 420 at 64 -- 0.57 and 0.45 -- which is what the comparison with the cluster schedule uses)
     const double eff = tn >= 256 ? 1.0 : (tn >= 192 ? 0.85 : (!calibrated ? 0.65 : (tn >= 128 ? 0.57 : 0.45)));
+    // (grouped problems run long enough for power to set the clock, and single CTAs draw less of it: 64 groups, 16384 x 2048
+    // -> 2048 195 us as 157 single tiles, 201 as 93 pairs; 8 groups, 3000 x 4096 -> 14336 gated 777 and 829; 32 groups,
+    // 16384 rows 162 and 158, 145 tiles against 81)
+    const double cg1_wide = q.groups > 0 ? 75.0 : 120.0;
     auto per_tile = [&](double kb) {
-      return kb * 512.0 * std::max(tn, 96) / 256.0 / eff + 1500.0 + (cg == 1 ? (tn >= 192 ? 120.0 : (tn >= 128 ? 100.0 : 30.0)) * kb : 0.0);
+      return kb * 512.0 * std::max(tn, 96) / 256.0 / eff + 1500.0 + (cg == 1 ? (tn >= 192 ? cg1_wide : (tn >= 128 ? 100.0 : 30.0)) * kb : 0.0);
     };
     // (a pair's launch costs about 1 us more -- cluster placement, the pair's barriers: 744 x 768 -> 2304 takes 7.3 us as
     // pairs of 128-column tiles and 6.6 as single CTAs, 2000 rows 9.7 and 8.8 with 256 columns -- which its cheaper k-blocks
