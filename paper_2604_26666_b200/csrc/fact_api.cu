@@ -138,7 +138,7 @@ struct fact_handle_s {
   long long launches = 0;
   std::map<TuneKey, fact_config_t> table;
   std::unordered_map<ChoiceKey, Choice, ChoiceHash> choices;  // cleared with every change of the table
-  std::bitset<192> configured_mask;  // kernels whose dynamic shared-memory limit was raised
+  std::bitset<200> configured_mask;  // kernels whose dynamic shared-memory limit was raised
   std::unique_ptr<AttnDeal> attn_deal;         // the host's deal of the last causal attention shape (see fact_attention)
   std::array<long long, 6> attn_deal_key{};
   std::unique_ptr<AttnTilesDeal> attn_tiles_deal;  // the same at head_dim 64
@@ -1422,7 +1422,7 @@ fact_status_t attention_tiles(fact_handle_t h, AttnParams p, const CUtensorMap& 
   const auto plain = fact_attention_tiles_kernel<TILES, false>;
   const auto dealt = fact_attention_tiles_kernel<TILES, true>;
   const int smem = std::max((int)L::kSmemBytes, kMinSmemRequest);
-  const size_t bit = TILES == 3 ? 29 : 28;
+  const size_t bit = TILES == 3 ? 193 : 192;  // (above every slot of the GEMM instantiations)
   if (!h->configured_mask.test(bit)) {
     for (const void* kern : {reinterpret_cast<const void*>(plain), reinterpret_cast<const void*>(dealt)}) {
       cudaFuncAttributes fa;

@@ -59,3 +59,20 @@ def test_output_rows(h, B, pad, off):  # noqa: F811
     assert torch.equal(out, want)
     out.fill_(-7.0)
     assert bool((buf == -7.0).all())
+
+
+def test_after_stream_k_products_on_the_same_handle():
+    """Every kernel's shared-memory limit is raised once per handle and remembered under a bit of its own: the first attention
+    calls of a handle that has run stream-K products of pairs with the last epilogues."""
+    from paper_2604_26666_b200.binding import Handle
+    hd = Handle(0)
+    g = torch.Generator().manual_seed(80)
+    X = torch.randn(640, 512, generator=g).to(torch.bfloat16).cuda()
+    W = torch.randn(512, 512, generator=g).to(torch.bfloat16).cuda()
+    R = torch.randn(640, 512, generator=g).to(torch.bfloat16).cuda()
+    cfg = {"cta_group": 2, "tile_n": 256, "split_k": -1}
+    hd.linear(X, W, residual=R, epilogue="BIAS_RESIDUAL", layout="NK", cfg=cfg)
+    hd.linear(X, W, epilogue="SILU_GATE", layout="NK", cfg=cfg)
+    for B in (1, 16):
+        check(hd, rnd((B, 300, 12, 64), 81), rnd((B, 300, 12, 64), 82), rnd((B, 300, 12, 64), 83), True, rows=rows_of(300))
+    hd.close()
