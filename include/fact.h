@@ -356,12 +356,14 @@ fact_status_t fact_linear_fp8(fact_handle_t handle, int64_t M, int64_t N_out, in
  * shared key/value heads are read in place)
  * Q: BF16 [batch][seq_q][heads_q][head_dim], K and V: BF16 [batch][seq_kv][heads_kv][head_dim], O: BF16 like Q,
  * each addressed by three strides in elements (batch, token, head; head_dim itself is contiguous), so the
- * operands may be views into a fused QKV projection or stored heads-first.  Query head h uses key/value
+ * operands may be views into a fused QKV projection or stored heads-first.  A batch stride of 0 means that all
+ * batch entries share one Q, K or V (a common prefix's cache); O's must not be 0 when batch > 1.  Query head h uses key/value
  * head h / (heads_q / heads_kv).  Scores and probabilities are FP32, P is rounded to BF16 for the second
  * product, O is accumulated in FP32 and rounded once.  causal != 0 masks keys j > i and requires
  * seq_q == seq_kv; scale <= 0 means 1 / sqrt(head_dim).
  * Requirements: head_dim 64 or 128; heads_q a multiple of heads_kv; all four pointers 16-byte aligned and
- * every stride a multiple of 8 elements (operands are read and O is written through TMA).  Errors: FACT_ERR_UNSUPPORTED for another head_dim or causal with seq_q != seq_kv,
+ * every stride a multiple of 8 elements (K and V are read through TMA, Q and O through TMA or in 4- to 32-byte
+ * pieces).  Errors: FACT_ERR_UNSUPPORTED for another head_dim or causal with seq_q != seq_kv,
  * FACT_ERR_BAD_ALIGNMENT, FACT_ERR_INVALID_ARG; nothing is launched on an error.  batch == 0 or
  * seq_q == 0 is a successful no-op. */
 fact_status_t fact_attention(fact_handle_t handle, int64_t batch, int64_t seq_q, int64_t seq_kv, int64_t heads_q,

@@ -60,6 +60,7 @@ struct AttnParams {
   __nv_bfloat16* O;           // rows are stored from registers: batch, token and head strides in elements
   long long o_sb, o_st, o_sh;
   int o_vec32;                // rows of O start on 32 bytes
+  int q_each, k_each, v_each; // 1; 0 where all batch entries share one Q, K or V (batch stride 0: a map of one entry)
   uint64_t kmajor_desc;       // UMMA descriptor template, K-major 128B-swizzled tiles (Q, K)
   uint64_t v_desc;            // UMMA descriptor template, V as an N-major operand
   uint32_t idesc_s, idesc_pv;
@@ -315,7 +316,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             ptx::mbar_arrive_expect_tx(bar(Q_FULL + t), tile_bytes);
             for (int c = 0; c < chunks; ++c)
               ptx::tma_load_4d(q_s0 + (uint32_t)t * tile_bytes + c * kAttnChunkBytes, &tmQ, bar(Q_FULL + t), c * 64,
-                               t ? it.h1 : it.h, PAIR ? 0 : it.t0 + t * kAttnBlockQ, t ? it.b1 : it.b);
+                               t ? it.h1 : it.h, PAIR ? 0 : it.t0 + t * kAttnBlockQ, (t ? it.b1 : it.b) * p.q_each);
           }
         }
         for (int r = 0; ok && r < it.nbi; ++r, ++g) {
@@ -329,16 +330,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (ptx::elect_one()) {
             ptx::mbar_arrive_expect_tx(bar(K_FULL + s), kv_bytes);
             for (int c = 0; c < chunks; ++c)
-              ptx::tma_load_4d_hint(k_s0 + s * kv_bytes + c * kv_chunk, &tmK, bar(K_FULL + s), c * 64, kvh, j * BK, kb,
-                                    keep);
+              ptx::tma_load_4d_hint(k_s0 + s * kv_bytes + c * kv_chunk, &tmK, bar(K_FULL + s), c * 64, kvh, j * BK,
+                                    kb * p.k_each, keep);
           }
           ok = wait_all(bar(V_EMPTY + s), par);
           if (!ok) break;
           if (ptx::elect_one()) {
             ptx::mbar_arrive_expect_tx(bar(V_FULL + s), kv_bytes);
             for (int c = 0; c < chunks; ++c)
-              ptx::tma_load_4d_hint(v_s0 + s * kv_bytes + c * kv_chunk, &tmV, bar(V_FULL + s), c * 64, kvh, j * BK, kb,
-                                    keep);
+              ptx::tma_load_4d_hint(v_s0 + s * kv_bytes + c * kv_chunk, &tmV, bar(V_FULL + s), c * 64, kvh, j * BK,
+                                    kb * p.v_each, keep);
           }
         }
       }

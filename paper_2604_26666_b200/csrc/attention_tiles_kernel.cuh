@@ -176,11 +176,11 @@ __global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
         AttnTile it;
       };
       Cursor kc{0, 0, 0, item_of(0)}, vc{0, 0, 0, kc.it};
-      auto load_kv = [&](Cursor& c, const CUtensorMap* map, uint32_t ring, int full, int stages) {
+      auto load_kv = [&](Cursor& c, const CUtensorMap* map, uint32_t ring, int full, int stages, int each) {
         if (c.n >= n_items) return;
         if (ptx::elect_one()) {
           ptx::mbar_arrive_expect_tx(bar(full + c.slot), L::kKvBytes);
-          ptx::tma_load_4d_hint(ring + (uint32_t)c.slot * L::kKvBytes, map, bar(full + c.slot), 0, c.it.kvh, c.j * BK, c.it.b, keep);
+          ptx::tma_load_4d_hint(ring + (uint32_t)c.slot * L::kKvBytes, map, bar(full + c.slot), 0, c.it.kvh, c.j * BK, c.it.b * each, keep);
         }
         __syncwarp();
         if (++c.slot == stages) c.slot = 0;
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
       auto load_q = [&](const AttnTile& it) {
         if (ptx::elect_one()) {
           ptx::mbar_arrive_expect_tx(bar(L::kQFull), L::kTileBytes);
-          ptx::tma_load_4d(q_s, &tmQ, bar(L::kQFull), 0, it.h, it.t0, it.b);
+          ptx::tma_load_4d(q_s, &tmQ, bar(L::kQFull), 0, it.h, it.t0, it.b * p.q_each);
         }
         __syncwarp();
       };
@@ -200,8 +200,8 @@ __global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
       load_q(it);
 #pragma unroll 1
       for (int i = 0; i < L::kKStages; ++i) {
-        load_kv(kc, &tmK, k_s, L::kKFull, L::kKStages);
-        if (i < L::kVStages) load_kv(vc, &tmV, v_s, L::kVFull, L::kVStages);
+        load_kv(kc, &tmK, k_s, L::kKFull, L::kKStages, p.k_each);
+        if (i < L::kVStages) load_kv(vc, &tmV, v_s, L::kVFull, L::kVStages, p.v_each);
       }
       const uint64_t qdesc0 = p.kmajor_desc | (uint64_t)((q_s >> 4) & 0x3fffu);
       int ks = 0, vs = 0;         // ring slots of the next first and second product
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
             it = item_of(n + 1);
             load_q(it);
           }
-          load_kv(kc, &tmK, k_s, L::kKFull, L::kKStages);  // ... into the slot of the block whose scores have been read
+          load_kv(kc, &tmK, k_s, L::kKFull, L::kKStages, p.k_each);  // ... into the slot of the block whose scores have been read
           ok = wait_all(bar(L::kPFull), (uint32_t)gt & 1u);
           // the first block of an item overwrites O: the previous item's must have been read
           if (ok && j == 0 && n > 0) ok = wait_all(bar(L::kOFree), (uint32_t)(n - 1) & 1u);
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
             vpar ^= 1u;
           }
           // the probabilities were stored after the second product of the block before: its V slot is free
-          if (gt > 0) load_kv(vc, &tmV, v_s, L::kVFull, L::kVStages);
+          if (gt > 0) load_kv(vc, &tmV, v_s, L::kVFull, L::kVStages, p.v_each);
         }
       }
       __syncwarp();

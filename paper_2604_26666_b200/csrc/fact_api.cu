@@ -2338,10 +2338,15 @@ fact_status_t fact_tune_cache_load(fact_handle_t h, const char* path) {
 // ---------------------------------------------------------------------------------------------
 // Fused multi-head attention
 namespace {
-// Rank-4 BF16 tensor map over [B][T][H][D]-like storage, dims ordered (D, H, T, B), box 64 x 1 x box_rows x 1.
+// Rank-4 BF16 tensor map over [B][T][H][D]-like storage, dims ordered (D, H, T, B), box 64 x 1 x box_rows x 1.  A batch
+// stride of 0 (one Q, K or V for all entries) is a map of one entry, which the kernels address with coordinate 0.
 fact_status_t encode_map_bthd(fact_handle_t h, CUtensorMap* map, const void* base, long long D, long long H, long long T,
                               long long B, long long stride_h, long long stride_t, long long stride_b,
                               int box_rows = kAttnBlockQ) {
+  if (B == 1 || stride_b == 0) {  // (the stride is not used, but has to be a valid one)
+    B = 1;
+    stride_b = std::max<long long>(stride_t * T, 8);
+  }
   cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T, (cuuint64_t)B};
   cuuint64_t strides[3] = {(cuuint64_t)stride_h * 2, (cuuint64_t)stride_t * 2, (cuuint64_t)stride_b * 2};
   cuuint32_t box[4] = {64, 1, (cuuint32_t)box_rows, 1};
@@ -2361,12 +2366,9 @@ fact_status_t attention_decode(fact_handle_t h, int64_t batch, int64_t seq_q, in
                                int64_t head_dim, const void* Q, const int64_t (&strides)[12], const void* K, const void* V,
                                void* O, float scale, cudaStream_t stream) {
   CUtensorMap tk, tv;
-  auto bs = [&](int64_t s, int64_t fallback) { return (batch > 1 && s > 0) ? s : std::max<int64_t>(fallback, 8); };
-  fact_status_t st = encode_map_bthd(h, &tk, K, head_dim, heads_kv, seq_kv, batch, strides[5], strides[4],
-                                     bs(strides[3], strides[4] * seq_kv), kDecBlockK);
+  fact_status_t st = encode_map_bthd(h, &tk, K, head_dim, heads_kv, seq_kv, batch, strides[5], strides[4], strides[3], kDecBlockK);
   if (st == FACT_OK)
-    st = encode_map_bthd(h, &tv, V, head_dim, heads_kv, seq_kv, batch, strides[8], strides[7],
-                         bs(strides[6], strides[7] * seq_kv), kDecBlockK);
+    st = encode_map_bthd(h, &tv, V, head_dim, heads_kv, seq_kv, batch, strides[8], strides[7], strides[6], kDecBlockK);
   if (st != FACT_OK) return st;
   DecodeParams p;
   memset(&p, 0, sizeof p);
@@ -2383,6 +2385,8 @@ fact_status_t attention_decode(fact_handle_t h, int64_t batch, int64_t seq_q, in
   p.Hkv = (int)heads_kv;
   p.group = (int)(heads_q / heads_kv);
   p.rows = p.Tq * p.group;
+  p.k_each = strides[3] != 0;
+  p.v_each = strides[6] != 0;
   p.scale_log2 = (float)((scale > 0.f ? (double)scale : 1.0 / std::sqrt((double)head_dim)) * 1.4426950408889634);
   p.status = h->d_status;
   const long long pairs = (long long)batch * heads_kv;
@@ -2442,6 +2446,7 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     if (strides[i] % 8) return FACT_ERR_BAD_ALIGNMENT;
     if (!batch_stride && strides[i] < head_dim) return FACT_ERR_INVALID_ARG;
   }
+  if (batch > 1 && o_sb == 0) return FACT_ERR_INVALID_ARG;  // (one Q, K or V for all entries is fine, one O is not)
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_v);
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return FACT_ERR_CUDA;
@@ -2453,19 +2458,18 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     return ds;
   }
   CUtensorMap tq, tk, tv, to;
-  auto bs = [&](int64_t s, int64_t fallback) { return (batch > 1 && s > 0) ? s : std::max<int64_t>(fallback, 8); };
   const long long q_tiles = (seq_q + kAttnBlockQ - 1) / kAttnBlockQ;
   const long long tile_items = q_tiles * heads_q * batch;
   const int tiles = head_dim == 64 ? attention_tiles_choice(q_tiles, heads_q * batch, seq_kv, causal != 0, h->sm_count) : 0;
   // keys go in blocks of 128 or 64, as the kernels' tensor-memory budgets have it
   const int block_k = tiles == 3 ? AttnTiles<3>::kBlockK : (tiles == 2 ? AttnTiles<2>::kBlockK : attn_block_k((int)head_dim));
-  fact_status_t st = encode_map_bthd(h, &tq, Q, head_dim, heads_q, seq_q, batch, q_sh, q_st, bs(q_sb, q_st * seq_q));
+  fact_status_t st = encode_map_bthd(h, &tq, Q, head_dim, heads_q, seq_q, batch, q_sh, q_st, q_sb);
   if (st == FACT_OK)
-    st = encode_map_bthd(h, &tk, K, head_dim, heads_kv, seq_kv, batch, k_sh, k_st, bs(k_sb, k_st * seq_kv), block_k);
+    st = encode_map_bthd(h, &tk, K, head_dim, heads_kv, seq_kv, batch, k_sh, k_st, k_sb, block_k);
   if (st == FACT_OK)
-    st = encode_map_bthd(h, &tv, V, head_dim, heads_kv, seq_kv, batch, v_sh, v_st, bs(v_sb, v_st * seq_kv), block_k);
+    st = encode_map_bthd(h, &tv, V, head_dim, heads_kv, seq_kv, batch, v_sh, v_st, v_sb, block_k);
   if (st == FACT_OK && tiles == 0)
-    st = encode_map_bthd(h, &to, O, head_dim, heads_q, seq_q, batch, o_sh, o_st, bs(o_sb, o_st * seq_q));
+    st = encode_map_bthd(h, &to, O, head_dim, heads_q, seq_q, batch, o_sh, o_st, o_sb);
   if (st == FACT_OK) {
     AttnParams p;
     memset(&p, 0, sizeof p);
@@ -2476,6 +2480,9 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     p.Hkv = (int)heads_kv;
     p.D = (int)head_dim;
     p.causal = causal != 0;
+    p.q_each = q_sb != 0;
+    p.k_each = k_sb != 0;
+    p.v_each = v_sb != 0;
     const double sc = scale > 0.f ? (double)scale : 1.0 / std::sqrt((double)head_dim);
     p.scale_log2 = (float)(sc * 1.4426950408889634);
     p.kmajor_desc = smem_desc_template(16, 1024);
@@ -2489,10 +2496,10 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
       p.q_tiles = (int)q_tiles;
       p.items = (int)tile_items;
       p.O = static_cast<__nv_bfloat16*>(O);
-      p.o_sb = bs(o_sb, o_st * seq_q);
+      p.o_sb = o_sb;
       p.o_st = o_st;
       p.o_sh = o_sh;
-      p.o_vec32 = (reinterpret_cast<uintptr_t>(O) & 31u) == 0 && p.o_sb % 16 == 0 && o_st % 16 == 0 && o_sh % 16 == 0;
+      p.o_vec32 = (reinterpret_cast<uintptr_t>(O) & 31u) == 0 && (batch == 1 || o_sb % 16 == 0) && o_st % 16 == 0 && o_sh % 16 == 0;
       st = tiles == 3 ? attention_tiles<3>(h, p, tq, tk, tv, stream) : attention_tiles<2>(h, p, tq, tk, tv, stream);
       if (dev != h->device) cudaSetDevice(dev);
       return st;
