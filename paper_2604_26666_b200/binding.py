@@ -569,7 +569,8 @@ class Handle:
         (and w_colsum for "layer") folds a normalisation of X's rows into the product (fact_linear_ex)."""
         if cfg is None and stream is None and stats_out is None and x_norm is None and x_stats is None and w_colsum is None:
             r = self._bind.linear(self._hp, self.device, self._ws, self._ws_streams, X, W, None, bias, residual,
-                                  EPILOGUES.get(epilogue, -1), LAYOUTS.get(layout, -1), out, _OUT_CODES.get(out_dtype, -1), None)
+                                  EPILOGUES.get(epilogue, -1), LAYOUTS.get(layout, -1), out, _OUT_CODES.get(out_dtype, -1), None,
+                                  0)
             if r is not None:
                 return r
         _need(X, "X", torch.bfloat16, 2)
@@ -660,7 +661,7 @@ class Handle:
         (layout "NK") or [G, K, Nw] ("KN"); group_rows: G row counts summing to M (host integers)."""
         if cfg is None and stream is None:
             r = self._bind.linear(self._hp, self.device, None, None, X, W, None, bias, residual, EPILOGUES.get(epilogue, -1),
-                                  LAYOUTS.get(layout, -1), out, _OUT_CODES.get(out_dtype, -1), group_rows)
+                                  LAYOUTS.get(layout, -1), out, _OUT_CODES.get(out_dtype, -1), group_rows, 2)
             if r is not None:
                 return r
         _need(X, "X", torch.bfloat16, 2)
@@ -694,7 +695,7 @@ class Handle:
         """fact_linear_grouped_fp8: X [M, K] and W [G, Nw, K] are FP8 E4M3 (torch.float8_e4m3fn or uint8 codes)."""
         if cfg is None and stream is None:
             r = self._bind.linear(self._hp, self.device, None, None, X, W, scale, bias, None, EPILOGUES.get(epilogue, -1), 1,
-                                  out, _OUT_CODES.get(out_dtype, -1), group_rows)
+                                  out, _OUT_CODES.get(out_dtype, -1), group_rows, 3)
             if r is not None:
                 return r
         def codes(t, name, nd):
@@ -729,7 +730,7 @@ class Handle:
         tensors, or torch.uint8 tensors holding the codes."""
         if cfg is None and stream is None:
             r = self._bind.linear(self._hp, self.device, self._ws, self._ws_streams, X, W, scale, bias, residual,
-                                  EPILOGUES.get(epilogue, -1), 1, out, _OUT_CODES.get(out_dtype, -1), None)
+                                  EPILOGUES.get(epilogue, -1), 1, out, _OUT_CODES.get(out_dtype, -1), None, 1)
             if r is not None:
                 return r
         def codes(t, name):
@@ -821,7 +822,7 @@ class Handle:
 
     def block_forward(self, desc, x, out=None, workspace=None, stream=None):
         """One transformer block forward (fact_block_forward).  x: [batch * seq, hidden] BF16, contiguous."""
-        if stream is None and workspace is None:
+        if stream is None and workspace is None and type(desc) is Block:  # (only the address is passed on)
             r = self._bind.block_forward(self._hp, self.device, self._ws, self._ws_streams, ctypes.addressof(desc), x, out)
             if r is not None:
                 return r

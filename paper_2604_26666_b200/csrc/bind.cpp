@@ -166,14 +166,15 @@ const Tensor* codes(PyObject* o, int64_t ndim, int dev) {
   return t != nullptr ? t : plain(o, at::kByte, ndim, dev);
 }
 
-// (handle, device, ws, streams, X, W, scale or None, bias, residual, epilogue, layout, out, type of a new one, group rows
-// or None): the linear layers; scale given = FP8 operands, group rows given = one weight matrix per group
+// (handle, device, ws, streams, X, W, scale, bias, residual, epilogue, layout, out, type of a new one, group rows, which):
+// the linear layers; bit 0 of `which`: FP8 operands with their scale, bit 1: one weight matrix per group of rows
 PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded([&]() -> PyObject* {
-    if (n != 14) return nullptr;
+    if (n != 15) return nullptr;
     Call c(a[0], a[1]);
     if (!c.ok) return nullptr;
-    const bool fp8 = a[6] != Py_None, grouped = a[13] != Py_None;
+    const long which = PyLong_AsLong(a[14]);
+    const bool fp8 = which & 1, grouped = which & 2;
     const auto epi = (fact_epilogue_t)PyLong_AsLong(a[9]);
     const auto layout = (fact_blayout_t)PyLong_AsLong(a[10]);
     const double scale = fp8 ? PyFloat_AsDouble(a[6]) : 1.0;

@@ -1,5 +1,7 @@
 """The extension's marshalling against the ctypes marshalling (a call that names its stream): the same bits from every
 method, the same errors for wrong arguments, and the library's kept choices follow the tuner's table."""
+import ctypes
+
 import pytest
 import torch
 
@@ -85,6 +87,14 @@ def test_wrong_arguments_raise_what_they_raised(h):
         h.linear_grouped(x, rnd(2, 96, 128), [10, 20])
     with pytest.raises(FactError):
         h.attention(rnd(1, 4, 3, 64), rnd(1, 4, 2, 64), rnd(1, 4, 2, 64))
+    # (None for what makes a call a grouped or an FP8 one does not make it another method's call)
+    x8, w8 = x.to(torch.float8_e4m3fn), w.to(torch.float8_e4m3fn)
+    for wrong in (lambda: h.linear_grouped(x, w, None), lambda: h.linear_fp8(x, w, None), lambda: h.linear_fp8(x8, w8, None),
+                  lambda: h.linear_grouped_fp8(x, torch.stack([w, w]), [32, 32], None), lambda: h.linear_grouped_fp8(x8, w8, None)):
+        with pytest.raises((TypeError, ValueError)):
+            wrong()
+    with pytest.raises((TypeError, ctypes.ArgumentError)):
+        h.block_forward(ctypes.pointer(h.block_desc("gpt", 1, 64, 2, 2, 64, 128, {})), x)
     assert h.launch_count() == launches
     assert torch.isfinite(h.gemm(x, w, layout="NK").float()).all()
 
