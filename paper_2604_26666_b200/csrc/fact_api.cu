@@ -366,7 +366,8 @@ uint32_t skinny_part_bytes(int rows, int groups) {
   return (uint32_t)(kSkinnyWarps / (rows == 64 ? 2 : 1)) * 8u * (uint32_t)groups * (uint32_t)(rows + 4) * 4u;
 }
 
-// Fill every zero field of `cfg`.  Returns FACT_ERR_UNSUPPORTED for a combination the kernels cannot run.
+// Fill every zero field of `cfg`.  Returns FACT_ERR_UNSUPPORTED for a combination the kernels cannot run;
+// `from_table_out` says then, too, whether it was the tuner's table that asked for it.
 fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const fact_config_t* user, int splits_override,
                              fact_config_t* out, bool* from_table_out = nullptr) {
   fact_config_t c;
@@ -374,12 +375,15 @@ fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const f
   bool from_table = false;
   if (user) c = *user;
   else {
+    // (the key knows nothing of row sums, a folded normalisation or groups: an entry of the few-rows kernel, tuned on a
+    // plain call of the shape, says nothing about such a call)
     auto it = h->table.find(make_key(q));
-    if (it != h->table.end()) {
+    if (it != h->table.end() && (it->second.schedule != 4 || skinny_ok(q))) {
       c = it->second;
       from_table = true;
     }
   }
+  if (from_table_out) *from_table_out = from_table;
   if (splits_override > 0) c.split_k = splits_override;
   // At most 64 rows: the kernel that streams the weights.  Above 32 rows and several waves of CTAs the rows' own traffic
   // from L2 costs more than the tile kernels' padding (64 rows, 4096 -> 2 x 14336: 55.0 us against 43.5).
@@ -396,7 +400,6 @@ fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const f
     if (stages < 2 || stages > smax) return FACT_ERR_UNSUPPORTED;
     const fact_config_t sk = {8 * groups, rows, kTileK, stages, 1, 1, 1, 1, 4};
     *out = sk;
-    if (from_table_out) *from_table_out = from_table;
     return FACT_OK;
   }
   if (c.tile_k != 0 && c.tile_k != q.k_elems()) return FACT_ERR_UNSUPPORTED;
@@ -570,7 +573,6 @@ fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const f
   if (c.schedule < 0 || c.schedule > 4) return FACT_ERR_INVALID_ARG;
   if (c.schedule == 0) c.schedule = 1;
   *out = c;
-  if (from_table_out) *from_table_out = from_table;
   return FACT_OK;
 }
 
@@ -590,10 +592,8 @@ fact_status_t resolve_config(fact_handle_t h, const Problem& q, const fact_confi
     if (h->choices.size() >= kMaxChoices) h->choices.clear();
     it = h->choices.emplace(key, c).first;
   }
-  if (it->second.status == FACT_OK) {
-    *out = it->second.cfg;
-    if (from_table_out) *from_table_out = it->second.from_table;
-  }
+  if (it->second.status == FACT_OK) *out = it->second.cfg;
+  if (from_table_out) *from_table_out = it->second.from_table;
   return it->second.status;
 }
 
@@ -1134,8 +1134,8 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
   Plan plan;
   st = make_plan(h, q, user, splits_override, &plan);
   if (st == FACT_ERR_UNSUPPORTED && plan.from_table) {
-    // a table entry with K slices as a cluster or the few-rows kernel, tuned on a plain call of this shape: this call
-    // (row sums, a folded normalisation) takes the library's own choice instead
+    // a table entry that this call cannot run (K slices as a cluster, tuned on a plain call of the shape: not with row sums,
+    // a folded normalisation or groups): the library's own choice instead
     fact_config_t none;
     memset(&none, 0, sizeof none);
     none.split_k = 1;

@@ -66,3 +66,25 @@ def test_what_it_does_not_serve_is_refused_or_goes_elsewhere(h):  # noqa: F811
     y = h.linear(X, W, stats_out=stats)  # (row sums out: the tile kernel)
     assert (y == 128.0).all() and (stats[..., 0] == 64 * 128.0).all()
     assert (h.linear(X, W.t().contiguous(), layout="KN", epilogue="SILU_GATE") > 0).all()
+
+
+def test_a_tuned_entry_is_for_plain_calls_only(h, tmp_path):  # noqa: F811
+    # the table's key is the shape: calls of it that the kernel does not serve take the library's own choice
+    from paper_2604_26666_b200.binding import Handle
+
+    M, N, K = 8, 256, 128
+    X, W = torch.ones(M, K, dtype=torch.bfloat16).cuda(), torch.ones(N, K, dtype=torch.bfloat16).cuda()
+    path = tmp_path / "table.txt"
+    for entry in ("8 16 64 4 1 1 1 1 4", "128 64 64 4 1 1 2 0 3"):  # few rows; K slices as a cluster
+        path.write_text(f"3 0 1 0 1 {M} {N} {K} | {entry}\n")
+        t = Handle(0, load_table=False)
+        t.tune_cache_load(str(path))
+        assert t.get_config("linear", 1, M, N, K, "NONE", "NK").schedule == int(entry[-1])
+        assert (t.linear(X, W) == K).all()
+        stats = torch.empty(N // 64, M, 2, device="cuda")
+        assert (t.linear(X, W, stats_out=stats) == K).all() and (stats[..., 0] == 64 * K).all()
+        folded = t.linear(X, W, x_norm="rms", x_stats=t.row_stats(X), eps=0.0)
+        assert torch.allclose(folded.float(), torch.full_like(folded, K).float(), rtol=2 ** -7)
+        assert (t.linear_grouped(X, W.expand(3, N, K).contiguous(), [3, 0, 5]) == K).all()
+        assert t.device_status() == 0
+        t.close()
