@@ -214,6 +214,13 @@ def _check(code: int, where: str, handle=None):
         raise FactError(code, where)
 
 
+def _result(r, where: str, handle):
+    """What the extension answered: the output, or the status of a call that failed after it had launched something."""
+    if type(r) is int:
+        _check(r, where, handle)
+    return r
+
+
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else c_void_p(t.data_ptr())
 
@@ -475,7 +482,7 @@ class Handle:
             r = self._bind.matmul(self._hp, self.device, self._ws, self._ws_streams, 0, A, B, LAYOUTS.get(layout, -1), out,
                                   _OUT_CODES.get(out_dtype, -1))
             if r is not None:
-                return r
+                return _result(r, "fact_gemm", self._h)
         _, M, N, K = _validate_matmul(A, B, out, layout)
         if out is None:
             out = torch.empty((M, N), dtype=out_dtype, device=A.device)
@@ -531,7 +538,7 @@ class Handle:
             r = self._bind.matmul(self._hp, self.device, self._ws, self._ws_streams, 1, A, B, LAYOUTS.get(layout, -1), out,
                                   _OUT_CODES.get(out_dtype, -1))
             if r is not None:
-                return r
+                return _result(r, "fact_gemm_batched", self._h)
         batch, M, N, K = _validate_matmul(A, B, out, layout, batched=True)
         if out is None:
             out = torch.empty((batch, M, N), dtype=out_dtype, device=A.device)
@@ -549,7 +556,7 @@ class Handle:
             r = self._bind.matmul(self._hp, self.device, self._ws, self._ws_streams, 2, A, B, LAYOUTS.get(layout, -1), out,
                                   _OUT_CODES.get(out_dtype, -1))
             if r is not None:
-                return r
+                return _result(r, "fact_gemm_splitk", self._h)
         _, M, N, K = _validate_matmul(A, B, out, layout)
         if out is None:
             out = torch.empty((M, N), dtype=out_dtype, device=A.device)
@@ -572,7 +579,7 @@ class Handle:
                                   EPILOGUES.get(epilogue, -1), LAYOUTS.get(layout, -1), out, _OUT_CODES.get(out_dtype, -1), None,
                                   0)
             if r is not None:
-                return r
+                return _result(r, "fact_linear", self._h)
         _need(X, "X", torch.bfloat16, 2)
         _need(W, "W", torch.bfloat16, 2)
         M, K = X.shape
@@ -663,7 +670,7 @@ class Handle:
             r = self._bind.linear(self._hp, self.device, None, None, X, W, None, bias, residual, EPILOGUES.get(epilogue, -1),
                                   LAYOUTS.get(layout, -1), out, _OUT_CODES.get(out_dtype, -1), group_rows, 2)
             if r is not None:
-                return r
+                return _result(r, "fact_linear_grouped", self._h)
         _need(X, "X", torch.bfloat16, 2)
         _need(W, "W", torch.bfloat16, 3)
         rows = [int(r) for r in group_rows]
@@ -697,7 +704,7 @@ class Handle:
             r = self._bind.linear(self._hp, self.device, None, None, X, W, scale, bias, None, EPILOGUES.get(epilogue, -1), 1,
                                   out, _OUT_CODES.get(out_dtype, -1), group_rows, 3)
             if r is not None:
-                return r
+                return _result(r, "fact_linear_grouped_fp8", self._h)
         def codes(t, name, nd):
             if isinstance(t, torch.Tensor) and t.dtype == torch.float8_e4m3fn:
                 t = t.view(torch.uint8)
@@ -732,7 +739,7 @@ class Handle:
             r = self._bind.linear(self._hp, self.device, self._ws, self._ws_streams, X, W, scale, bias, residual,
                                   EPILOGUES.get(epilogue, -1), 1, out, _OUT_CODES.get(out_dtype, -1), None, 1)
             if r is not None:
-                return r
+                return _result(r, "fact_linear_fp8", self._h)
         def codes(t, name):
             if isinstance(t, torch.Tensor) and t.dtype == torch.float8_e4m3fn:
                 t = t.view(torch.uint8)
@@ -775,7 +782,7 @@ class Handle:
         if stream is None:
             r = self._bind.attention(self._hp, self.device, q, k, v, causal, scale, out)
             if r is not None:
-                return r
+                return _result(r, "fact_attention", self._h)
         for name, t in (("q", q), ("k", k), ("v", v)):
             _need(t, name, torch.bfloat16, 4)
         B, Tq, Hq, D = q.shape
@@ -795,7 +802,7 @@ class Handle:
         if stream is None:
             r = self._bind.norm(self._hp, self.device, x, gamma, beta, NORMS.get(kind, -1), eps, out)
             if r is not None:
-                return r
+                return _result(r, "fact_norm", self._h)
         _need(x, "x", torch.bfloat16, 2)
         M, C = x.shape
         if out is None:
@@ -825,7 +832,7 @@ class Handle:
         if stream is None and workspace is None and type(desc) is Block:  # (only the address is passed on)
             r = self._bind.block_forward(self._hp, self.device, self._ws, self._ws_streams, ctypes.addressof(desc), x, out)
             if r is not None:
-                return r
+                return _result(r, "fact_block_forward", self._h)
         _need(x, "x", torch.bfloat16, 2)
         if not x.is_contiguous():
             raise ValueError("x must be contiguous")

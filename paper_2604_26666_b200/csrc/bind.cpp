@@ -7,7 +7,9 @@
 // call takes the host 4 us instead of 15-20 (512^3 with bias and ReLU, one after another: 16.6 -> 5.1 us, the kernel 4.7).
 //
 // Every function returns the output tensor, or None if anything about the call is not ordinary or the library refused
-// it: the Python method then goes its own way, whose checks name the mistake.  Nothing is launched before None.
+// it: the Python method then goes its own way, whose checks name the mistake.  Nothing has been launched when the answer is
+// None; where the library failed after a launch (a late stage of a block, the reduction behind a sliced product), it is the
+// library's status, which the Python method raises.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -45,11 +47,19 @@ struct Call {
   int dev = 0;
   cudaStream_t stream = nullptr;
   bool ok = false;
+  int64_t launches = 0;  // of the handle, before this call
   Call(PyObject* handle, PyObject* device) {
     h = reinterpret_cast<fact_handle_t>(PyLong_AsVoidPtr(handle));
     dev = (int)PyLong_AsLong(device);
     ok = h != nullptr && !PyErr_Occurred();
-    if (ok) stream = c10::cuda::getCurrentCUDAStream((c10::DeviceIndex)dev).stream();
+    if (!ok) return;
+    stream = c10::cuda::getCurrentCUDAStream((c10::DeviceIndex)dev).stream();
+    launches = fact_launch_count(h);
+  }
+  template <typename O>
+  PyObject* answer(fact_status_t st, O& out) const {
+    if (st == FACT_OK) return out.result();
+    return fact_launch_count(h) != launches ? PyLong_FromLong((long)st) : nullptr;
   }
 };
 
@@ -156,7 +166,7 @@ PyObject* matmul(PyObject*, PyObject* const* a, Py_ssize_t n) {
     } else {
       st = without_gil([&] { return fact_gemm(c.h, M, N, K, pa, lda, pb, ldb, layout, pc, ldc, ot, nullptr, ws, need, c.stream); });
     }
-    return st == FACT_OK ? out.result() : nullptr;
+    return c.answer(st, out);
   });
 }
 
@@ -243,7 +253,7 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
                                  c.stream);
       });
     }
-    return st == FACT_OK ? out.result() : nullptr;
+    return c.answer(st, out);
   });
 }
 
@@ -267,7 +277,7 @@ PyObject* attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
                             v->stride(0), v->stride(1), v->stride(2), out.t->data_ptr(), out.t->stride(0), out.t->stride(1),
                             out.t->stride(2), causal, (float)scale, c.stream);
     });
-    return st == FACT_OK ? out.result() : nullptr;
+    return c.answer(st, out);
   });
 }
 
@@ -288,7 +298,7 @@ PyObject* norm(PyObject*, PyObject* const* a, Py_ssize_t n) {
       return fact_norm(c.h, kind, x->size(0), x->size(1), x->const_data_ptr(), ld(*x), g->const_data_ptr(),
                        b ? b->const_data_ptr() : nullptr, (float)eps, out.t->data_ptr(), ld(*out.t), c.stream);
     });
-    return st == FACT_OK ? out.result() : nullptr;
+    return c.answer(st, out);
   });
 }
 
@@ -308,7 +318,7 @@ PyObject* block_forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (need == 0 || !workspace_for(a[2], a[3], need, c, &ws)) return nullptr;
     const fact_status_t st = without_gil(
         [&] { return fact_block_forward(c.h, desc, x->const_data_ptr(), out.t->data_ptr(), ws, need, c.stream); });
-    return st == FACT_OK ? out.result() : nullptr;
+    return c.answer(st, out);
   });
 }
 

@@ -99,6 +99,25 @@ def test_wrong_arguments_raise_what_they_raised(h):
     assert torch.isfinite(h.gemm(x, w, layout="NK").float()).all()
 
 
+def test_a_call_that_fails_after_a_launch_is_raised_not_repeated(h):
+    # the last linear layer of a block has misaligned weights: six kernels have been launched by then
+    from paper_2604_26666_b200.binding import FactError
+
+    C, ffn, T = 128, 256, 96
+    x = rnd(T, C)
+    w = {"norm1_gamma": rnd(C), "norm2_gamma": rnd(C), "wqkv": rnd(3 * C, C), "wo": rnd(C, C), "w1": rnd(ffn, C), "b1": rnd(ffn)}
+    good = h.block_desc("gpt", 1, T, 2, 2, 64, ffn, dict(w, w2=rnd(C, ffn)))
+    bad = h.block_desc("gpt", 1, T, 2, 2, 64, ffn, dict(w, w2=rnd(C * ffn + 1)[1:].view(C, ffn)))
+    h.block_forward(good, x)  # (the workspace has its size now)
+    n = h.launch_count()
+    h.block_forward(good, x)
+    seven = h.launch_count() - n
+    with pytest.raises(FactError, match="fact_block_forward"):
+        h.block_forward(bad, x)
+    assert h.launch_count() - n == 2 * seven - 1
+    assert torch.isfinite(h.block_forward(good, x).float()).all() and h.device_status() == 0
+
+
 def test_kept_choices_follow_the_table(h, tmp_path):
     M, N, K = 192, 256, 320
     x, w = rnd(M, K), rnd(N, K, scale=0.05)
