@@ -239,7 +239,7 @@ fact_status_t fact_gemm_batched(fact_handle_t handle, int64_t batch, int64_t M, 
  * tail of the same kernel (the grid never exceeds the SM count, so all CTAs are resident; the wait is
  * bounded like every other device wait) all threads share out the output and add the partials of
  * each element in a fixed order: L sums over slices q, q+L, q+2L, ... (ascending, q = 0..L-1; L = 4 up to 8 slices, else
- * a power of two up to 32 that shares the work out over the SMs), combined pairwise, ((s0 + s1) + (s2 + s3)) + ...; then the
+ * a power of two from 4 to 32 that shares the work out over the SMs), combined pairwise, ((s0 + s1) + (s2 + s3)) + ...; then the
  * epilogue and the store.  Slice boundaries and the order of every
  * addition depend only on (M, N, K, config), so repeated calls return bit-identical results.  Split-K
  * calls through one handle must be stream-ordered with respect to each other (they share the handle's

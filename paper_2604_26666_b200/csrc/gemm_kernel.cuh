@@ -607,13 +607,14 @@ constexpr int kReduceBatch = 10;
 
 // How many lanes share a group, for `threads` threads and `groups` groups of columns: as few passes of the threads over
 // the groups, and as few trips to L2 per pass, as possible.  (Four lanes always: 80 x 128 x 209992, 148 slices, kept 29 of
-// 148 CTAs busy for four trips; sixteen share it out in one: 25.8 -> 24.2 us, 79 x 160 x 83512 18.6 -> 16.6.)  Up to 8 slices
-// four lanes, the association of the wide walk below.
+// 148 CTAs busy for four trips; sixteen share it out in one: 25.8 -> 24.2 us, 79 x 160 x 83512 18.6 -> 16.6.)  Never fewer
+// than four: a lane's chain of additions, and its trips, get longer (256 x 256 x 131072, 37 slices: ten terms in one trip
+// by four lanes, nineteen in two by two).  Up to 8 slices four lanes, the association of the wide walk below.
 __host__ __device__ inline int reduce_lanes_log2(long long groups, long long threads, int splits, bool gate) {
   if (splits <= 8) return 2;
   int best = 2;
   long long best_cost = -1;
-  for (int l = 0; l <= 5; ++l) {
+  for (int l = 2; l <= 5; ++l) {
     const long long passes = ((groups << l) + threads - 1) / threads;
     const int loads = (splits + (1 << l) - 1) >> l;
     const long long cost = passes * (1200LL * ((loads + kReduceBatch - 1) / kReduceBatch) + 60LL * loads * (gate ? 2 : 1) + 60LL * l);
@@ -686,19 +687,18 @@ __device__ __forceinline__ void reduce_groups(const ReduceParams& p, long long f
         if (gate) up[j] += __shfl_xor_sync(0xffffffffu, up[j], o);
       }
     }
-    // lanes 0-3 of the group finish columns n .. n + 3 (or however many lanes there are, several columns each)
-    if (valid) {
-      for (int j = sub; j < nvalid; j += L) {
-        const float av = j == 0 ? a[0] : j == 1 ? a[1] : j == 2 ? a[2] : a[3];
-        const float uv = j == 0 ? up[0] : j == 1 ? up[1] : j == 2 ? up[2] : up[3];
-        const float bias = p.bias ? __bfloat162float(p.bias[n + j]) : 0.f;
-        const float res =
-            (p.epi == kEpiBiasResidual) ? __bfloat162float(p.R[(long long)b * p.strideR + (long long)m * p.ldr + n + j]) : 0.f;
-        const float y = reduce_epilogue(p.epi, av * p.alpha, uv * p.alpha, bias, res);
-        const long long off = (long long)b * p.strideC + (long long)m * p.ldc + n + j;
-        if (p.out_f32) reinterpret_cast<float*>(p.C)[off] = y;
-        else reinterpret_cast<__nv_bfloat16*>(p.C)[off] = __float2bfloat16_rn(y);
-      }
+    // lanes 0-3 of the group finish columns n .. n + 3
+    if (valid && sub < nvalid) {
+      const int j = sub;
+      const float av = j == 0 ? a[0] : j == 1 ? a[1] : j == 2 ? a[2] : a[3];
+      const float uv = j == 0 ? up[0] : j == 1 ? up[1] : j == 2 ? up[2] : up[3];
+      const float bias = p.bias ? __bfloat162float(p.bias[n + j]) : 0.f;
+      const float res =
+          (p.epi == kEpiBiasResidual) ? __bfloat162float(p.R[(long long)b * p.strideR + (long long)m * p.ldr + n + j]) : 0.f;
+      const float y = reduce_epilogue(p.epi, av * p.alpha, uv * p.alpha, bias, res);
+      const long long off = (long long)b * p.strideC + (long long)m * p.ldc + n + j;
+      if (p.out_f32) reinterpret_cast<float*>(p.C)[off] = y;
+      else reinterpret_cast<__nv_bfloat16*>(p.C)[off] = __float2bfloat16_rn(y);
     }
   }
 }
