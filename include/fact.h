@@ -165,7 +165,9 @@ typedef enum {
  *                tile_n (16, 32 or 64; 32 or 64 for FACT_B_KN) weight rows and all of K per CTA, tile_m the rows rounded
  *                up to 8, 16, 32 or 64; no workspace.  BF16 operands of fact_gemm / fact_linear (not the row softmax,
  *                row sums, a folded normalisation or SILU_GATE with FACT_B_KN: FACT_ERR_UNSUPPORTED).  An untuned call
- *                of at most 64 rows takes it on its own. */
+ *                of at most 64 rows takes it on its own unless K slices (few columns, a long K) or wide tiles (many
+ *                columns and more than 16 rows) are expected to be faster, and instead of K slices if it brings no
+ *                workspace for them. */
 typedef struct {
   int tile_m, tile_n, tile_k, stages, cta_group, raster_group, split_k, store_mode, schedule;
 } fact_config_t;

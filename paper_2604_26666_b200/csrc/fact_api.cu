@@ -358,6 +358,31 @@ int skinny_rows(fact_handle_t h, const Problem& q) {
   if (q.layout == FACT_B_NK && nw <= 16LL * h->sm_count) return 16;
   return nw <= 64LL * h->sm_count ? 32 : 64;
 }
+// Whether the few-rows kernel is done before the tile kernels would be.  It never cuts K: a CTA takes `per_k` ns for every k
+// (the serial walk of its ring), where all CTAs together wait for HBM it is `stream`; the tile kernels cut K where there are
+// few tiles, and pay about 6 us (`fixed`) for adding the slices up.  Timed over 1-64 rows, 64-28672 columns, K 256-131072,
+// few rows / tiles in us: 8 rows, 64 columns, K 4096 5.9 / 8.1, 8192 9.8 / 7.7, 131072 125 / 11.4; 2048 columns, K 14336 16.7 /
+// 18.0, 32768 35.1 / 31.2; 4096 columns, K 14336 20.7 / 28.1; 64 rows, 64 columns, K 4096 7.9 / 8.1, 8192 13.6 / 8.6.  Within
+// 5 % of the better one but for 256 columns x K 8192 (9.4 / 11.7).
+// The rows' own traffic from L2 decides where there are several waves of CTAs: above 32 rows from 40 columns per SM on (64 x
+// 8192 -> 8192 32.0 / 30.3), above 16 from 128 (32 x 256 -> 28672 8.9 / 6.9), above 8 for [K, N] weights (16 x 4096 -> 28672
+// 40.7 / 39.1).
+bool skinny_wins(fact_handle_t h, const Problem& q) {
+  const double nw = (double)q.Nw(), sms = h->sm_count;
+  const bool kn = q.layout == FACT_B_KN;
+  if (nw > 40.0 * sms && q.M > 32) return false;
+  if (nw > 128.0 * sms && (q.M > 16 || (q.M > 8 && kn && q.K >= 2048))) return false;
+  const double stream = 2.0 * nw / 6400.0;
+  double per_k, fixed;
+  if (q.M > 32) {
+    per_k = kn ? 1.4 : (nw <= 16.0 * sms ? 1.42 : 2.0);
+    fixed = 5800.0;
+  } else {
+    per_k = kn ? (q.M <= 16 ? 0.72 : 0.88) : 0.96;
+    fixed = (kn ? 5600.0 : 6200.0) + nw;
+  }
+  return (double)q.K * (per_k - stream) <= fixed;
+}
 int skinny_groups(const Problem& q) { return q.M <= 8 ? 1 : (q.M <= 16 ? 2 : (q.M <= 32 ? 4 : 8)); }
 uint32_t skinny_stage_bytes(int rows, int groups) {
   return (uint32_t)(rows + 8 * groups <= 64 ? 4 : 2) * 128u * (uint32_t)(rows + 8 * groups);
@@ -385,10 +410,8 @@ fact_status_t resolve_config_uncached(fact_handle_t h, const Problem& q, const f
   }
   if (from_table_out) *from_table_out = from_table;
   if (splits_override > 0) c.split_k = splits_override;
-  // At most 64 rows: the kernel that streams the weights.  Above 32 rows and several waves of CTAs the rows' own traffic
-  // from L2 costs more than the tile kernels' padding (64 rows, 4096 -> 2 x 14336: 55.0 us against 43.5).
-  if (c.schedule == 4 || (user == nullptr && !from_table && splits_override == 0 && skinny_ok(q) &&
-                          !(q.M > 32 && q.Nw() > 64LL * h->sm_count))) {
+  // At most 64 rows: the kernel that streams the weights, where it is the faster one.
+  if (c.schedule == 4 || (user == nullptr && !from_table && splits_override == 0 && skinny_ok(q) && skinny_wins(h, q))) {
     if (!skinny_ok(q) || c.split_k > 1 || c.split_k < 0 || (c.store_mode != 0 && c.store_mode != 1)) return FACT_ERR_UNSUPPORTED;
     const int rows = c.tile_n ? c.tile_n : skinny_rows(h, q), groups = skinny_groups(q);
     if ((rows != 16 && rows != 32 && rows != 64) || (rows == 16 && q.layout == FACT_B_KN)) return FACT_ERR_UNSUPPORTED;
@@ -1146,11 +1169,6 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
   if (cudaGetDevice(&dev) != cudaSuccess) return FACT_ERR_CUDA;
   if (dev != h->device && cudaSetDevice(h->device) != cudaSuccess) return FACT_ERR_CUDA;
 
-  if (plan.skinny) {
-    st = launch_skinny(h, q, plan, stream);
-    if (dev != h->device) cudaSetDevice(dev);
-    return st;
-  }
   std::vector<int> group_table;  // more than kParamGroups groups: goes to the handle's device buffer in stream order
   GroupTable group_param;
   if (q.groups > 0) {
@@ -1216,16 +1234,22 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
   if (plan.cfg.split_k > 1 && !plan.kcluster && (plan.from_table || !user || user->split_k == 0) && splits_override == 0 &&
       q.op != FACT_OP_GEMM_SPLITK && (!ws || ws_bytes < plan.ws_bytes || !aligned16(ws))) {
     // K slices from the tuner's table or the library's own model, but this caller brought no (or too little)
-    // scratch: one slice
+    // scratch: one slice, or the kernel that needs none
     fact_config_t dp = plan.cfg;
     if (!plan.from_table) {  // the model's choice: choose the tiles again, for one slice
       memset(&dp, 0, sizeof dp);
       if (user) dp = *user;
+      else if (skinny_ok(q)) dp.schedule = 4;
     }
     dp.split_k = 1;
     dp.store_mode = plan.from_table ? 0 : dp.store_mode;
     st = make_plan(h, q, &dp, 0, &plan);
     if (st != FACT_OK) return st;
+  }
+  if (plan.skinny) {
+    st = launch_skinny(h, q, plan, stream);
+    if (dev != h->device) cudaSetDevice(dev);
+    return st;
   }
   if (q.K == 0 && q.epi == FACT_EPI_BIAS_SOFTMAX) return FACT_ERR_UNSUPPORTED;  // (the stand-alone epilogue has no softmax)
   if (q.K == 0) {  // empty sum: the epilogue of a zero accumulator

@@ -88,3 +88,25 @@ def test_a_tuned_entry_is_for_plain_calls_only(h, tmp_path):  # noqa: F811
         assert (t.linear_grouped(X, W.expand(3, N, K).contiguous(), [3, 0, 5]) == K).all()
         assert t.device_status() == 0
         t.close()
+
+
+@pytest.mark.parametrize("layout", ["NK", "KN"])
+@pytest.mark.parametrize("M,N,K,few", [(8, 64, 4096, True), (8, 64, 16384, False), (64, 64, 131072, False), (1, 512, 32768, False),
+                                       (16, 2048, 14336, True), (64, 4096, 4096, True), (64, 8192, 1024, False),
+                                       (32, 28672, 256, False), (8, 28672, 256, True)])
+def test_long_k_of_few_columns_is_cut_into_slices(h, layout, M, N, K, few):  # noqa: F811
+    """One CTA's walk over all of K is not what a few columns wait for; a call without scratch has no slices to take."""
+    from paper_2604_26666_b200 import binding as bd
+
+    case = mk("few_long", M, N, K, op="gemm", layout=layout, out="f32")
+    ins = small_int_inputs(case, 9, lo=-2, hi=2)
+    c = h.get_config("gemm", 1, M, N, K, layout=layout, out_dtype=torch.float32)
+    assert (c.schedule == 4) == few
+    X, W = ins.X.cuda(), ins.W.cuda()
+    want = (ins.X.float() @ (ins.W if layout == "KN" else ins.W.t()).float())  # (exact: integers below 2^24)
+    assert torch.equal(h.gemm(X, W, layout=layout, out_dtype=torch.float32).cpu(), want)
+    out = torch.empty(M, N, dtype=torch.float32, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    assert bd.lib().fact_gemm(h._h, M, N, K, X.data_ptr(), K, W.data_ptr(), W.stride(0), bd.LAYOUTS[layout], out.data_ptr(), N,
+                              1, None, None, 0, s) == 0
+    assert torch.equal(out.cpu(), want) and h.device_status() == 0
