@@ -2385,6 +2385,50 @@ fact_status_t encode_map_bthd(fact_handle_t h, CUtensorMap* map, const void* bas
   return FACT_OK;
 }
 
+// CTAs (a cluster) per problem of the few-rows kernel.  More of them only where they have SMs of their own, with the large
+// ring: three quarters of the SMs is what clusters of 8 can fill at once (15 of them; at 16 the sixteenth is a second wave:
+// 21.2 us instead of 14.1 with clusters of 4 for 2 sequences x 8192 keys x 8 heads of 128).  The cluster's merge costs as much
+// as about six blocks (1.2 us): 260 keys 3.6 us in one CTA, 4.3 in two; 1000 keys 6.3 / 5.6 / 4.7 / 4.5 in 1 / 2 / 4 / 8; 8192
+// keys 36.2 / 21.0 / 13.0 / 9.7.  A head alone on an SM streams 64 keys in 0.27 us with the large ring, 0.36 with the small.
+int decode_splits(fact_handle_t h, long long pairs, long long seq_kv) {
+  int splits = 1;
+  if ((seq_kv + kDecBlockK - 1) / kDecBlockK >= 12)
+    while (splits < 8 && 2 * pairs * splits <= h->sm_count * 3 / 4) splits *= 2;
+  return splits;
+}
+
+// Whether the few-rows kernel is done before the tile kernels would be.  It reads the keys of a group of query heads once and
+// cuts them over CTAs where there are few problems; against that a CTA of it has a start and a merge of its own (2 us above 16
+// rows, where one CTA fills an SM), which many problems of few keys pay again and again: 1024 sequences x 32 queries x 16 keys x
+// 12 heads of 64 333 us against 86, 256 x 12 x 64 34.2 / 21.7, 64 x 32 x 256 35.5 / 18.1, 64 x 1 x 64 8.1 / 8.3; four query heads
+// a key head, 64 x 8 x 64 of 128 23.9 / 20.1, 64 x 8 x 256 35.9 / 44.8, one query row each always here (64 x 1 x 16 5.6 / 19.9).
+// Microseconds of a first round over the SMs and of each further one, constant and per key, fitted to 1367 timed calls (1-32
+// rows, 16-4096 keys, 1-1024 sequences of 8, 12 and 32 heads): at most 14 % from the better kernel, 0.1 % in the mean.
+bool decode_wins(fact_handle_t h, int head_dim, long long rows, long long pairs, long long heads, long long seq_kv) {
+  if (decode_splits(h, pairs, seq_kv) > 1) return true;
+  struct Cost {
+    double first, first_key, more, more_key, hbm, hbm_key;
+  };
+  static const Cost few[2][3] = {{{2.2, .0031, 1.0, .0037, .3, .0062}, {2.8, .0039, 1.4, .0040, .5, .0065}, {0., .0062, 3.6, .0108, 0., 0.}},
+                                 {{2.6, .0042, 1.3, .0060, .4, .0125}, {3.5, .0060, 2.0, .0062, .6, .0130}, {0., .0118, 5.6, .0135, 0., 0.}}};
+  const double k = (double)seq_kv;
+  const bool wide = head_dim == 128, shared = heads > pairs;  // shared: several query heads read a key head, from L2
+  const Cost& c = few[wide][rows <= 8 ? 0 : (rows <= 16 ? 1 : 2)];
+  const double start = rows <= 16 ? c.first : (wide ? 3.5 + .068 * (double)rows : 2.75 + .042 * (double)rows);
+  double tile_first, tile_more;
+  if (wide) {
+    tile_first = std::max(5.4, 3.6 + .0125 * k);
+    tile_more = shared ? std::max(1.15, .2 + .0105 * k) : std::max(1.2, .4 + .0165 * k);
+  } else {
+    tile_first = std::max(4.6, 3.3 + .0079 * k);
+    tile_more = k <= 64. ? (shared ? .8 : .87) : (shared ? .6 + .006 * k : .65 + .0075 * k);
+  }
+  const long long sms = h->sm_count;
+  const double t_few = start + c.first_key * k + (double)((pairs + sms - 1) / sms - 1) * std::max(c.more + c.more_key * k, c.hbm + c.hbm_key * k);
+  const double t_tiles = tile_first + (double)((heads + sms - 1) / sms - 1) * tile_more;
+  return t_few <= 1.05 * t_tiles;
+}
+
 // Attention of few query rows (attention_decode_kernel.cuh).  `strides`: batch, token and head of Q, K, V, O.
 fact_status_t attention_decode(fact_handle_t h, int64_t batch, int64_t seq_q, int64_t seq_kv, int64_t heads_q, int64_t heads_kv,
                                int64_t head_dim, const void* Q, const int64_t (&strides)[12], const void* K, const void* V,
@@ -2414,15 +2458,7 @@ fact_status_t attention_decode(fact_handle_t h, int64_t batch, int64_t seq_q, in
   p.scale_log2 = (float)((scale > 0.f ? (double)scale : 1.0 / std::sqrt((double)head_dim)) * 1.4426950408889634);
   p.status = h->d_status;
   const long long pairs = (long long)batch * heads_kv;
-  const long long blocks = (seq_kv + kDecBlockK - 1) / kDecBlockK;
-  // CTAs per problem.  More of them only where they have SMs of their own, with the large ring: three quarters of the
-  // SMs is what clusters of 8 can fill at once (15 of them; at 16 the sixteenth is a second wave: 21.2 us instead of 14.1
-  // with clusters of 4 for 2 sequences x 8192 keys x 8 heads of 128).  The cluster's merge costs as much as about six
-  // blocks (1.2 us): 260 keys 3.6 us in one CTA, 4.3 in two; 1000 keys 6.3 / 5.6 / 4.7 / 4.5 in 1 / 2 / 4 / 8; 8192 keys
-  // 36.2 / 21.0 / 13.0 / 9.7.  A head alone on an SM streams 64 keys in 0.27 us with the large ring, 0.36 with the small.
-  p.splits = 1;
-  if (blocks >= 12)
-    while (p.splits < 8 && 2 * pairs * p.splits <= h->sm_count * 3 / 4) p.splits *= 2;
+  p.splits = decode_splits(h, pairs, seq_kv);
   const uint32_t ring = pairs * p.splits <= h->sm_count ? 2 * kDecRingBytes : kDecRingBytes;
   p.stages = (int)(ring / dec_stage_bytes((int)head_dim));
   if (pairs * p.splits > 0x7fffffffLL) return FACT_ERR_UNSUPPORTED;
@@ -2475,8 +2511,10 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return FACT_ERR_CUDA;
   if (dev != h->device && cudaSetDevice(h->device) != cudaSuccess) return FACT_ERR_CUDA;
-  // Few query rows per key/value head: the kernel that streams the keys once for all of them.
-  if ((!causal || seq_kv == 1) && seq_q * (heads_q / heads_kv) <= kDecMaxRows) {
+  // Few query rows per key/value head: the kernel that streams the keys once for all of them, where it is the faster one.
+  const int64_t rows = seq_q * (heads_q / heads_kv);
+  if ((!causal || seq_kv == 1) && rows <= kDecMaxRows &&
+      decode_wins(h, (int)head_dim, rows, batch * heads_kv, batch * heads_q, seq_kv)) {
     const fact_status_t ds = attention_decode(h, batch, seq_q, seq_kv, heads_q, heads_kv, head_dim, Q, strides, K, V, O, scale, stream);
     if (dev != h->device) cudaSetDevice(dev);
     return ds;

@@ -42,3 +42,17 @@ def test_views_large_scores_and_repeatability(h, D):  # noqa: F811
     c, t = attention_gates(q, k, v, False, to_f64(wide[:, :, :Hq]))
     # (values of size 6: the contract's absolute 1e-2 is meant for unit variance, the tight gate is the derived one)
     assert t <= 1.0, (c, t)
+
+
+# many problems of few keys go to the tile kernels: a query row's bits are then those of a call with more rows than the
+# few-rows kernel takes (every head size's kernels: two and three tiles an SM, halves, pairs of heads)
+@pytest.mark.parametrize("B,Tq,Tk,Hq,Hkv,D", [(40, 32, 40, 12, 12, 64), (64, 17, 256, 12, 12, 64), (300, 1, 64, 12, 12, 64),
+                                              (256, 8, 33, 8, 2, 64), (40, 32, 16, 12, 12, 128), (64, 20, 130, 8, 8, 128),
+                                              (64, 8, 64, 32, 8, 128), (3, 32, 200, 32, 32, 128)])
+def test_many_problems_of_few_keys_go_to_the_tiles(h, B, Tq, Tk, Hq, Hkv, D):  # noqa: F811
+    q, k, v = rnd((B, 33, Hq, D), 36), rnd((B, Tk, Hkv, D), 37), rnd((B, Tk, Hkv, D), 38)
+    few = h.attention(q[:, :Tq].contiguous().cuda(), k.cuda(), v.cuda(), causal=False)
+    more = h.attention(q.cuda(), k.cuda(), v.cuda(), causal=False)
+    assert h.device_status() == 0 and torch.equal(few, more[:, :Tq])
+    c, t = attention_gates(q[:4, :Tq], k[:4], v[:4], False, to_f64(few[:4]))
+    assert c <= 1.0 and t <= 1.0, (c, t)
