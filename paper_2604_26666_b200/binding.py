@@ -17,6 +17,7 @@ from __future__ import annotations
 import ctypes
 import importlib.machinery
 import importlib.util
+import warnings
 from ctypes import POINTER, Structure, byref, c_char_p, c_double, c_float, c_int, c_int64, c_size_t, c_void_p
 from pathlib import Path
 from typing import Optional
@@ -192,18 +193,33 @@ def lib() -> ctypes.CDLL:
 _bind = None
 
 
+class _CtypesOnly:
+    """In the place of an extension that cannot be used: it takes no call, and all are marshalled through ctypes."""
+
+    matmul = linear = attention = norm = block_forward = staticmethod(lambda *args: None)
+
+
 def bind():
-    """The extension that marshals ordinary calls (built in-tree with libfact.so)."""
+    """The extension that marshals ordinary calls (built in-tree with libfact.so).  A call needs it for its speed only: where
+    it is missing or was built for something else, a warning says so and ctypes serves every call."""
     global _bind
     if _bind is None:
+        from . import build
+
         lib()
-        path = _PKG / "_fact_bind.so"
-        if not path.exists():
-            raise RuntimeError(f"{path} is missing: build it with `python -m paper_2604_26666_b200.build`")
-        loader = importlib.machinery.ExtensionFileLoader("_fact_bind", str(path))
-        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fact_bind", loader))
-        loader.exec_module(module)
-        _bind = module
+        why = build.bind_problem()
+        if why is None:
+            try:
+                loader = importlib.machinery.ExtensionFileLoader("_fact_bind", str(build.BIND_LIB))
+                module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fact_bind", loader))
+                loader.exec_module(module)
+                _bind = module
+            except ImportError as e:
+                why = str(e)
+        if _bind is None:
+            warnings.warn(f"{why}: calls go through ctypes and cost the host 10-15 us more each (build it with "
+                          "`python -m paper_2604_26666_b200.build`)", RuntimeWarning, stacklevel=2)
+            _bind = _CtypesOnly()
     return _bind
 
 

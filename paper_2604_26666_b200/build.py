@@ -108,6 +108,15 @@ def build_bind(force: bool = False) -> Path:
     return BIND_LIB
 
 
+def bind_problem():
+    """Why the extension in the tree cannot be used, or None."""
+    if not BIND_LIB.exists():
+        return f"{BIND_LIB} is missing"
+    if BIND_STAMP.exists() and BIND_SOURCE.exists() and BIND_STAMP.read_text().strip() != bind_hash():
+        return f"{BIND_LIB} was built from other sources, or for another torch or Python"
+    return None
+
+
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="--verbose" in sys.argv))
     print(build_bind(force="--force" in sys.argv))

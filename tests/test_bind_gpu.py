@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 def h():
     from paper_2604_26666_b200.binding import Handle
     hd = Handle(0)
+    assert hd._bind.__name__ == "_fact_bind"  # (the tree's extension is current and in use)
     yield hd
     hd.close()
 

@@ -280,3 +280,24 @@ def test_attention_deal_argument_errors(libfact):
     assert libfact.fact_attention_deal(4, 4, 512, 64, 4, 4, buf, ctypes.byref(n)) == 1
     assert libfact.fact_attention_deal(4, 4, 512, 64, 0, 4, buf, None) == 1
     assert libfact.fact_attention_deal(148, 10000, 512, 64, 0, 4, buf, ctypes.byref(n)) == 3  # more than 8192 items
+
+
+def test_an_extension_that_is_missing_or_stale_leaves_the_calls_to_ctypes(libfact, monkeypatch, tmp_path):
+    from paper_2604_26666_b200 import binding, build
+
+    def used():
+        monkeypatch.setattr(binding, "_bind", None)
+        return binding.bind()
+
+    build.build_bind()
+    assert build.bind_problem() is None and used().__name__ == "_fact_bind"
+    (tmp_path / "stamp").write_text("of other sources\n")
+    (tmp_path / "not_a_library.so").write_text("")
+    for stamp, so in ((tmp_path / "stamp", build.BIND_LIB), (build.BIND_STAMP, tmp_path / "none.so"),
+                      (build.BIND_STAMP, tmp_path / "not_a_library.so")):
+        with monkeypatch.context() as m:
+            m.setattr(build, "BIND_STAMP", stamp)
+            m.setattr(build, "BIND_LIB", so)
+            with pytest.warns(RuntimeWarning, match="ctypes"):
+                b = used()
+            assert all(f(1, 2, 3) is None for f in (b.matmul, b.linear, b.attention, b.norm, b.block_forward))
