@@ -1423,7 +1423,10 @@ void build_attention_tiles_deal(int G, int pipes, int bk, long long bh, int q_ti
 //  - causal: a pair's first tile waits out the blocks that only its second sees.  Three from one and a half tiles an SM on
 //    for short sequences and three for long (16 x 1000 53.4 / 53.4 / 45.5, 128 x 512 128 / 133 / 113, 10 x 256 8.4 / 7.5 /
 //    7.2), two below that, where a tile is mostly alone on its SM and blocks of 128 keys get it done sooner (1 x 4096
-//    55.6 / 48.8 / 53.7, 1 x 1500 23.0 / 17.5 / 21.0).
+//    55.6 / 48.8 / 53.7, 1 x 1500 23.0 / 17.5 / 21.0).  From 32 tiles an SM on, where the keys no longer stay in L2 between
+//    the tiles of a head and the host no longer deals, pairs again: calls back to back 130 x 1000 443 / 497 / 509, 65 x 2000
+//    757 / 866 / 879, 16 x 8192 2585 / 2915 / 2913 (16 x 4096, 42 an SM, 670 / 730 / 682; 8 x 4096, 21 an SM, 325 / 335 / 320)
+//    -- but not where the blocks that a pair computes for nothing are a quarter of its work: 217 x 300 197 / 157 / 152.
 //  - full: pairs load their keys once for two tiles and are the best where both are busy (16 x 1024 81.9 / 87.1 / 85.4, 128
 //    x 512 151 / 186 / 189); tiles where items of 256 rows leave a sixth of the SMs' time or more empty (1 x 1000 18.4 /
 //    13.5 / 15.9, 40 x 384 45.0 / 38.3 / 41.3, 16 x 300 22.5 / 17.8 / 17.4; three a SM exactly: 1 x 4096 104 / 95.6 / 81.2).
@@ -1431,7 +1434,13 @@ int attention_tiles_choice(long long q_tiles, long long bh, long long seq_kv, bo
   const long long items = q_tiles * bh;
   if (items > 0x7fffffffLL) return 0;
   if (q_tiles == 1) return items <= sms ? 2 : (seq_kv <= AttnTiles<3>::kBlockK ? 3 : 0);
-  if (causal) return items >= 3 * sms || (q_tiles <= 4 && 2 * items >= 3 * sms) ? 3 : 2;
+  if (causal) {
+    // blocks of 128 x 128 that a head's pairs go through, two tiles at a time, and those that its tiles see
+    const long long pairs = (q_tiles + 1) / 2;
+    const long long in_pairs = 2 * (q_tiles % 2 ? pairs * (pairs - 1) + q_tiles : pairs * (pairs + 1)), seen = q_tiles * (q_tiles + 1) / 2;
+    if (items >= 32 * sms && 100 * seen > 76 * in_pairs) return 0;
+    return items >= 3 * sms || (q_tiles <= 4 && 2 * items >= 3 * sms) ? 3 : 2;
+  }
   const long long tiles_each = (items + sms - 1) / sms;
   const long long as_pairs = 2 * (((q_tiles + 1) / 2 * bh + sms - 1) / sms);
   if (5 * as_pairs < 6 * tiles_each) return 0;
@@ -2580,7 +2589,7 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     const int smem = std::max((int)attn_smem_bytes(p.D), kMinSmemRequest);
     typedef void (*Plain)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams, AttnNoDeal);
     typedef void (*Dealt)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams, AttnDeal);
-    // (head_dim 64: neither causal problems of more than a tile nor one head per item, see attention_tiles_choice)
+    // (head_dim 64: neither causal problems of few rounds nor one head per item, see attention_tiles_choice)
     static const Plain plain[2][3] = {{fact_attention_kernel<64, false, kAttnRows>, fact_attention_kernel<64, false, kAttnPair>, nullptr},
                                       {fact_attention_kernel<128, false, kAttnRows>, fact_attention_kernel<128, false, kAttnPair>,
                                        fact_attention_kernel<128, false, kAttnHalf>}};

@@ -4,7 +4,8 @@ import numpy as np
 import pytest
 import torch
 
-from tests.test_attention_gpu import check, h, rnd  # noqa: F401
+from tests.helpers import to_f64
+from tests.test_attention_gpu import attention_gates, check, h, rnd  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -76,3 +77,15 @@ def test_after_stream_k_products_on_the_same_handle():
     for B in (1, 16):
         check(hd, rnd((B, 300, 12, 64), 81), rnd((B, 300, 12, 64), 82), rnd((B, 300, 12, 64), 83), True, rows=rows_of(300))
     hd.close()
+
+
+@pytest.mark.parametrize("B,T,Hq,Hkv", [(50, 1000, 12, 12), (160, 400, 8, 2), (20, 2048, 15, 5)])
+def test_long_causal_runs_go_in_pairs(h, B, T, Hq, Hkv):  # noqa: F811
+    """From 32 tiles an SM on two tiles share their keys.  The last query sees every key with and without the mask: its bits
+    are those of the call without, which goes in pairs at this size (blocks of 128 keys; single tiles take 64)."""
+    q, k, v = rnd((B, T, Hq, 64), 71).cuda(), rnd((B, T, Hkv, 64), 72).cuda(), rnd((B, T, Hkv, 64), 73).cuda()
+    out = h.attention(q, k, v, causal=True)
+    assert torch.equal(out[:, -1], h.attention(q, k, v, causal=False)[:, -1]) and h.device_status() == 0
+    some = [0, B - 1]
+    c, t = attention_gates(q[some].cpu(), k[some].cpu(), v[some].cpu(), True, to_f64(out[some][:, rows_of(T)]), rows=rows_of(T))
+    assert c <= 1.0 and t <= 1.0, (c, t)
