@@ -39,7 +39,7 @@ struct DecodeParams {
   int Tq, Tk, Hkv, group, rows;  // rows = Tq * group; row r is query position r / group, head kvh * group + r % group
   int stages;                    // of the ring
   int splits;                    // CTAs (a cluster) per (batch, key/value head)
-  int k_each, v_each;            // 1; 0 where all batch entries share one K or V
+  int k_each, v_each;            // mask of the batch coordinate: all ones; 0 where all entries share one K or V
   float scale_log2;
   int* status;
 };
@@ -114,10 +114,10 @@ __global__ void __launch_bounds__(kDecThreads, NT <= 2 ? 2 : 1)
         ptx::mbar_arrive_expect_tx(full_bar(s), dec_stage_bytes(HD));
 #pragma unroll
         for (int c = 0; c < HD / 64; ++c)
-          ptx::tma_load_4d(dst + (uint32_t)c * chunk_bytes, &tmK, full_bar(s), c * 64, kvh, j * kDecBlockK, b * p.k_each);
+          ptx::tma_load_4d(dst + (uint32_t)c * chunk_bytes, &tmK, full_bar(s), c * 64, kvh, j * kDecBlockK, b & p.k_each);
 #pragma unroll
         for (int c = 0; c < HD / 64; ++c)
-          ptx::tma_load_4d(dst + kv_bytes + (uint32_t)c * chunk_bytes, &tmV, full_bar(s), c * 64, kvh, j * kDecBlockK, b * p.v_each);
+          ptx::tma_load_4d(dst + kv_bytes + (uint32_t)c * chunk_bytes, &tmV, full_bar(s), c * 64, kvh, j * kDecBlockK, b & p.v_each);
       }
       __syncwarp();
       if (++s == NS) {

@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
         if (c.n >= n_items) return;
         if (ptx::elect_one()) {
           ptx::mbar_arrive_expect_tx(bar(full + c.slot), L::kKvBytes);
-          ptx::tma_load_4d_hint(ring + (uint32_t)c.slot * L::kKvBytes, map, bar(full + c.slot), 0, c.it.kvh, c.j * BK, c.it.b * each, keep);
+          ptx::tma_load_4d_hint(ring + (uint32_t)c.slot * L::kKvBytes, map, bar(full + c.slot), 0, c.it.kvh, c.j * BK, c.it.b & each, keep);
         }
         __syncwarp();
         if (++c.slot == stages) c.slot = 0;
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
       auto load_q = [&](const AttnTile& it) {
         if (ptx::elect_one()) {
           ptx::mbar_arrive_expect_tx(bar(L::kQFull), L::kTileBytes);
-          ptx::tma_load_4d(q_s, &tmQ, bar(L::kQFull), 0, it.h, it.t0, it.b * p.q_each);
+          ptx::tma_load_4d(q_s, &tmQ, bar(L::kQFull), 0, it.h, it.t0, it.b & p.q_each);
         }
         __syncwarp();
       };

@@ -2462,8 +2462,8 @@ fact_status_t attention_decode(fact_handle_t h, int64_t batch, int64_t seq_q, in
   p.Hkv = (int)heads_kv;
   p.group = (int)(heads_q / heads_kv);
   p.rows = p.Tq * p.group;
-  p.k_each = strides[3] != 0;
-  p.v_each = strides[6] != 0;
+  p.k_each = strides[3] != 0 ? -1 : 0;
+  p.v_each = strides[6] != 0 ? -1 : 0;
   p.scale_log2 = (float)((scale > 0.f ? (double)scale : 1.0 / std::sqrt((double)head_dim)) * 1.4426950408889634);
   p.status = h->d_status;
   const long long pairs = (long long)batch * heads_kv;
@@ -2551,9 +2551,9 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     p.Hkv = (int)heads_kv;
     p.D = (int)head_dim;
     p.causal = causal != 0;
-    p.q_each = q_sb != 0;
-    p.k_each = k_sb != 0;
-    p.v_each = v_sb != 0;
+    p.q_each = q_sb != 0 ? -1 : 0;
+    p.k_each = k_sb != 0 ? -1 : 0;
+    p.v_each = v_sb != 0 ? -1 : 0;
     const double sc = scale > 0.f ? (double)scale : 1.0 / std::sqrt((double)head_dim);
     p.scale_log2 = (float)(sc * 1.4426950408889634);
     p.kmajor_desc = smem_desc_template(16, 1024);
