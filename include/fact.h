@@ -583,13 +583,21 @@ fact_status_t fact_selftest_wait_timeout(fact_handle_t handle, void* cuda_stream
 /* Diagnostic, host arithmetic only (no device is touched): the items CTA `cta` of `ctas` works through in a causal
  * fact_attention call of few rounds (more items than CTAs, fewer than 16 per CTA, at most 8192 items; other calls
  * deal the items out in closed form inside the kernel) whose items are pairs of tiles: head_dim 128.  (At head_dim 64
- * such calls hand out single tiles, three or two to a CTA at a time; the function shows the pairs there too.)  An item is 256 query rows of one (batch, head); item idx
- * is head idx % batch_heads and the (idx / batch_heads)-th pair of tiles counted from the END of the sequence, so
+ * such calls hand out single tiles, see below; the arithmetic of pairs is shown there too.)  An item is 256 query rows of
+ * one (batch, head); item idx is head idx % batch_heads and the (idx / batch_heads)-th pair of tiles counted from the END of the sequence, so
  * items come heaviest first.  The host gives each item, in that order, to the CTA whose items so far see the fewest
  * key blocks (plus a fixed cost per item; the lower CTA on a tie) and hands the list to the kernel as a parameter.
  * Writes at most max_items item numbers and their count to *n_items.  FACT_ERR_UNSUPPORTED above 8192 items. */
 fact_status_t fact_attention_deal(int ctas, int64_t batch_heads, int64_t seq, int head_dim, int cta, int max_items,
                                   int32_t* items, int* n_items);
+
+/* The same for causal calls at head_dim 64 whose CTAs work on `tiles` (3 or 2) tiles of 128 query rows at a time, each a
+ * pipeline with items of its own (fewer than 16 per pipeline, at most 8192 items): the items of pipeline `pipeline` of CTA
+ * `cta`.  Item idx is head idx % batch_heads and the (idx / batch_heads)-th tile counted from the end of the sequence; in
+ * that order the host gives each to the CTA whose items so far see the fewest key blocks (of 64 or 128 keys, plus a fixed
+ * cost per item; the lower CTA on a tie), and there to the pipeline with the fewest. */
+fact_status_t fact_attention_tiles_deal(int ctas, int64_t batch_heads, int64_t seq, int tiles, int cta, int pipeline,
+                                        int max_items, int32_t* items, int* n_items);
 
 /* Diagnostic, host arithmetic only (no device is touched): the stream-K schedule of one CTA group.  With
  * `sk_tiles` tiles of `k_blocks` k-blocks each shared out over `groups` CTA groups, writes the pieces group

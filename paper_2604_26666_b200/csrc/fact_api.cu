@@ -1625,6 +1625,22 @@ fact_status_t fact_attention_deal(int ctas, int64_t batch_heads, int64_t seq, in
   return FACT_OK;
 }
 
+fact_status_t fact_attention_tiles_deal(int ctas, int64_t batch_heads, int64_t seq, int tiles, int cta, int pipeline,
+                                        int max_items, int32_t* items, int* n_items) {
+  if (ctas < 1 || ctas > kAttnDealCtas || batch_heads < 1 || seq < 1 || (tiles != 2 && tiles != 3) || cta < 0 || cta >= ctas ||
+      pipeline < 0 || pipeline >= tiles || max_items < 0 || !n_items || (max_items > 0 && !items))
+    return FACT_ERR_INVALID_ARG;
+  const long long q_tiles = (seq + kAttnBlockQ - 1) / kAttnBlockQ;
+  if (q_tiles > kAttnDealItems || batch_heads > kAttnDealItems / q_tiles) return FACT_ERR_UNSUPPORTED;
+  std::unique_ptr<AttnTilesDeal> d(new AttnTilesDeal());
+  build_attention_tiles_deal(ctas, tiles, tiles == 3 ? AttnTiles<3>::kBlockK : AttnTiles<2>::kBlockK, batch_heads, (int)q_tiles, *d);
+  const int worker = pipeline * ctas + cta;
+  const int n = (int)d->off[worker + 1] - (int)d->off[worker];
+  *n_items = n;
+  for (int i = 0; i < n && i < max_items; ++i) items[i] = d->list[d->off[worker] + i];
+  return FACT_OK;
+}
+
 fact_status_t fact_stream_k_pieces(int groups, int64_t sk_tiles, int64_t k_blocks, int group, int max_pieces,
                                    int32_t* pieces, int* n_pieces) {
   if (groups < 1 || sk_tiles < 0 || k_blocks < 1 || group < 0 || group >= groups || max_pieces < 0 || !n_pieces ||

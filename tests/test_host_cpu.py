@@ -301,3 +301,36 @@ def test_an_extension_that_is_missing_or_stale_leaves_the_calls_to_ctypes(libfac
             with pytest.warns(RuntimeWarning, match="ctypes"):
                 b = used()
             assert all(f(1, 2, 3) is None for f in (b.matmul, b.linear, b.attention, b.norm, b.block_forward))
+
+
+@pytest.mark.parametrize("ctas,bh,seq,tiles", [(148, 192, 1000, 3), (148, 1536, 512, 3), (148, 12, 1500, 2), (148, 600, 256, 3),
+                                               (7, 5, 1500, 3), (148, 149, 300, 2), (3, 1, 2048, 2), (148, 64, 8192, 3)])
+def test_attention_tiles_deal_gives_every_tile_to_one_pipeline_and_balances_both(libfact, ctas, bh, seq, tiles):
+    """The deal that head_dim 64 hands to the kernel: every tile of every head once, heaviest first in every pipeline; no CTA
+    carries more than the mean plus one tile's weight, and no pipeline of a CTA more than its share plus one (what giving
+    each tile, heaviest first, to the one with the least so far guarantees)."""
+    from paper_2604_26666_b200.binding import attention_tiles_deal
+
+    bk, q_tiles = (64 if tiles == 3 else 128), -(-seq // 128)
+
+    def weight(idx):
+        return ((q_tiles - 1 - idx // bh) * 128 + 127) // bk + 1 + 64 // bk
+
+    per = [[attention_tiles_deal(ctas, bh, seq, tiles, c, t) for t in range(tiles)] for c in range(ctas)]
+    assert sorted(i for c in per for t in c for i in t) == list(range(bh * q_tiles))
+    loads = [[sum(map(weight, t)) for t in c] for c in per]
+    mean = sum(map(sum, loads)) / ctas
+    for c, own in zip(per, loads):
+        assert all(t == sorted(t) for t in c)
+        assert sum(own) <= mean + weight(0) and max(own) <= sum(own) / tiles + weight(0)
+
+
+def test_attention_tiles_deal_argument_errors(libfact):
+    import ctypes
+
+    n, buf = ctypes.c_int(0), (ctypes.c_int32 * 4)()
+    call = lambda *a: libfact.fact_attention_tiles_deal(*a, 4, buf, ctypes.byref(n))  # noqa: E731
+    assert call(148, 12, 512, 3, 0, 0) == 0
+    for bad in ((0, 4, 512, 3, 0, 0), (4, 4, 512, 1, 0, 0), (4, 4, 512, 3, 4, 0), (4, 4, 512, 2, 0, 2), (4, 0, 512, 2, 0, 0)):
+        assert call(*bad) == 1
+    assert call(148, 10000, 512, 3, 0, 0) == 3 and call(148, 1, 1 << 40, 3, 0, 0) == 3  # more than 8192 items
