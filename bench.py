@@ -8,9 +8,10 @@ and 8192^3, BF16 in, FP32 accumulate, BF16 out, operands N(0,1)/sqrt(K),
 seed 1).  The headline value is whole-job TFLOP/s (2 M N K per product,
 epilogue work not counted) with inputs resident in HBM; `e2e` repeats it with
 pinned-host inputs copied in and the result copied out inside the timed region.
-`shapes` adds, for every shape of the five configurations, its own time,
-TFLOP/s, GB/s and roofline fraction, next to a cuBLAS (torch.matmul) side
-reference that is never on the product path.
+The tables on stderr (`shapes` and others, a JSON line each) add, for every
+shape of the five configurations, its own time, TFLOP/s, GB/s and roofline
+fraction, next to a cuBLAS (torch.matmul) side reference that is never on the
+product path.
 
 With N > 1 (torchrun) every rank runs the same workload on its own GPU (the
 path shards by rows / batch entries with no exchange step): weak scaling, value
@@ -412,14 +413,13 @@ def main():
             "gpu_launches": launches, "debug_flags": h.debug_flags(),
             "clocks": dict(clocks, sm_mhz_in_dominant_kernel=(1e3 * k_cycles / k_ns if k_ns else None)),
             "cpu_baseline": cpu,
-            "shapes": shapes,
-            "attention": attention,
-            "fp8": fp8,
-            "grouped": grouped,
-            "norm_fold": norm_fold,
-            "blocks": blocks,
         }
-        print(json.dumps(line))
+        # the line is the headline alone: with the tables in it, it is 25 KB long, too long for what reads such lines
+        for name, table in (("shapes", shapes), ("attention", attention), ("fp8", fp8), ("grouped", grouped),
+                            ("norm_fold", norm_fold), ("blocks", blocks)):
+            if table:
+                print(json.dumps({name: table}), file=sys.stderr)
+        print(json.dumps(line), flush=True)
     if dist is not None:
         dist.destroy_process_group()
     h.close()
