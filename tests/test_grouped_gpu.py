@@ -198,21 +198,22 @@ def test_group_tables_as_a_parameter_and_in_device_memory(h, groups):
     """Up to 256 groups the table is a kernel parameter, beyond that it is copied to the device: the same sums (exact on
     integers) either way, some groups empty, the sizes different in consecutive calls on two streams."""
     g = torch.Generator().manual_seed(groups)
-    K, N = 72, 64
-    W = torch.randint(-2, 3, (groups, N, K), generator=g).to(torch.bfloat16)
+    K, N = 1032, 264
+    Wd = torch.randint(-2, 3, (groups, N, K), generator=g).to(torch.bfloat16).cuda()
     sides = [torch.cuda.Stream(), torch.cuda.Stream()] if groups <= 256 else [torch.cuda.current_stream()] * 2
-    Wd = W.cuda()
-    for turn in range(4):
-        rows = torch.randint(0, 9, (groups,), generator=g).tolist()
-        M = sum(rows)
-        X = torch.randint(-2, 3, (M, K), generator=g).to(torch.bfloat16)
-        Xd = X.cuda()
-        torch.cuda.synchronize()
+    rows = [torch.randint(0, 90, (groups,), generator=g).tolist() for _ in range(8)]
+    X = [torch.randint(-2, 3, (sum(r), K), generator=g).to(torch.bfloat16).cuda() for r in rows]
+    Y = [torch.full((sum(r), N), -7.0, dtype=torch.bfloat16, device="cuda") for r in rows]
+    torch.cuda.synchronize()
+    for turn in range(8):  # (nothing waits between the calls: those of the two streams overlap)
         with torch.cuda.stream(sides[turn % 2]):
-            y = h.linear_grouped(Xd, Wd, rows)
-        ref = torch.cat([x.double() @ W[i].double().t() for i, x in enumerate(X.split(rows))])
-        torch.cuda.synchronize()
-        assert torch.equal(y.cpu().double(), ref.to(torch.bfloat16).double())
+            h.linear_grouped(X[turn], Wd, rows[turn], out=Y[turn])
+    torch.cuda.synchronize()
+    for r, x, y in zip(rows, X, Y):
+        at = 0
+        for gi, n in enumerate(r):
+            assert torch.equal(y[at:at + n], (x[at:at + n].float() @ Wd[gi].float().t()).to(torch.bfloat16)), (gi, n)
+            at += n
     assert h.device_status() == 0
 
 
