@@ -681,6 +681,7 @@ int sk_tiles_for(fact_handle_t h, const Problem& q, const fact_config_t& c) {
   // the pieces are parked and finished by the staged epilogue, which stores whole 128-byte chunks per tile
   const bool f32 = q.out == FACT_OUT_F32;
   if (out_cols % (f32 ? 32 : 64) != 0 || (f32 && q.epi == FACT_EPI_BIAS_RESIDUAL) || c.store_mode == 1 || c.store_mode == 3) return 0;
+  if (q.N_out % (f32 ? 4 : 8) != 0) return 0;  // (its tensor stores write whole 16-byte pieces)
   const long long tiles = q.batch * ((q.M + c.tile_m - 1) / c.tile_m) * ((q.N_out + out_cols - 1) / out_cols);
   const long long groups = std::max(1, h->sm_count / c.cta_group);
   const long long k_blocks = (q.K + q.k_elems() - 1) / q.k_elems();

@@ -64,6 +64,9 @@ def test_batched_odd_strides_and_stream_k_choice(h):  # noqa: F811
     # a stream-K choice runs data-parallel for an output that tensor stores cannot address
     X, W = torch.ones(300, 1024, dtype=torch.bfloat16).cuda(), torch.ones(601, 1024, dtype=torch.bfloat16).cuda()
     assert (h.gemm(X, W, layout="NK", cfg={"split_k": -1}) == 1024.0).all()
+    # ... and asks for no scratch; an output of whole 16-byte pieces does
+    assert h.workspace_bytes("gemm", 1, 300, 601, 1024, "NONE", "NK", cfg={"split_k": -1}) == 0
+    assert h.workspace_bytes("gemm", 1, 300, 600, 1024, "NONE", "NK", cfg={"split_k": -1}) > 0
     assert h.device_status() == 0
 
 
