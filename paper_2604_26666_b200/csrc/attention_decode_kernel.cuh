@@ -14,8 +14,10 @@
 //     loop has no barrier among them.  Keys are the M dimension of both products (S^T = K Q^T, O^T = V^T P^T) and the
 //     8, 16 or 32 query rows the N dimension of mma.sync.m16n8k16: with M = 128 query rows, as tcgen05 wants them,
 //     the products would be padding, and the round trip of the scores through tensor memory would be a serial chain.
-// Measured (32 query / 8 key-value heads of 128, one query row per sequence, caches rotating through HBM; before -> now):
-// 32 sequences x 2000 keys 218 -> 39.3 us (6.7 TB/s), 7 x 276 17.1 -> 4 us; 25 x 4217 keys of 12 heads of 64 158 -> 49 us.
+// Measured (32 query / 8 key-value heads of 128, one query row per sequence, caches rotating through HBM; device time in a
+// train, the two-tile kernel -> this): 32 sequences x 2000 keys 218 -> 39.3 us, 7 x 276 17.1 -> 4; 25 x 4217 keys of 12 heads
+// of 64 158 -> 49.  A call of the first, one after another: 240 -> 40.4 us, 6.5 TB/s, the rate of a plain copy.  Calls of many
+// problems of few keys are faster on the tile kernels: decode_wins (fact_api.cu).
 // Masking only in the last block; probabilities are rounded to BF16 for the second product, sums are FP32 and taken
 // over the unrounded values, the reference maximum moves (and O is rescaled) only when a score exceeds it by more than
 // 8 in log2 units, as in the two-tile kernel.

@@ -11,9 +11,10 @@
 //   output each): three softmax warps per SM partition hide more of each other's latencies (score loads, maxima, hand-overs),
 //   and half of a causal tile's warps have nothing to do in its last block;
 //   two tiles, blocks of 128 keys: half the hand-overs per key, for problems too small to have three tiles on every SM.
-// Causal, 12 heads, microseconds, pairs -> this kernel: 16 x 1000 53.4 -> 45.5, 128 x 512 128 -> 113, 40 x 384 42.1 -> 27.6,
-// 16 x 300 19.9 -> 12.7, 8 x 4096 285 -> 266; two tiles: 1 x 1500 23.0 -> 17.5.  Which call takes what is in
-// attention_tiles_choice (fact_api.cu).  What is left: about 11 of 16 exponentials a cycle and SM within a block; about 2500
+// Causal, 12 heads, microseconds, pairs -> this kernel, short runs: 16 x 1000 53.4 -> 45.5, 40 x 384 42.1 -> 27.6, 16 x 300
+// 19.9 -> 12.7; two tiles: 1 x 1500 23.0 -> 17.5.  Calls back to back, at the clock that the power limit leaves: 16 x 1000
+// 55.3 -> 51.6, 8 x 4096 322 -> 316, 256 x 300 226 -> 175; from 32 tiles an SM on pairs are faster (128 x 1000 422 against 500).
+// Which call takes what is in attention_tiles_choice (fact_api.cu).  What is left: about 11 of 16 exponentials a cycle and SM within a block; about 2500
 // cycles per tile for its last product and its output, under which only the other pipelines run.
 // Tried and slower: two tiles in blocks of 64 keys with scores and probabilities double-buffered and the next block's
 // scores loaded under the exponentials (16 x 1024 full 99 us against 85, the loop is no longer one straight block).

@@ -1114,7 +1114,6 @@ fact_status_t launch_skinny(fact_handle_t h, const Problem& q, const Plan& plan,
   p.N = (int)q.N_out;
   p.K = (int)q.K;
   p.gate = gate;
-  p.b_kn = kn;
   p.stages = plan.cfg.stages;
   p.epi = (int)q.epi;
   p.out_f32 = q.out == FACT_OUT_F32;

@@ -23,7 +23,7 @@ struct NormParams {
   const __nv_bfloat16* gamma;  // [C]
   const __nv_bfloat16* beta;   // [C] or null
   long long M;
-  int C;                       // a multiple of 8, at most 256 * CH
+  int C;                       // a multiple of 8, at most 256 CH (a warp per row) or 8 T CH (a CTA of T threads)
   long long ldx, ldy;          // in elements, multiples of 8
   float eps;
 };
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kNormWarps * 32, 2) fact_norm_kernel(const Nor
 // The same with one CTA of T threads per row, CH chunks of 8 values per thread: for long rows, and for shorter ones where
 // there are few of them.  A warp that holds 4096 values has sixteen loads per lane to issue and add up before it can go on,
 // and a few rows are a few warps on one SM: 16 rows RMSNorm 6.9 -> 1.5 us, 4096 rows 15.4 -> 9.4, 32768 rows 94.3 -> 77.7
-// (6.9 TB/s); LayerNorm 7.5 -> 1.7, 17.2 -> 12.9 and 104.3 -> 94.5; 8192 values, 4096 rows 52.0 -> 19.8.  The gains and
+// (537 MB: 6.9 TB/s, a copy's 6.5 and what L2 still holds of the run before); LayerNorm 7.5 -> 1.7, 17.2 -> 12.9 and 104.3 -> 94.5; 8192 values, 4096 rows 52.0 -> 19.8.  The gains and
 // offsets are loaded with the row, so that one trip to memory serves both.
 template <int T, int CH, bool RMS>
 __global__ void __launch_bounds__(T, (CH <= 2 ? 1536 : 768) / T) fact_norm_long_kernel(const NormParams p) {

@@ -12,8 +12,8 @@
 //     tokens, in groups of 8, as the other: 64 tokens are 4 % of the tensor rate a tile kernel needs, and no
 //     accumulator has to travel through tensor memory;
 //   - the warps' sums are added up in a fixed order through shared memory, then the epilogue and the store.
-// Measured, weights rotating through HBM, the tile kernels' choice -> this: 16 x 4096 -> 4096 14.1 -> 7.8 us (HBM alone
-// 5.1), 1 x 4096 -> 6144 23.3 -> 10.1, 1 x 4096 -> 2 x 14336 gated 54.9 -> 37.2 (6.3 TB/s), 16 x 14336 -> 4096 28.7 ->
+// Measured, weights rotating through HBM, device time in a train, the tile kernels' choice -> this: 16 x 4096 -> 4096 14.1 ->
+// 7.8 us (HBM alone 5.2; a call one after another 17.8 -> 7.6, the host's share gone with it), 1 x 4096 -> 6144 23.3 -> 10.1, 1 x 4096 -> 2 x 14336 gated 54.9 -> 37.2 (6.3 TB/s), 16 x 14336 -> 4096 28.7 ->
 // 20.3, 16 x 768 -> 2304 6.9 -> 3.1.  (Sets of warps that take stages in turn, four steps each, were no faster.)
 #pragma once
 #include "gemm_kernel.cuh"
@@ -42,7 +42,7 @@ struct SkinnyShape {
 
 struct SkinnyParams {
   int M, N, K;        // N output columns
-  int gate, b_kn;
+  int gate;
   int stages;
   int epi, out_f32;
   void* C;
