@@ -1423,7 +1423,8 @@ void build_attention_tiles_deal(int G, int pipes, int bk, long long bh, int q_ti
 //  - causal: a pair's first tile waits out the blocks that only its second sees.  Three from one and a half tiles an SM on
 //    for short sequences and three for long (16 x 1000 53.4 / 53.4 / 45.5, 128 x 512 128 / 133 / 113, 10 x 256 8.4 / 7.5 /
 //    7.2), two below that, where a tile is mostly alone on its SM and blocks of 128 keys get it done sooner (1 x 4096
-//    55.6 / 48.8 / 53.7, 1 x 1500 23.0 / 17.5 / 21.0).  From 32 tiles an SM on, where the keys no longer stay in L2 between
+//    55.6 / 48.8 / 53.7, 1 x 1500 23.0 / 17.5 / 21.0).  From 32 tiles an SM on (48 below 8 tiles a
+//    sequence: 128 x 512, 41 an SM, 145.5 / 156.2 / 142.6), where the keys no longer stay in L2 between
 //    the tiles of a head and the host no longer deals, pairs again: calls back to back 130 x 1000 443 / 497 / 509, 65 x 2000
 //    757 / 866 / 879, 16 x 8192 2585 / 2915 / 2913 (16 x 4096, 42 an SM, 670 / 730 / 682; 8 x 4096, 21 an SM, 325 / 335 / 320)
 //    -- but not where the blocks that a pair computes for nothing are a quarter of its work: 217 x 300 197 / 157 / 152.
@@ -1438,7 +1439,7 @@ int attention_tiles_choice(long long q_tiles, long long bh, long long seq_kv, bo
     // blocks of 128 x 128 that a head's pairs go through, two tiles at a time, and those that its tiles see
     const long long pairs = (q_tiles + 1) / 2;
     const long long in_pairs = 2 * (q_tiles % 2 ? pairs * (pairs - 1) + q_tiles : pairs * (pairs + 1)), seen = q_tiles * (q_tiles + 1) / 2;
-    if (items >= 32 * sms && 100 * seen > 76 * in_pairs) return 0;
+    if (items >= (q_tiles >= 8 ? 32 : 48) * sms && 100 * seen > 76 * in_pairs) return 0;
     return items >= 3 * sms || (q_tiles <= 4 && 2 * items >= 3 * sms) ? 3 : 2;
   }
   const long long tiles_each = (items + sms - 1) / sms;
