@@ -583,7 +583,9 @@ fact_status_t fact_selftest_wait_timeout(fact_handle_t handle, void* cuda_stream
 /* Diagnostic, host arithmetic only (no device is touched): the items CTA `cta` of `ctas` works through in a causal
  * fact_attention call of few rounds (more items than CTAs, fewer than 16 per CTA, at most 8192 items; other calls
  * deal the items out in closed form inside the kernel) whose items are pairs of tiles: head_dim 128.  (At head_dim 64
- * such calls hand out single tiles, see below; the arithmetic of pairs is shown there too.)  An item is 256 query rows of
+ * such calls hand out single tiles, see below; the arithmetic of pairs is shown there too.  Calls whose keys and values exceed
+ * 48 MB take heads in chunks that stay in L2, in this order within each chunk; query heads that share a key/value head may go
+ * together as one head of as many more rows.)  An item is 256 query rows of
  * one (batch, head); item idx is head idx % batch_heads and the (idx / batch_heads)-th pair of tiles counted from the END of the sequence, so
  * items come heaviest first.  The host gives each item, in that order, to the CTA whose items so far see the fewest
  * key blocks (plus a fixed cost per item; the lower CTA on a tie) and hands the list to the kernel as a parameter.

@@ -51,16 +51,18 @@ constexpr int kAttnRegsAtLaunch = 168;
 static_assert(4 * kAttnRegsOther + 8 * kAttnRegsSoftmax <= 12 * kAttnRegsAtLaunch, "setmaxnreg requests exceed the pool");
 
 struct AttnParams {
-  int B, Tq, Tk, Hq, Hkv, D;  // D = 64 or 128
+  int B, Tq, Tk, Hq, Hkv;
+  int chunk;                  // heads (or groups of packed heads) whose items come before the next heads' (attn_item_place)
   int causal;
   float scale_log2;           // softmax scale * log2(e)
-  int q_pairs;                // ceil(Tq / 256)
+  int q_pairs;                // ceil(Tq / (2 * attn_tile_tokens)): ceil(Tq / 256) where no heads are packed
   int q_tiles;                // ceil(Tq / 128) (independent tiles, like the four below)
   int items;                  // work items, ordered heaviest first
   __nv_bfloat16* O;           // rows are stored from registers: batch, token and head strides in elements
   long long o_sb, o_st, o_sh;
   int o_vec32;                // rows of O start on 32 bytes
   int8_t q_each, k_each, v_each;  // mask of the batch coordinate: all ones; 0 where all entries share one Q, K or V
+  int8_t pack_log2;               // a tile's 128 rows are 128 >> pack_log2 tokens of 1 << pack_log2 query heads (paired tiles)
   uint64_t kmajor_desc;       // UMMA descriptor template, K-major 128B-swizzled tiles (Q, K)
   uint64_t v_desc;            // UMMA descriptor template, V as an N-major operand
   uint32_t idesc_s, idesc_pv;
@@ -70,6 +72,21 @@ struct AttnParams {
   int debug;                  // experiment switches, 0 in normal use: 8 no softmax arithmetic, 64 / 128 no first /
                               // second products (timing experiments; the output is then meaningless), 256 counters
 };
+
+// Query positions in a tile of 128 rows: row r holds token r >> pack_log2, head r & (pack - 1) of the group.
+__host__ __device__ inline int attn_tile_tokens(const AttnParams& p) { return kAttnBlockQ >> p.pack_log2; }
+
+// Item idx is the qr-th of its head's `per_head` items, of head bh: heads go in chunks, inside a chunk the heads fastest.
+// Causal items come heaviest first inside a chunk.  A chunk is as many heads as have their keys and values in L2 together,
+// so that the later items of a head find them there: 128 sequences x 512 x 12 heads of 64, causal, read their 201 MB of keys
+// and values 2.5 times over when every head's heaviest item came first.
+__device__ __forceinline__ void attn_item_place(int idx, int bh_count, int per_head, int chunk, int& bh, int& qr) {
+  const int first = chunk < bh_count ? idx / (chunk * per_head) * chunk : 0;
+  const int in = idx - first * per_head;
+  const int width = min(chunk, bh_count - first);
+  qr = in / width;
+  bh = first + in - qr * width;
+}
 
 // (The masks lie in what was padding.  With three words more the paired kernel's items of one key block take 2-3 % longer --
 // 64 x 500 queries x 50 keys x 12 heads of 64 40.2 -> 41.2 us -- although it reads no word of them then.)
@@ -117,7 +134,7 @@ __device__ __forceinline__ uint64_t attn_exp2_poly(uint64_t x2) {
 }
 
 struct AttnItem {
-  int b, h, kvh, t0;   // of tile 0 (tile 1: the same head 128 rows on, or, with two heads per item, b1, h1, kvh1 at row 0)
+  int b, h, kvh, t0;   // of tile 0 (tile 1: the same head a tile's tokens on, or, with two heads per item, b1, h1, kvh1 at row 0)
   int b1, h1, kvh1;
   int nb0, nb1;        // key blocks tile 0 / tile 1 see
   int nbi;             // key blocks the item loads
@@ -149,8 +166,8 @@ struct AttnDealArg<true> {
 //   kAttnRows   256 query rows of one head, as two tiles;
 //   kAttnPair   sequences of at most 128 queries, which fill one tile: two query heads, tile t the whole sequence of head
 //               2 i + t; the two tiles' key blocks alternate in the rings, each released by the one issuer that uses it;
-//   kAttnHalf   the same sequences where there are no more heads than SMs: one head, tile 0 only; tile 1 passes its
-//               hand-overs on and releases the blocks unused.
+//   kAttnHalf   no more tiles than SMs: one tile, tile 0 only; tile 1 passes its hand-overs on and releases the blocks
+//               unused (alone on its SM a tile is done sooner: q_pairs counts tiles here).
 // (As 256-row items such sequences computed a second tile of padding: 106 x 97 x 12 heads of 64 34.0 -> 19.3 us,
 // 256 x 64 x 12 73.2 -> 35.5, 60 x 128 x 32 heads of 128 50.5 -> 34.4 in pairs; 7 x 84 x 32 heads of 128 11.1 -> 8.4 as
 // halves.)
@@ -253,40 +270,45 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     n_items = (int)deal.off[blockIdx.x + 1] - deal_first;
   }
   const int kv_blocks_all = (p.Tk + BK - 1) / BK;
-  const int bh_count = p.B * p.Hq;
+  const int tok = attn_tile_tokens(p);
+  const int heads = p.Hq >> p.pack_log2;                  // a "head" of an item is a group of packed heads: they share K and V
+  const int per_kv = (p.Hq / p.Hkv) >> p.pack_log2;
+  const int bh_count = p.B * heads;
   auto item_of = [&](int n) -> AttnItem {
     int idx = n * G + pos_in_round(n);
     if constexpr (DEAL) idx = deal.list[deal_first + n];
     AttnItem it;
     if constexpr (PAIR) {
       const int bh0 = 2 * idx, bh1 = min(2 * idx + 1, bh_count - 1);  // (an odd count: the last head twice, stored once)
-      it.h = bh0 % p.Hq;
-      it.b = bh0 / p.Hq;
-      it.kvh = it.h / (p.Hq / p.Hkv);
-      it.h1 = bh1 % p.Hq;
-      it.b1 = bh1 / p.Hq;
-      it.kvh1 = it.h1 / (p.Hq / p.Hkv);
+      it.b = bh0 / heads;
+      it.b1 = bh1 / heads;
+      const int hg0 = bh0 - it.b * heads, hg1 = bh1 - it.b1 * heads;
+      it.kvh = hg0 / per_kv;
+      it.kvh1 = hg1 / per_kv;
+      it.h = hg0 << p.pack_log2;
+      it.h1 = hg1 << p.pack_log2;
       it.t0 = 0;
       it.nb0 = it.nb1 = kv_blocks_all;  // (causal: as many keys as queries, so every block holds a visible key)
       it.nbi = 2 * kv_blocks_all;
       it.store1 = bh0 + 1 < bh_count;
     } else {
-      const int qr = idx / bh_count;
-      const int bh = idx - qr * bh_count;
+      int qr, bh;
+      attn_item_place(idx, bh_count, p.q_pairs, DEAL ? bh_count : p.chunk, bh, qr);
       const int qp = p.causal ? (p.q_pairs - 1 - qr) : qr;
-      it.h = it.h1 = bh % p.Hq;
-      it.b = it.b1 = bh / p.Hq;
-      it.kvh = it.kvh1 = it.h / (p.Hq / p.Hkv);
-      it.t0 = qp * 2 * kAttnBlockQ;
+      it.b = it.b1 = bh / heads;
+      const int hg = bh - it.b * heads;
+      it.kvh = it.kvh1 = hg / per_kv;
+      it.h = it.h1 = hg << p.pack_log2;
+      it.t0 = HALF ? qp * tok : qp * 2 * tok;
       // causal: a tile whose last row is r sees keys 0 .. r
-      it.nb0 = p.causal ? min(kv_blocks_all, (it.t0 + kAttnBlockQ - 1) / BK + 1) : kv_blocks_all;
-      it.nb1 = p.causal ? min(kv_blocks_all, (it.t0 + 2 * kAttnBlockQ - 1) / BK + 1) : kv_blocks_all;
+      it.nb0 = p.causal ? min(kv_blocks_all, (it.t0 + tok - 1) / BK + 1) : kv_blocks_all;
+      it.nb1 = p.causal ? min(kv_blocks_all, (it.t0 + 2 * tok - 1) / BK + 1) : kv_blocks_all;
       it.nbi = it.nb1;
       if constexpr (HALF) {
         it.nbi = it.nb0;
         it.nb1 = 0;
       }
-      it.store1 = it.t0 + kAttnBlockQ < p.Tq;
+      it.store1 = !HALF && it.t0 + tok < p.Tq;
     }
     return it;
   };
@@ -320,7 +342,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             ptx::mbar_arrive_expect_tx(bar(Q_FULL + t), tile_bytes);
             for (int c = 0; c < chunks; ++c)
               ptx::tma_load_4d(q_s0 + (uint32_t)t * tile_bytes + c * kAttnChunkBytes, &tmQ, bar(Q_FULL + t), c * 64,
-                               t ? it.h1 : it.h, PAIR ? 0 : it.t0 + t * kAttnBlockQ, (t ? it.b1 : it.b) & p.q_each);
+                               t ? it.h1 : it.h, PAIR ? 0 : it.t0 + t * tok, (t ? it.b1 : it.b) & p.q_each);
           }
         }
         for (int r = 0; ok && r < it.nbi; ++r, ++g) {
@@ -454,7 +476,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             if (t == 0 || it.store1) {
               for (int c = 0; c < chunks; ++c)
                 ptx::tma_store_4d(&tmO, o_stage + c * kAttnChunkBytes, c * 64, t ? it.h1 : it.h,
-                                  PAIR ? 0 : it.t0 + t * kAttnBlockQ, t ? it.b1 : it.b);
+                                  PAIR ? 0 : it.t0 + t * tok, t ? it.b1 : it.b);
               ptx::bulk_commit_group();
               ptx::bulk_wait_group_read<0>();  // the staging buffer may be rewritten
             }
@@ -482,7 +504,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     for (int n = 0; ok && n < n_items; ++n) {
       const AttnItem it = item_of(n);
       const int nbt = t ? it.nb1 : it.nb0;
-      const int t_row = PAIR ? row : it.t0 + t * kAttnBlockQ + row;
+      const int t_row = (PAIR ? 0 : it.t0 + t * tok) + (row >> p.pack_log2);
       float m = -INFINITY;  // reference maximum of scale_log2 * score the exponentials are taken against
       float l = 0.f;        // running sum of 2^(scale_log2 * score - m)
       for (int j = 0; ok && j < nbt; ++j, ++gt) {

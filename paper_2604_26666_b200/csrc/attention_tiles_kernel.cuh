@@ -13,7 +13,8 @@
 //   two tiles, blocks of 128 keys: half the hand-overs per key, for problems too small to have three tiles on every SM.
 // Causal, 12 heads, microseconds, pairs -> this kernel, short runs: 16 x 1000 53.4 -> 45.5, 40 x 384 42.1 -> 27.6, 16 x 300
 // 19.9 -> 12.7; two tiles: 1 x 1500 23.0 -> 17.5.  Calls back to back, at the clock that the power limit leaves: 16 x 1000
-// 55.3 -> 51.6, 8 x 4096 322 -> 316, 256 x 300 226 -> 175; from 32 tiles an SM on pairs are faster (128 x 1000 422 against 500).
+// 55.3 -> 51.6, 8 x 4096 322 -> 316, 256 x 300 226 -> 175; with heads in chunks that fit L2 (attn_item_place) 128 x 512 152 -> 109,
+// 65 x 1000 202 -> 171, 32 x 2048 326 -> 285.
 // Which call takes what is in attention_tiles_choice (fact_api.cu).  What is left: about 11 of 16 exponentials a cycle and SM within a block; about 2500
 // cycles per tile for its last product and its output, under which only the other pipelines run.
 // Tried and slower: two tiles in blocks of 64 keys with scores and probabilities double-buffered and the next block's
@@ -145,8 +146,8 @@ __global__ void __launch_bounds__(AttnTiles<TILES>::kThreads, 1)
   auto item_of = [&](int n) -> AttnTile {
     int idx = n * W + pos_in_round(n);
     if constexpr (DEAL) idx = deal.list[deal_first + n];
-    const int qr = idx / bh_count;
-    const int bh = idx - qr * bh_count;
+    int qr, bh;
+    attn_item_place(idx, bh_count, p.q_tiles, DEAL ? bh_count : p.chunk, bh, qr);
     AttnTile it;
     it.h = bh % p.Hq;
     it.b = bh / p.Hq;

@@ -142,7 +142,7 @@ struct fact_handle_s {
   std::unique_ptr<AttnDeal> attn_deal;         // the host's deal of the last causal attention shape (see fact_attention)
   std::array<long long, 6> attn_deal_key{};
   std::unique_ptr<AttnTilesDeal> attn_tiles_deal;  // the same at head_dim 64
-  std::array<long long, 4> attn_tiles_deal_key{};
+  std::array<long long, 5> attn_tiles_deal_key{};
   int kc_clusters[6] = {0, 0, 0, 0, 0, 0};  // clusters of 2 / 4 / 8 CTAs of the K-slice kernel (single CTAs, pairs) the
                                             // device holds at once
   std::string last_error;        // text of the most recent CUDA failure
@@ -1364,23 +1364,32 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
 // Which items of a causal attention problem every CTA takes: the items in order of weight (the key blocks an item's
 // later tile sees, plus about one block of fixed cost), each given to the CTA that has the least so far (the lower
 // CTA on a tie, so the first round is CTA c <- item c).  Item idx is (query pair qr = idx / bh counted from the
-// end of the sequence, head idx % bh), the kernel's own numbering.
-void build_attention_deal(int G, long long bh, int q_pairs, int bk, long long seq_kv, AttnDeal& d) {
-  const int items = (int)(bh * q_pairs);
+// end of the sequence, head idx % bh), the kernel's own numbering.  `tokens`: query positions of a tile.  Heads come in
+// chunks of `chunk` (attention_chunk; 0: all at once), a chunk's items in order of weight.
+template <typename F>
+void for_each_item(long long bh, int per_head, long long chunk, F&& f) {
+  if (chunk <= 0) chunk = bh;
+  for (long long first = 0; first < bh; first += chunk)
+    for (int qr = 0; qr < per_head; ++qr)
+      for (long long head = first; head < std::min(bh, first + chunk); ++head) f((int)(qr * bh + head), qr);
+}
+
+void build_attention_deal(int G, long long bh, int q_pairs, int bk, long long seq_kv, AttnDeal& d, int tokens = kAttnBlockQ,
+                          long long chunk = 0) {
   const int kv_blocks = (int)((seq_kv + bk - 1) / bk);
   std::vector<std::vector<uint16_t>> mine((size_t)G);
   using Slot = std::pair<double, int>;  // (load, CTA)
   std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
   for (int c = 0; c < G; ++c) heap.push({0.0, c});
-  for (int idx = 0; idx < items; ++idx) {
-    const int qp = q_pairs - 1 - (int)(idx / bh);
-    const int nb1 = std::min(kv_blocks, (qp * 2 * kAttnBlockQ + 2 * kAttnBlockQ - 1) / bk + 1);
+  for_each_item(bh, q_pairs, chunk, [&](int idx, int qr) {
+    const int qp = q_pairs - 1 - qr;
+    const int nb1 = std::min(kv_blocks, (qp * 2 * tokens + 2 * tokens - 1) / bk + 1);
     const double w = nb1 + (bk == 128 ? 1.0 : 2.0);
     const Slot s = heap.top();
     heap.pop();
     mine[(size_t)s.second].push_back((uint16_t)idx);
     heap.push({s.first + w, s.second});
-  }
+  });
   int pos = 0;
   for (int c = 0; c < G; ++c) {
     d.off[c] = (uint16_t)pos;
@@ -1391,15 +1400,14 @@ void build_attention_deal(int G, long long bh, int q_pairs, int bk, long long se
 
 // The same for the kernel of independent tiles (attention_tiles_kernel.cuh), whose items are tiles of 128 rows: each to the
 // CTA with the least so far, and there to the pipeline with the least.
-void build_attention_tiles_deal(int G, int pipes, int bk, long long bh, int q_tiles, AttnTilesDeal& d) {
-  const int items = (int)(bh * q_tiles);
+void build_attention_tiles_deal(int G, int pipes, int bk, long long bh, int q_tiles, AttnTilesDeal& d, long long chunk = 0) {
   std::vector<std::vector<uint16_t>> mine((size_t)G * pipes);
   std::vector<int> load((size_t)G * pipes, 0);
   using Slot = std::pair<int, int>;  // (load, CTA)
   std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
   for (int c = 0; c < G; ++c) heap.push({0, c});
-  for (int idx = 0; idx < items; ++idx) {
-    const int qt = q_tiles - 1 - (int)(idx / bh);
+  for_each_item(bh, q_tiles, chunk, [&](int idx, int qr) {
+    const int qt = q_tiles - 1 - qr;
     const int w = (qt * kAttnBlockQ + kAttnBlockQ - 1) / bk + 1 + 64 / bk;
     const Slot s = heap.top();
     heap.pop();
@@ -1409,7 +1417,7 @@ void build_attention_tiles_deal(int G, int pipes, int bk, long long bh, int q_ti
       if (load[(size_t)(t * G + s.second)] < load[(size_t)best]) best = t * G + s.second;
     load[(size_t)best] += w;
     mine[(size_t)best].push_back((uint16_t)idx);
-  }
+  });
   int pos = 0;
   for (int c = 0; c < G * pipes; ++c) {
     d.off[c] = (uint16_t)pos;
@@ -1418,38 +1426,112 @@ void build_attention_tiles_deal(int G, int pipes, int bk, long long bh, int q_ti
   d.off[G * pipes] = (uint16_t)pos;
 }
 
+// How many heads' items come before the next heads' (attn_item_place): as many as have their keys and values in L2 together,
+// in whole rounds over the workers where that is possible (a round of items of one weight, the next one in the opposite
+// direction, leaves nobody behind), and at least two rounds.  Causal, 12 heads of 64, three tiles an SM, microseconds with
+// all heads at once / in chunks of 32 MB: 128 x 512 118.0 / 109.1, 65 x 1000 185 / 171, 32 x 2048 322 / 285, 43 x 1500 257 /
+// 223, 21 x 3000 436 / 412; problems of up to 48 MB stay whole (16 x 1000 44.8 / 44.6, 10 x 3000 195 / 203 in chunks).
+long long attention_chunk(long long bh, long long per_head, long long kv_bytes, long long workers) {
+  constexpr long long kFits = 32LL << 20;
+  if (bh * kv_bytes <= kFits + kFits / 2) return bh;
+  long long n = std::max<long long>(1, kFits / kv_bytes), a = workers, b = per_head;
+  while (b) std::swap(a %= b, b);
+  const long long whole = workers / a;  // heads that make whole rounds
+  if (n >= whole) n -= n % whole;
+  return std::min(bh, std::max(n, (2 * workers + per_head - 1) / per_head));
+}
+
+// How a call of the paired kernel is cut into items.  The query heads that share a key/value head lie side by side in a tile, 2^pack of
+// them with 128 >> pack tokens each (head_dim 128), and an item is two such tiles, two heads' (groups of heads') only tile, or
+// one tile where there are no more tiles than SMs.  Packed tiles cover fewer positions, so a causal problem computes fewer
+// blocks above its diagonal and a ragged one less padding: 32 query heads on 8 of 128, microseconds unpacked / packed, causal 53 x 300
+// 137 / 84, 123 x 130 126 / 88, 26 x 300 72.1 / 41.5, 8 x 1000 80.3 / 75.0, 3 x 2048 99.9 / 95.7, full 26 x 300 82.7 / 58.0.  Where the
+// work is the same (full 62 x 256 85.3 / 94.5, 80 x 200 103 / 109) unpacked tiles stay.  One tile per item, 32 heads of 128: 1 x 256 9.1 -> 8.6 us, 1 x 512
+// 14.4 -> 12.9.
+struct AttnCut {
+  int pack_log2, mode;
+  long long bh, per_head, items;
+};
+AttnCut attention_cut(long long batch, long long heads_q, long long seq_q, long long seq_kv, int head_dim, bool causal, int max_pack,
+                      long long sms) {
+  AttnCut best = {0, kAttnRows, 0, 0, 0};
+  double best_cost = 1e300;
+  const int bk = attn_block_k(head_dim);
+  const long long kv_blocks = (seq_kv + bk - 1) / bk;
+  if (head_dim == 128)
+    for (int pk = 0; pk <= max_pack; ++pk) {
+      const long long bh = batch * heads_q >> pk, tokens = kAttnBlockQ >> pk, tiles = (seq_q + tokens - 1) / tokens;
+      if (bh * tiles <= sms) return {pk, kAttnHalf, bh, tiles, bh * tiles};
+    }
+  for (int i = 0; i <= max_pack; ++i) {
+    const int pk = causal ? max_pack - i : i;  // (of equals the first)
+    const long long bh = batch * heads_q >> pk, tokens = kAttnBlockQ >> pk, tiles = (seq_q + tokens - 1) / tokens;
+    AttnCut c = {pk, tiles == 1 ? kAttnPair : kAttnRows, bh, (tiles + 1) / 2, 0};
+    c.items = tiles == 1 ? (bh + 1) / 2 : bh * c.per_head;
+    // in key blocks; about two for an item's start and end
+    double cost = (double)((c.items + sms - 1) / sms) * (2.0 + (double)kv_blocks);
+    if (causal && c.mode == kAttnRows) {
+      auto blocks = [&](long long tiles_seen) { return (double)std::min(kv_blocks, (tokens * tiles_seen - 1) / bk + 1); };
+      if (c.items <= sms) {  // one round: the heaviest item, a block that only one of its tiles sees at three quarters
+        cost = 2.0 + 0.25 * blocks(2 * c.per_head - 1) + 0.75 * blocks(2 * c.per_head);
+      } else {
+        double total = 0.5 * (double)c.per_head * (4.0 + (double)kv_blocks);
+        if (c.per_head <= 64) {
+          total = 0.0;
+          for (long long q = 1; q <= c.per_head; ++q) total += 2.0 + blocks(2 * q);
+        }
+        cost = total * (double)bh / (double)sms + 0.5 * (2.0 + (double)kv_blocks);
+      }
+    }
+    if (cost < 0.98 * best_cost) {
+      best_cost = cost;
+      best = c;
+    }
+  }
+  return best;
+}
+
 // Which kernel an attention call at head_dim 64 takes: 3 or 2 independent tiles of 128 rows per SM
 // (attention_tiles_kernel.cuh), or 0, tiles in pairs that share their keys (attention_kernel.cuh).  Microseconds measured
 // as pairs / two / three (12 heads):
-//  - sequences of one tile: two while every head has an SM (4 x 100 6.1 / 5.3 / 6.7); three where one block of 64 keys is
-//    all there is, which the blocks of 128 compute twice over (256 x 64 36.4 / 43.3 / 29.4); pairs else (64 x 128 full
-//    13.6 / 14.9 / 15.6).
-//  - causal: a pair's first tile waits out the blocks that only its second sees.  Three from one and a half tiles an SM on
-//    for short sequences and three for long (16 x 1000 53.4 / 53.4 / 45.5, 128 x 512 128 / 133 / 113, 10 x 256 8.4 / 7.5 /
-//    7.2), two below that, where a tile is mostly alone on its SM and blocks of 128 keys get it done sooner (1 x 4096
-//    55.6 / 48.8 / 53.7, 1 x 1500 23.0 / 17.5 / 21.0).  From 32 tiles an SM on (48 below 8 tiles a
-//    sequence: 128 x 512, 41 an SM, 145.5 / 156.2 / 142.6), where the keys no longer stay in L2 between
-//    the tiles of a head and the host no longer deals, pairs again: calls back to back 130 x 1000 443 / 497 / 509, 65 x 2000
-//    757 / 866 / 879, 16 x 8192 2585 / 2915 / 2913 (16 x 4096, 42 an SM, 670 / 730 / 682; 8 x 4096, 21 an SM, 325 / 335 / 320)
-//    -- but not where the blocks that a pair computes for nothing are a quarter of its work: 217 x 300 197 / 157 / 152.
-//  - full: pairs load their keys once for two tiles and are the best where both are busy (16 x 1024 81.9 / 87.1 / 85.4, 128
-//    x 512 151 / 186 / 189); tiles where items of 256 rows leave a sixth of the SMs' time or more empty (1 x 1000 18.4 /
-//    13.5 / 15.9, 40 x 384 45.0 / 38.3 / 41.3, 16 x 300 22.5 / 17.8 / 17.4; three a SM exactly: 1 x 4096 104 / 95.6 / 81.2).
-int attention_tiles_choice(long long q_tiles, long long bh, long long seq_kv, bool causal, long long sms) {
+//  - sequences of one tile: three where one block of 64 keys is all there is, which the blocks of 128 compute twice over
+//    (1 x 40 - / 6.2 / 5.4, 256 x 64 36.4 / 43.3 / 29.4); two while an SM has no more than two (1 x 100 - / 5.4 / 5.5, 20 x 100 7.5 / 7.0 / 7.0, 23 x 84
+//    7.5 / 6.9 / 6.9); pairs else (64 x 128 full 13.6 / 14.9 / 15.6).
+//  - causal: a pair's first tile waits out the blocks that only its second sees.  Three from three tiles an SM on, and from
+//    one and a half for short sequences (16 x 1000 57.5 / 52.6 / 44.6, 128 x 512 152 / 141 / 109, 10 x 256 8.4 / 7.5 / 7.2, 32 x 2048
+//    326 / 320 / 285, 16 x 4096 625 / 671 / 560); two below that, where a tile is mostly alone on its SM and
+//    blocks of 128 keys get it done sooner (1 x 4096 55.6 / 48.0 / 53.5, 1 x 1500 23.3 / 17.6 / 21.1).
+//  - full, few tiles: up to two an SM two (7 x 256 8.9 / 8.2 / 8.9, 5 x 400 13.0 / 12.3 / 12.3; from 16 tiles a sequence on
+//    pairs again, 1 x 3000 45.0 / 45.9 / 52.4), up to three three (1 x 4096 107 / 96.4 / 81.6).
+//  - full, more tiles: rounds of rows and keys as the three compute them, with what an item costs besides, in keys (100
+//    alone, 60 in a pair; a ragged last block 25 and 80, its mask touches all 64 or 128 of a row's scores): pairs
+//    where every tile is full and keys come in whole blocks (16 x 1024 81.9 / 87.1 / 85.4, 128 x 512 159 / 170 / 172, 62 x 256 30.5 / 32.2 / 34.6), three
+//    where pairs pad (123 x 130 58.5 / 56.0 / 44.5, 106 x 300 112 / 90.8 / 79.0, 80 x 200 42.2 / 39.6 / 39.8, 22 x 700 68.8 / 70.0 / 64.7).
+//  - grouped queries (`shared`): heads that share their keys read them from L2 together in either kernel, and neither the chunks
+//    nor the rounds above were measured for them: causal pairs from 32 tiles an SM on (48 below 8 tiles a sequence) unless a
+//    quarter of their blocks would be for nothing, full ones unless items of 256 rows leave a sixth of the SMs' time empty.
+int attention_tiles_choice(long long q_tiles, long long bh, long long seq_kv, bool causal, bool shared, long long sms) {
   const long long items = q_tiles * bh;
   if (items > 0x7fffffffLL) return 0;
-  if (q_tiles == 1) return items <= sms ? 2 : (seq_kv <= AttnTiles<3>::kBlockK ? 3 : 0);
+  constexpr long long kBlock3 = AttnTiles<3>::kBlockK, kBlock0 = attn_block_k(64);
+  if (q_tiles == 1) return seq_kv <= kBlock3 ? 3 : (items <= 2 * sms ? 2 : 0);
+  const long long tiles_each = (items + sms - 1) / sms, pairs = (q_tiles + 1) / 2;
+  const long long pair_rounds = (pairs * bh + sms - 1) / sms;
   if (causal) {
     // blocks of 128 x 128 that a head's pairs go through, two tiles at a time, and those that its tiles see
-    const long long pairs = (q_tiles + 1) / 2;
     const long long in_pairs = 2 * (q_tiles % 2 ? pairs * (pairs - 1) + q_tiles : pairs * (pairs + 1)), seen = q_tiles * (q_tiles + 1) / 2;
-    if (items >= (q_tiles >= 8 ? 32 : 48) * sms && 100 * seen > 76 * in_pairs) return 0;
+    if (shared && items >= (q_tiles >= 8 ? 32 : 48) * sms && 100 * seen > 76 * in_pairs) return 0;
     return items >= 3 * sms || (q_tiles <= 4 && 2 * items >= 3 * sms) ? 3 : 2;
   }
-  const long long tiles_each = (items + sms - 1) / sms;
-  const long long as_pairs = 2 * (((q_tiles + 1) / 2 * bh + sms - 1) / sms);
-  if (5 * as_pairs < 6 * tiles_each) return 0;
-  return tiles_each == 3 ? 3 : 2;
+  if (tiles_each <= 2) return tiles_each == 2 && q_tiles >= 16 ? 0 : 2;
+  if (tiles_each == 3) return 3;
+  if (shared) return 10 * pair_rounds < 6 * tiles_each ? 0 : 2;
+  auto keys = [&](long long block, long long item, long long ragged) {
+    return (seq_kv + block - 1) / block * block + item + (seq_kv % block ? ragged : 0);
+  };
+  const long long as_three = 3 * ((items + 3 * sms - 1) / (3 * sms)) * keys(kBlock3, 100, 25);
+  const long long as_pairs = 2 * pair_rounds * keys(kBlock0, 60, 80);
+  return 100 * as_three < 97 * as_pairs ? 3 : 0;
 }
 
 // Attention at head_dim 64 by independent tiles (attention_tiles_kernel.cuh), items = (batch, head, 128 query rows).
@@ -1479,12 +1561,15 @@ fact_status_t attention_tiles(fact_handle_t h, AttnParams p, const CUtensorMap& 
   // Problems of few rounds are dealt out by the host, as in the kernel of paired tiles.
   const bool deal = p.causal && p.q_tiles > 1 && p.items > ctas && p.items <= kAttnDealItems && ctas <= kAttnDealCtas &&
                     p.items < 16LL * TILES * ctas;
+  const long long bh = (long long)p.B * p.Hq;
+  const long long chunk = attention_chunk(bh, p.q_tiles, 4LL * p.Tk * 64 * p.Hkv / p.Hq, (long long)ctas * TILES);
+  p.chunk = (int)chunk;  // (a deal's list is in this order already)
   cudaError_t e;
   if (deal) {
-    const std::array<long long, 4> key = {(long long)p.B * p.Hq, p.q_tiles, TILES, ctas};
+    const std::array<long long, 5> key = {bh, p.q_tiles, TILES, ctas, chunk};
     if (!h->attn_tiles_deal || h->attn_tiles_deal_key != key) {
       if (!h->attn_tiles_deal) h->attn_tiles_deal.reset(new AttnTilesDeal());
-      build_attention_tiles_deal(ctas, TILES, L::kBlockK, (long long)p.B * p.Hq, p.q_tiles, *h->attn_tiles_deal);
+      build_attention_tiles_deal(ctas, TILES, L::kBlockK, bh, p.q_tiles, *h->attn_tiles_deal, chunk);
       h->attn_tiles_deal_key = key;
     }
     e = launch_pdl(h, dealt, (unsigned)ctas, (unsigned)L::kThreads, (size_t)smem, stream, 1, tq, tk, tv, p, *h->attn_tiles_deal);
@@ -2392,18 +2477,18 @@ fact_status_t fact_tune_cache_load(fact_handle_t h, const char* path) {
 // ---------------------------------------------------------------------------------------------
 // Fused multi-head attention
 namespace {
-// Rank-4 BF16 tensor map over [B][T][H][D]-like storage, dims ordered (D, H, T, B), box 64 x 1 x box_rows x 1.  A batch
+// Rank-4 BF16 tensor map over [B][T][H][D]-like storage, dims ordered (D, H, T, B), box 64 x box_heads x box_rows x 1.  A batch
 // stride of 0 (one Q, K or V for all entries) is a map of one entry, which the kernels address with coordinate 0.
 fact_status_t encode_map_bthd(fact_handle_t h, CUtensorMap* map, const void* base, long long D, long long H, long long T,
                               long long B, long long stride_h, long long stride_t, long long stride_b,
-                              int box_rows = kAttnBlockQ) {
+                              int box_rows = kAttnBlockQ, int box_heads = 1) {
   if (B == 1 || stride_b == 0) {  // (the stride is not used, but has to be a valid one)
     B = 1;
     stride_b = std::max<long long>(stride_t * T, 8);
   }
   cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T, (cuuint64_t)B};
   cuuint64_t strides[3] = {(cuuint64_t)stride_h * 2, (cuuint64_t)stride_t * 2, (cuuint64_t)stride_b * 2};
-  cuuint32_t box[4] = {64, 1, (cuuint32_t)box_rows, 1};
+  cuuint32_t box[4] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_rows, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   CUresult r = h->encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -2552,16 +2637,22 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
   CUtensorMap tq, tk, tv, to;
   const long long q_tiles = (seq_q + kAttnBlockQ - 1) / kAttnBlockQ;
   const long long tile_items = q_tiles * heads_q * batch;
-  const int tiles = head_dim == 64 ? attention_tiles_choice(q_tiles, heads_q * batch, seq_kv, causal != 0, h->sm_count) : 0;
+  const int tiles = head_dim == 64 ? attention_tiles_choice(q_tiles, heads_q * batch, seq_kv, causal != 0, heads_q != heads_kv, h->sm_count) : 0;
   // keys go in blocks of 128 or 64, as the kernels' tensor-memory budgets have it
   const int block_k = tiles == 3 ? AttnTiles<3>::kBlockK : (tiles == 2 ? AttnTiles<2>::kBlockK : attn_block_k((int)head_dim));
-  fact_status_t st = encode_map_bthd(h, &tq, Q, head_dim, heads_q, seq_q, batch, q_sh, q_st, q_sb);
+  int max_pack = 0;
+  if (head_dim == 128)
+    while (max_pack < 7 && (heads_q / heads_kv) % (2 << max_pack) == 0) ++max_pack;
+  AttnCut cut = {0, kAttnRows, 0, 0, 0};
+  if (tiles == 0) cut = attention_cut(batch, heads_q, seq_q, seq_kv, (int)head_dim, causal != 0, max_pack, h->sm_count);
+  const int pack = 1 << cut.pack_log2, tokens = kAttnBlockQ >> cut.pack_log2;  // query heads / positions of a tile
+  fact_status_t st = encode_map_bthd(h, &tq, Q, head_dim, heads_q, seq_q, batch, q_sh, q_st, q_sb, tokens, pack);
   if (st == FACT_OK)
     st = encode_map_bthd(h, &tk, K, head_dim, heads_kv, seq_kv, batch, k_sh, k_st, k_sb, block_k);
   if (st == FACT_OK)
     st = encode_map_bthd(h, &tv, V, head_dim, heads_kv, seq_kv, batch, v_sh, v_st, v_sb, block_k);
   if (st == FACT_OK && tiles == 0)
-    st = encode_map_bthd(h, &to, O, head_dim, heads_q, seq_q, batch, o_sh, o_st, o_sb);
+    st = encode_map_bthd(h, &to, O, head_dim, heads_q, seq_q, batch, o_sh, o_st, o_sb, tokens, pack);
   if (st == FACT_OK) {
     AttnParams p;
     memset(&p, 0, sizeof p);
@@ -2570,11 +2661,11 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
     p.Tk = (int)seq_kv;
     p.Hq = (int)heads_q;
     p.Hkv = (int)heads_kv;
-    p.D = (int)head_dim;
     p.causal = causal != 0;
     p.q_each = q_sb != 0 ? -1 : 0;
     p.k_each = k_sb != 0 ? -1 : 0;
     p.v_each = v_sb != 0 ? -1 : 0;
+    p.pack_log2 = (int8_t)cut.pack_log2;
     const double sc = scale > 0.f ? (double)scale : 1.0 / std::sqrt((double)head_dim);
     p.scale_log2 = (float)(sc * 1.4426950408889634);
     p.kmajor_desc = smem_desc_template(16, 1024);
@@ -2596,18 +2687,15 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
       if (dev != h->device) cudaSetDevice(dev);
       return st;
     }
-    p.q_pairs = (int)((seq_q + 2 * kAttnBlockQ - 1) / (2 * kAttnBlockQ));  // an item is two tiles of 128 query rows
-    // ... or, for sequences that fit one tile, two heads' tiles once there are more heads than SMs, one head's before that
-    const bool one_tile = seq_q <= kAttnBlockQ;
-    const bool pair = one_tile && batch * heads_q > h->sm_count;
-    const long long items = pair ? (batch * heads_q + 1) / 2 : (long long)p.q_pairs * heads_q * batch;
-    if (items > 0x7fffffffLL) {
+    if (cut.items > 0x7fffffffLL) {
       if (dev != h->device) cudaSetDevice(dev);
       return FACT_ERR_UNSUPPORTED;
     }
-    p.items = (int)items;
+    const long long bh = cut.bh;  // (a head: a group of packed heads)
+    p.q_pairs = (int)cut.per_head;
+    p.items = (int)cut.items;
     const long long ctas = std::min<long long>(p.items, h->sm_count);  // persistent: one CTA per SM
-    const int smem = std::max((int)attn_smem_bytes(p.D), kMinSmemRequest);
+    const int smem = std::max((int)attn_smem_bytes((int)head_dim), kMinSmemRequest);
     typedef void (*Plain)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams, AttnNoDeal);
     typedef void (*Dealt)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, AttnParams, AttnDeal);
     // (head_dim 64: neither causal problems of few rounds nor one head per item, see attention_tiles_choice)
@@ -2646,16 +2734,19 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
       // the host deals the items out itself -- heaviest first, each to the CTA with the least so far -- and hands the
       // list to the kernel as a parameter.  The list is kept for the next call of the same shape.
       const int bk = block_k;
-      const bool deal = causal != 0 && head_dim == 128 && !one_tile && p.items > ctas && p.items <= kAttnDealItems && ctas <= kAttnDealCtas &&
+      const long long per_kv = heads_q / heads_kv / pack;
+      const long long chunk = attention_chunk(bh, p.q_pairs, 4 * seq_kv * head_dim / per_kv, ctas);
+      const bool deal = causal != 0 && head_dim == 128 && cut.mode == kAttnRows && p.items > ctas && p.items <= kAttnDealItems && ctas <= kAttnDealCtas &&
                         p.items < 16 * ctas;
       if (deal) {
-        const std::array<long long, 6> key = {(long long)batch * heads_q, (long long)p.q_pairs, (long long)bk, (long long)seq_kv, (long long)ctas, (long long)seq_q};
+        const std::array<long long, 6> key = {bh, (long long)p.q_pairs, (long long)tokens, (long long)seq_kv, (long long)ctas, chunk};
         if (!h->attn_deal || h->attn_deal_key != key) {
           if (!h->attn_deal) h->attn_deal.reset(new AttnDeal());
-          build_attention_deal((int)ctas, batch * heads_q, p.q_pairs, bk, seq_kv, *h->attn_deal);
+          build_attention_deal((int)ctas, bh, p.q_pairs, bk, seq_kv, *h->attn_deal, tokens, chunk);
           h->attn_deal_key = key;
         }
       }
+      p.chunk = (int)chunk;  // (a deal's list is in this order already)
       const AttnNoDeal none = {0};
       cudaError_t e;
       const int d = head_dim == 128;
@@ -2663,7 +2754,7 @@ fact_status_t fact_attention(fact_handle_t h, int64_t batch, int64_t seq_q, int6
         e = launch_pdl(h, dealt, (unsigned)ctas, (unsigned)kAttnThreads, (size_t)smem, stream, 1, tq, tk, tv, to, p,
                        *h->attn_deal);
       else
-        e = launch_pdl(h, plain[d][pair ? kAttnPair : (one_tile ? kAttnHalf : kAttnRows)], (unsigned)ctas, (unsigned)kAttnThreads,
+        e = launch_pdl(h, plain[d][cut.mode], (unsigned)ctas, (unsigned)kAttnThreads,
                        (size_t)smem, stream, 1, tq, tk, tv, to, p, none);
       if (e != cudaSuccess) st = cuda_fail(h, "attention launch", e);
       else h->launches++;

@@ -257,3 +257,49 @@ def test_random_shapes(h, i, B, Tq, Tk, Hq, Hkv, D, causal):
     """Seeded random shapes: lengths on and around every border the kernel has (tile of 128 query rows, item of two
     tiles, key blocks of 64 or 128, a second tile wholly past the end), grouped queries, both head sizes."""
     check(h, rnd((B, Tq, Hq, D), 500 + i), rnd((B, Tk, Hkv, D), 600 + i), rnd((B, Tk, Hkv, D), 700 + i), causal)
+
+
+@pytest.mark.parametrize("B,T,Hq,Hkv,causal", [
+    (1, 33, 8, 2, True), (1, 129, 4, 1, True), (2, 300, 32, 8, False),   # one tile per item: no more tiles than SMs
+    (40, 31, 16, 4, True), (40, 32, 16, 4, False), (13, 40, 32, 8, True),  # ... two heads' (groups of heads') only tile
+    (20, 33, 32, 8, True), (20, 64, 32, 8, False), (9, 130, 32, 8, True), (9, 130, 32, 8, False), (5, 191, 24, 4, True),
+    (40, 65, 6, 2, True), (40, 257, 12, 2, False), (3, 200, 256, 1, True), (2, 97, 32, 8, True), (30, 63, 5, 5, True),
+], ids=lambda v: str(v))
+def test_packed_query_heads(h, B, T, Hq, Hkv, causal):
+    """head_dim 128: 1, 2, 4, ... query heads of a key/value head side by side in a tile, with lengths on both sides of the
+    tiles' 128 >> pack positions, in every kind of item; groups that are no power of two pack their largest one."""
+    rows = np.array(sorted({0, 15, 16, 31, 32, 63, 64, T // 2, T - 2, T - 1} & set(range(T))), dtype=np.int64)
+    check(h, rnd((B, T, Hq, 128), 801), rnd((B, T, Hkv, 128), 802), rnd((B, T, Hkv, 128), 803), causal, rows=rows)
+
+
+def test_packed_query_heads_of_strided_views(h):
+    """Q, K, V as column ranges of one buffer and O with heads outside tokens: the packed boxes follow the strides."""
+    B, T, Hq, Hkv, D = 6, 150, 32, 8, 128
+    dev = "cuda:0"
+    buf = rnd((B, T, Hq + 2 * Hkv, D), 811)
+    g = buf.to(dev)
+    out = torch.full((B, Hq, T, D), float("nan"), dtype=torch.bfloat16, device=dev)
+    h.attention(g[:, :, :Hq], g[:, :, Hq:Hq + Hkv], g[:, :, Hq + Hkv:], causal=True, out=out.permute(0, 2, 1, 3))
+    c, t = attention_gates(buf[:, :, :Hq], buf[:, :, Hq:Hq + Hkv], buf[:, :, Hq + Hkv:], True, to_f64(out.permute(0, 2, 1, 3)))
+    assert c <= 1.0 and t <= 1.0, (c, t)
+    assert h.device_status() == 0
+
+
+@pytest.mark.parametrize("B,T,Hq,Hkv,D,causal", [(130, 512, 12, 12, 64, True), (70, 1000, 12, 12, 64, True), (5, 8000, 12, 12, 64, True),
+                                                 (130, 512, 12, 12, 64, False), (60, 900, 16, 4, 128, True), (60, 900, 16, 4, 128, False),
+                                                 (20, 4000, 8, 2, 128, True)],
+                         ids=lambda v: str(v))
+def test_heads_in_chunks_that_fit_l2(h, B, T, Hq, Hkv, D, causal):
+    """More keys and values than L2 holds: heads go in chunks (dealt by the host or in closed form); every row of every entry
+    is written, and the first, a middle and the last entry's sampled rows are right."""
+    dev = "cuda:0"
+    gen = torch.Generator(device=dev).manual_seed(900)
+    q, k, v = (torch.randn(B, T, n, D, generator=gen, device=dev, dtype=torch.bfloat16) for n in (Hq, Hkv, Hkv))
+    out = torch.full_like(q, float("nan"))
+    h.attention(q, k, v, causal=causal, out=out)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0 and not bool(torch.isnan(out).any())
+    rows = np.array(sorted({0, 63, 64, 127, 128, T // 2, T - 1}), dtype=np.int64)
+    for b in (0, B // 2, B - 1):
+        c, t = attention_gates(q[b:b + 1].cpu(), k[b:b + 1].cpu(), v[b:b + 1].cpu(), causal, to_f64(out[b:b + 1])[:, rows], rows=rows)
+        assert c <= 1.0 and t <= 1.0, (b, c, t)
