@@ -25,7 +25,7 @@ BIND_LIB = PKG / "_fact_bind.so"  # the ordinary call's marshalling (CPython ext
 BIND_STAMP = PKG / "_fact_bind.so.srchash"
 
 SOURCES = ["fact_api.cu"]
-HEADERS = ["gemm_kernel.cuh", "skinny_kernel.cuh", "kcluster_kernel.cuh", "attention_kernel.cuh", "attention_tiles_kernel.cuh", "attention_decode_kernel.cuh",
+HEADERS = ["gemm_kernel.cuh", "grouped_kernel.cuh", "skinny_kernel.cuh", "kcluster_kernel.cuh", "attention_kernel.cuh", "attention_tiles_kernel.cuh", "attention_decode_kernel.cuh",
            "norm_kernel.cuh", "tune_kernels.cuh", "ptx.cuh"]
 
 NVCC_FLAGS = [

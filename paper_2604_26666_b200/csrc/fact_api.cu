@@ -23,6 +23,7 @@
 
 #include "fact.h"
 #include "gemm_kernel.cuh"
+#include "grouped_kernel.cuh"
 #include "kcluster_kernel.cuh"
 #include "skinny_kernel.cuh"
 #include "attention_kernel.cuh"
@@ -1151,6 +1152,140 @@ fact_status_t launch_skinny(fact_handle_t h, const Problem& q, const Plan& plan,
   return FACT_OK;
 }
 
+// Grouped linear layers with the weights as the 256-row operand (grouped_kernel.cuh): weights as [N, K], an epilogue that works
+// on single columns, a BF16 output of whole 16-byte pieces, residual pairs on 4 bytes, at most kParamGroups groups.
+bool grouped_ok(const Problem& q) {
+  if (q.groups < 1 || q.groups > kParamGroups || q.K <= 0 || q.layout != FACT_B_NK) return false;
+  if (q.epi == FACT_EPI_SILU_GATE || q.epi == FACT_EPI_BIAS_SOFTMAX) return false;
+  if (q.out == FACT_OUT_BF16 && (q.N_out % 8 || q.ldc % 8 || !aligned16(q.C))) return false;
+  if (q.R && (q.N_out % 2 || q.ldr % 2 || (reinterpret_cast<uintptr_t>(q.R) & 3u))) return false;
+  long long units = 0;
+  for (int g = 0; g < q.groups; ++g) units += (q.group_rows[g] + kGrpTokens - 1) / kGrpTokens;
+  return units * ((q.N_out + kGrpFeatures - 1) / kGrpFeatures) <= 0x3fffffffLL;
+}
+
+// Most tokens of a unit: the width whose units are done first, as rounds over the pairs times a unit's cycles (a k-block takes
+// 332 at up to 128 tokens, what the weights' 16 KB a CTA need, and 2.1 a token above), where the units at 256 are few rounds.
+// One group of 900 x 8192 -> 256 as 4 units of 240 tokens 38.0 us, as 8 of 128 28.9; 8 groups of 900 x 8192 -> 768 as 96 units of 240 119.6, as 120
+// of 192 97.6.
+int grouped_tokens(fact_handle_t h, const Problem& q) {
+  const long long pairs = std::max(1, h->sm_count / 2), tiles_f = (q.N_out + kGrpFeatures - 1) / kGrpFeatures;
+  const double kb = (double)((q.K + q.k_elems() - 1) / q.k_elems());
+  int best = kGrpTokens;
+  double best_cost = 1e300;
+  for (int most = kGrpTokens; most >= 64; most -= 32) {
+    long long units = 0;
+    int widest = 16;
+    for (int g = 0; g < q.groups; ++g) {
+      const int count = (int)q.group_rows[g];
+      if (count == 0) continue;
+      const int tiles = (count + most - 1) / most;
+      units += tiles;
+      widest = std::max(widest, grouped_tile_width(count, tiles));
+    }
+    units *= tiles_f;
+    const double cost = (double)((units + pairs - 1) / pairs) * (kb * std::max(332.0, 2.1 * widest + 30.0) + 1500.0 + 8.0 * widest);
+    if (cost < 0.97 * best_cost) {
+      best_cost = cost;
+      best = most;
+    }
+    if (most == kGrpTokens && units > 3 * pairs) break;
+  }
+  return best;
+}
+
+template <int EPI>
+fact_status_t launch_grouped_instance(fact_handle_t h, const GroupedMaps& tm, const GroupedParams& p, const GroupedTable& tab,
+                                      size_t smem, cudaStream_t stream) {
+  const auto kern = fact_grouped_kernel<EPI>;
+  if (!h->configured_mask.test(194 + EPI)) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    if (e != cudaSuccess) return cuda_fail(h, "cudaFuncSetAttribute(grouped)", e);
+    h->configured_mask.set(194 + EPI);
+  }
+  const int pairs = std::min(std::max(1, h->sm_count / 2), p.total_units);
+  cudaError_t e = launch_pdl(h, kern, (unsigned)(2 * pairs), (unsigned)kThreads, smem, stream, 2, tm, p, tab);
+  if (e != cudaSuccess) return cuda_fail(h, "cudaLaunchKernelEx (grouped)", e);
+  h->launches++;
+  return FACT_OK;
+}
+
+fact_status_t launch_grouped(fact_handle_t h, const Problem& q, cudaStream_t stream) {
+  GroupedParams p;
+  GroupedTable tab;
+  memset(&p, 0, sizeof p);
+  struct Group {
+    int width, tiles, first, count;
+    int16_t g;
+  } groups[kParamGroups];
+  long long row = 0;
+  int rows_loaded = 8;  // most rows of X that a CTA's stage holds
+  const int most = grouped_tokens(h, q);
+  for (int g = 0; g < q.groups; ++g) {
+    const int count = (int)q.group_rows[g];
+    if (count > 0) {
+      const int tiles = (count + most - 1) / most, width = grouped_tile_width(count, tiles);
+      groups[p.groups++] = {width, tiles, (int)row, count, (int16_t)g};
+      int last = count - (tiles - 1) * width;  // (the last tile's own width loads its own boxes)
+      for (int n : {width, (last + 15) & ~15}) {
+        int first, second;
+        grouped_boxes(n / 2, first, second);
+        rows_loaded = std::max(rows_loaded, first + second);
+      }
+    }
+    row += count;
+  }
+  std::stable_sort(groups, groups + p.groups, [](const Group& x, const Group& y) { return x.width > y.width; });
+  int tiles = 0;
+  for (int i = 0; i < p.groups; ++i) {
+    tab.tiles[i] = tiles;
+    tab.first[i] = groups[i].first;
+    tab.count[i] = groups[i].count;
+    tab.group[i] = groups[i].g;
+    tiles += groups[i].tiles;
+  }
+  tab.tiles[p.groups] = tiles;
+  p.N_out = (int)q.N_out;
+  p.k_elems = q.k_elems();
+  p.k_blocks = (int)((q.K + p.k_elems - 1) / p.k_elems);
+  p.tiles_f = (int)((q.N_out + kGrpFeatures - 1) / kGrpFeatures);
+  p.total_units = tiles * p.tiles_f;
+  p.slab = (int)std::max<long long>(1, (32LL << 20) / ((long long)kGrpTokens * q.K * (q.fp8 ? 1 : 2)));
+  p.stage_bytes = kStageBytesA + (uint32_t)rows_loaded * 128u;
+  const uint32_t fixed = kGrpCtrlBytes + (q.out == FACT_OUT_F32 ? 0u : kGrpOutBytes);
+  p.stages = (int)std::min<uint32_t>(kMaxStages, (kSmemBudget - fixed) / p.stage_bytes);
+  p.desc = smem_desc_template(16, 1024);
+  p.idesc = (1u << 4) | (q.fp8 ? 0u : (1u << 7) | (1u << 10)) | ((uint32_t)(kGrpFeatures >> 4) << 24);
+  p.C = q.C;
+  p.ldc = q.ldc;
+  p.out_f32 = q.out == FACT_OUT_F32;
+  p.fp8 = q.fp8;
+  p.use_alpha = q.fp8 && q.alpha != 1.f;
+  p.alpha = q.alpha;
+  p.bias = reinterpret_cast<const __nv_bfloat16*>(q.bias);
+  p.R = reinterpret_cast<const __nv_bfloat16*>(q.R);
+  p.ldr = q.ldr;
+  p.status = h->d_status;
+  GroupedMaps tm;
+  const uint32_t kbox = (uint32_t)p.k_elems;
+  const uint64_t sB = q.groups > 1 ? (uint64_t)q.strideB : (uint64_t)q.ldb * (uint64_t)q.N_out;
+  fact_status_t st = encode_map(h, &tm.w, q.B, (uint64_t)q.K, (uint64_t)q.N_out, (uint64_t)q.groups, (uint64_t)q.ldb,
+                                std::max<uint64_t>(sB, 16), kbox, 128, false, q.fp8);
+  for (int i = 0; st == FACT_OK && i < kGrpMaps; ++i)
+    st = encode_map(h, &tm.x[i], q.A, (uint64_t)q.K, (uint64_t)q.M, 1, (uint64_t)q.lda,
+                    std::max<uint64_t>((uint64_t)q.lda * (uint64_t)q.M, 16), kbox, 128u >> i, false, q.fp8);
+  if (st != FACT_OK) return st;
+  const size_t smem = std::max<size_t>((size_t)p.stages * p.stage_bytes + fixed, (size_t)kMinSmemRequest);
+  switch ((int)q.epi) {
+    case kEpiNone: return launch_grouped_instance<kEpiNone>(h, tm, p, tab, smem, stream);
+    case kEpiBias: return launch_grouped_instance<kEpiBias>(h, tm, p, tab, smem, stream);
+    case kEpiBiasRelu: return launch_grouped_instance<kEpiBiasRelu>(h, tm, p, tab, smem, stream);
+    case kEpiBiasGeluTanh: return launch_grouped_instance<kEpiBiasGeluTanh>(h, tm, p, tab, smem, stream);
+    case kEpiBiasResidual: return launch_grouped_instance<kEpiBiasResidual>(h, tm, p, tab, smem, stream);
+    default: return FACT_ERR_INVALID_ARG;
+  }
+}
+
 fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, int splits_override, void* ws,
                   size_t ws_bytes, void* stream_v) {
   if (!h) return FACT_ERR_INVALID_ARG;
@@ -1158,6 +1293,14 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
   if (st != FACT_OK) return st;
   if (q.batch == 0 || q.M == 0 || q.N_out == 0) return FACT_OK;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_v);
+  if (user == nullptr && grouped_ok(q)) {
+    int now = -1;
+    if (cudaGetDevice(&now) != cudaSuccess) return FACT_ERR_CUDA;
+    if (now != h->device && cudaSetDevice(h->device) != cudaSuccess) return FACT_ERR_CUDA;
+    st = launch_grouped(h, q, stream);
+    if (now != h->device) cudaSetDevice(now);
+    return st;
+  }
   Plan plan;
   st = make_plan(h, q, user, splits_override, &plan);
   if (st == FACT_ERR_UNSUPPORTED && plan.from_table) {

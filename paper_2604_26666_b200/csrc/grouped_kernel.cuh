@@ -1,0 +1,388 @@
+// Grouped linear layers (one weight matrix per group of rows) for sm_100a with the weights as the 256-row operand.
+//
+// What bounds a layer of many experts with a few hundred tokens each is not the tensor pipe but what the SMs take in from L2
+// (about 12.5 TB/s over all of them) and the weights' DRAM stream.  With tokens as the operand of 128 or 256 rows (gemm_kernel.cuh) a
+// group of 270 tokens is a tile of 256 and a nearly empty one, and every tile brings its weights in again: 16384 tokens in 64
+// groups, 2048 -> 2048, were 1.9 GB into the SMs, 154 us of the call's 174-190.  Here the roles are the other way round: a CTA pair computes
+//   D^T[256 features, n tokens] = W[256 features, K] . X[n tokens, K]^T
+// (tcgen05.mma M = 256, cta_group 2: each CTA loads its 128 rows of W and half of the tokens), and a group's tokens are shared
+// out evenly over ceil(tokens / 256) tiles whose width is any multiple of 16: 270 tokens are two tiles of 144 and 128 columns, 4
+// tokens one of 16.  No column is computed for another group's rows but the last tile's padding to 16.
+// The same problem is 1.3 GB into the SMs: 157-163 -> 135 us (FP8 91.8 -> 76.7); 32 groups 134 -> 115, 4000 tokens in 32 groups 61.8 -> 52.7,
+// 256 tokens in 64 groups 90.3 -> 81.2 (the weights' stream at 6.6 TB/s), 8 groups of 8000 x 768 -> 3072 with GELU 39.1 -> 34.4.  What is left at
+// 16384 tokens: the weights' 537 MB from DRAM (102 us with the rows) beside the 1.3 GB.
+//
+// The accumulator has features in its lanes and tokens in its columns, so a thread holds one feature of 32 tokens at a time.
+// To FP32 a warp stores 128 contiguous bytes of a token's row per instruction.  To BF16 neighbouring lanes exchange halves of their
+// pairs of tokens (one shuffle a pair), the four warps of a lane quarter each put their 64 bytes of 32 rows side by side in shared
+// memory, and every warp writes eight of the rows, 256 bytes each; rows past the group's end are predicated off.  (Stored by each warp
+// for itself, 64 bytes a row, the output went to L2 at 1 TB/s: 8 groups, 16384 x 768 -> 3072 with GELU 101 us.)  A bias is one value
+// per thread.
+//
+// Roles, rings, waits and teardown are those of fact_gemm_kernel.  Units are numbered token tile by token tile, widest groups
+// first, so that what the pairs run at the same time costs the same and the last round is the cheapest.
+#pragma once
+#include "gemm_kernel.cuh"
+
+namespace fact {
+
+constexpr int kGrpFeatures = 256;  // features (rows of W) per unit: 128 per CTA of the pair
+constexpr int kGrpTokens = 256;    // most tokens per unit
+constexpr int kGrpMaps = 5;        // boxes of 128, 64, 32, 16 and 8 tokens: half a tile's tokens in one or two loads
+constexpr int kGrpBarriers = 2 * kMaxStages + 4 + 2;
+constexpr uint32_t kGrpRowBytes = 256;                           // of a token's row in a BF16 output: a CTA's 128 features
+constexpr uint32_t kGrpStageOutBytes = 32 * kGrpRowBytes;        // 32 rows on their way out
+constexpr uint32_t kGrpOutBytes = 4 * kGrpStageOutBytes;         // two such buffers for either set of four warps
+constexpr uint32_t kGrpCtrlBytes = kGrpBarriers * 8 + 16;
+
+struct GroupedParams {
+  int N_out;          // features
+  int k_blocks, k_elems;
+  int tiles_f;        // ceil(N_out / 256)
+  int total_units;
+  int slab;           // token tiles whose rows stay in L2 while the features go by
+  int groups;         // non-empty groups, in the order of the table
+  int stages;
+  uint32_t stage_bytes;  // 16 KB of W and the widest tile's half of X
+  uint64_t desc;      // UMMA descriptor template of both operands (K-major)
+  uint32_t idesc;     // without N
+  void* C;
+  long long ldc;
+  int out_f32, fp8, use_alpha;
+  float alpha;
+  const __nv_bfloat16* bias;
+  const __nv_bfloat16* R;
+  long long ldr;
+  int* status;
+};
+
+struct GroupedTable {
+  int tiles[kParamGroups + 1];  // token tiles before each group, in order
+  int first[kParamGroups];      // its first row of X and C
+  int count[kParamGroups];      // its rows (> 0)
+  int16_t group[kParamGroups];  // its weights
+};
+
+struct GroupedMaps {
+  CUtensorMap w;
+  CUtensorMap x[kGrpMaps];
+};
+
+// Width of every token tile of a group but the last: an even share, rounded up to 16.
+__host__ __device__ inline int grouped_tile_width(int count, int tiles) { return ((count + tiles - 1) / tiles + 15) & ~15; }
+
+// The boxes that bring in half a tile's tokens (a multiple of 8): one, where that loads at most 8 rows for nothing, or two.  (As many
+// boxes as the number has bits, up to four, cost more than the rows: a k-block of 112 tokens in three took 10 % longer than one of
+// 160 in two.)  `second` is 0 where there is one.
+__host__ __device__ inline void grouped_boxes(int half, int& first, int& second) {
+  int whole = 8;
+  while (whole < half) whole <<= 1;
+  first = whole;
+  second = 0;
+  if (whole - half <= 8) return;
+  int rest = 8;
+  while (whole / 2 + rest < half) rest <<= 1;
+  if (rest == whole / 2) return;
+  first = whole / 2;
+  second = rest;
+}
+
+struct GroupedUnit {
+  int g, f0;     // weights, first feature
+  int t0, t_end; // rows of X and C
+  int n;         // accumulator columns: the tokens rounded up to 16
+};
+
+__device__ __forceinline__ GroupedUnit grouped_unit(const GroupedParams& p, const GroupedTable& tab, int u) {
+  const int mt = u / p.tiles_f;
+  int lo = 0, hi = p.groups;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (tab.tiles[mid] <= mt) lo = mid;
+    else hi = mid;
+  }
+  const int first = tab.tiles[lo], tiles = tab.tiles[lo + 1] - first, count = tab.count[lo];
+  const int local = u - first * p.tiles_f;
+  const int per_slab = p.slab * p.tiles_f;
+  const int s = local / per_slab, rem = local - s * per_slab;
+  const int height = min(p.slab, tiles - s * p.slab);
+  const int ft = rem / height;
+  const int tt = s * p.slab + (rem - ft * height);
+  const int width = grouped_tile_width(count, tiles);
+  GroupedUnit w;
+  w.g = tab.group[lo];
+  w.f0 = ft * kGrpFeatures;
+  w.t0 = tab.first[lo] + tt * width;
+  w.t_end = min(tab.first[lo] + count, w.t0 + width);
+  w.n = (w.t_end - w.t0 + 15) & ~15;
+  return w;
+}
+
+// Lanes 2 i and 2 i + 1 hold (a0, a1) and (b0, b1): afterwards (a0, b0) and (a1, b1).  Its own inverse.
+__device__ __forceinline__ uint32_t transpose_pairs(uint32_t w, int lane) {
+  const uint32_t o = __shfl_xor_sync(0xffffffffu, w, 1);
+  return (lane & 1) ? __byte_perm(o, w, 0x7632) : __byte_perm(w, o, 0x5410);
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(kThreads, 1)
+    fact_grouped_kernel(const __grid_constant__ GroupedMaps tm, const __grid_constant__ GroupedParams p,
+                        const __grid_constant__ GroupedTable tab) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31;
+  const uint32_t cta_rank = ptx::cluster_ctarank();
+  const uint32_t smem_base = ptx::smem_u32(smem_raw);
+  if (smem_base & 1023u) {
+    if (threadIdx.x == 0) atomicExch(p.status, kDeviceTimeoutCode);
+    return;
+  }
+  const uint32_t out_base = smem_base + (uint32_t)p.stages * p.stage_bytes;
+  const uint32_t bar_base = out_base + (p.out_f32 ? 0u : kGrpOutBytes);
+  const uint32_t ctrl_off = bar_base - smem_base + kGrpBarriers * 8;
+  volatile uint32_t* tmem_holder_p = reinterpret_cast<volatile uint32_t*>(smem_raw + ctrl_off);
+  volatile int* abort_p = reinterpret_cast<volatile int*>(smem_raw + ctrl_off + 4);
+  auto full_bar = [&](int s) { return bar_base + 8u * (uint32_t)s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (uint32_t)(kMaxStages + s); };
+  auto accf_bar = [&](int b) { return bar_base + 8u * (uint32_t)(2 * kMaxStages + b); };
+  auto acce_bar = [&](int b) { return bar_base + 8u * (uint32_t)(2 * kMaxStages + 2 + b); };
+  auto rows_bar = [&](int set) { return bar_base + 8u * (uint32_t)(2 * kMaxStages + 4 + set); };
+
+  if (threadIdx.x < kGrpBarriers) {
+    const int i = (int)threadIdx.x;
+    ptx::mbar_init(bar_base + 8u * (uint32_t)i, i >= 2 * kMaxStages + 4 ? 4 : (i >= 2 * kMaxStages + 2 ? kEpiWarps * 2 : 1));
+    if (i == 0) *abort_p = 0;
+    ptx::fence_mbar_init();
+  }
+  if (warp == 0 && lane == 0) {
+    ptx::prefetch_tensormap(&tm.w);
+    for (int i = 0; i < kGrpMaps; ++i) ptx::prefetch_tensormap(&tm.x[i]);
+  }
+  if (warp == 1) {
+    __syncwarp();
+    ptx::tmem_alloc<2>(smem_base + ctrl_off, 512);
+    ptx::tmem_relinquish<2>();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::cluster_arrive();  // the peer's barriers must exist before anything arrives on them
+  ptx::cluster_wait();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = *tmem_holder_p;
+  ptx::grid_dependency_wait();  // everything above overlaps the tail of the kernel before; global memory from here on
+
+  long long t_clk0 = 0;
+  unsigned long long t_ns0 = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    t_clk0 = clock64();
+    t_ns0 = ptx::globaltimer_ns();
+  }
+  const int unit0 = (int)(blockIdx.x / 2), unit_stride = (int)(gridDim.x / 2);
+  auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
+    return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_p, p.status)) != 0;
+  };
+
+  if (warp == 0 || warp == kProducerBWarp) {
+    // ------------------------------------------------------------ TMA producers: warp 0 W, warp 6 X
+    const bool do_w = warp == 0;
+    const uint64_t pol = ptx::l2_policy(2);
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int u = unit0; ok && u < p.total_units; u += unit_stride) {
+      const GroupedUnit w = grouped_unit(p, tab, u);
+      const int half = w.n >> 1;
+      const int f = w.f0 + (int)cta_rank * 128, t = w.t0 + (int)cta_rank * half;
+      int first, second;
+      grouped_boxes(half, first, second);
+      const CUtensorMap* const map1 = &tm.x[__clz(first) - 24];  // (128 rows: map 0, ... 8 rows: map 4)
+      const CUtensorMap* const map2 = &tm.x[second ? __clz(second) - 24 : 0];
+      const uint32_t tx = 2u * (kStageBytesA + (uint32_t)(first + second) * 128u);  // both CTAs' loads complete on the leader's barrier
+      for (int kb = 0; kb < p.k_blocks; ++kb) {
+        if (!wait_all(empty_bar(stage), phase ^ 1u)) {
+          ok = false;
+          break;
+        }
+        const uint32_t sa = smem_base + (uint32_t)stage * p.stage_bytes;
+        if (ptx::elect_one()) {
+          const uint32_t fb = ptx::mapa(full_bar(stage), 0);
+          if (do_w) {
+            if (cta_rank == 0) ptx::mbar_arrive_expect_tx(full_bar(stage), tx);
+            ptx::tma_load_3d_cg2_hint(sa, &tm.w, fb, kb * p.k_elems, f, w.g, pol);
+          } else {
+            ptx::tma_load_3d_cg2_hint(sa + kStageBytesA, map1, fb, kb * p.k_elems, t, 0, pol);
+            if (second) ptx::tma_load_3d_cg2_hint(sa + kStageBytesA + (uint32_t)first * 128u, map2, fb, kb * p.k_elems, t + first, 0, pol);
+          }
+        }
+        if (++stage == p.stages) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+    // every stage this CTA filled has been released: no commit arrival is still on its way when it exits
+    for (int s = 0; ok && do_w && s < p.stages; ++s) {
+      if (!wait_all(empty_bar(stage), phase ^ 1u)) ok = false;
+      if (++stage == p.stages) {
+        stage = 0;
+        phase ^= 1u;
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer (of the leader CTA, for both)
+    auto issue_all = [&](auto fp8_tag) {
+      constexpr bool kFp8 = decltype(fp8_tag)::value;
+      int stage = 0, acc = 0;
+      uint32_t phase = 0, acc_phase = 0;
+      bool ok = true;
+      for (int u = unit0; ok && u < p.total_units; u += unit_stride) {
+        const GroupedUnit w = grouped_unit(p, tab, u);
+        const uint32_t idesc = p.idesc | ((uint32_t)(w.n >> 3) << 17);
+        if (!wait_all(acce_bar(acc), acc_phase ^ 1u)) break;
+        ptx::tc_fence_after();
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kGrpTokens);
+        for (int kb = 0; kb < p.k_blocks; ++kb) {
+          if (!wait_all(full_bar(stage), phase)) {
+            ok = false;
+            break;
+          }
+          ptx::tc_fence_after();
+          const uint32_t sa = smem_base + (uint32_t)stage * p.stage_bytes;
+          const uint64_t adesc = p.desc | (uint64_t)((sa >> 4) & 0x3fffu);
+          const uint64_t bdesc = p.desc | (uint64_t)(((sa + kStageBytesA) >> 4) & 0x3fffu);
+          if (ptx::elect_one()) {
+#pragma unroll
+            for (int k = 0; k < kTileK / kUmmaK; ++k) {  // 32 bytes of K per instruction
+              if constexpr (kFp8) ptx::umma_f8<2>(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+              else ptx::umma_bf16<2>(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            }
+            ptx::umma_commit_pair(empty_bar(stage));
+          }
+          if (++stage == p.stages) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+        if (!ok) break;
+        if (ptx::elect_one()) ptx::umma_commit_pair(accf_bar(acc));
+        acc ^= 1;
+        if (acc == 0) acc_phase ^= 1u;
+      }
+    };
+    if (cta_rank == 0) {
+      if (p.fp8) issue_all(FactTrue{});
+      else issue_all(FactFalse{});
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------ epilogue warps: a lane quarter's features, every other 32 tokens
+    const int q = warp & 3, half = warp >= kEpiSetBWarp0 ? 1 : 0;
+    int acc = 0;
+    uint32_t acc_phase = 0;
+    uint32_t chunks = 0;  // this set's chunks so far: buffer and phase of the exchange
+    bool ok = true;
+    for (int u = unit0; ok && u < p.total_units; u += unit_stride) {
+      const GroupedUnit w = grouped_unit(p, tab, u);
+      const int f_cta = w.f0 + (int)cta_rank * 128;
+      const int f = f_cta + q * 32 + lane;  // this thread's feature
+      float b = 0.f;
+      if constexpr (epi_has_bias<EPI>())
+        if (p.bias != nullptr && f < p.N_out) b = __bfloat162float(p.bias[f]);
+      const uint64_t bias2 = ptx::pack_f32x2(__float_as_uint(b), __float_as_uint(b));
+      if (!wait_all(accf_bar(acc), acc_phase)) break;
+      ptx::tc_fence_after();
+      const uint32_t t_acc = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kGrpTokens);
+      for (int c = half * 32; c < w.n; c += 64) {
+        uint32_t v[32];
+        ptx::tmem_ld_32x32b_x32(t_acc + (uint32_t)c, v);  // (columns from n on: of an earlier unit, stored by nobody)
+        uint32_t r[16];
+        if constexpr (EPI == kEpiBiasResidual) {
+          const int row = w.t0 + c + (lane & 1);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            r[i] = 0u;
+            if (f < p.N_out && row + 2 * i < w.t_end)  // (N_out is even: the pair exists)
+              r[i] = *reinterpret_cast<const uint32_t*>(p.R + (long long)(row + 2 * i) * p.ldr + (f & ~1));
+          }
+        }
+        ptx::tmem_wait_ld();
+        if (p.use_alpha) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * p.alpha);
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {  // tokens c + 2 i and c + 2 i + 1
+          uint64_t res2 = 0ull;
+          if constexpr (EPI == kEpiBiasResidual) res2 = ptx::bf16x2_to_f32x2(transpose_pairs(r[i], lane));
+          ptx::unpack_f32x2(epilogue_pair<EPI>(ptx::pack_f32x2(v[2 * i], v[2 * i + 1]), 0ull, bias2, res2), v[2 * i], v[2 * i + 1]);
+        }
+        if (p.out_f32) {
+          float* dst = reinterpret_cast<float*>(p.C) + (long long)(w.t0 + c) * p.ldc + f;
+#pragma unroll
+          for (int i = 0; i < 32; ++i, dst += p.ldc)
+            if (f < p.N_out && w.t0 + c + i < w.t_end) *dst = __uint_as_float(v[i]);
+          continue;
+        }
+        // rows of 128 features, 16-byte pieces with the lower bit of the row crossed into bit 2 of the piece: the two rows
+        // that a warp's words go to lie in different banks
+        const uint32_t buf = out_base + (uint32_t)(half * 2 + (int)(chunks & 1u)) * kGrpStageOutBytes;
+        const uint32_t mine = buf + (uint32_t)(lane & 1) * kGrpRowBytes +
+                              (((uint32_t)(q * 4 + (lane >> 3)) ^ (uint32_t)((lane & 1) << 2)) << 4) + (uint32_t)((lane >> 1) & 3) * 4u;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const uint32_t o = transpose_pairs(pack_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), lane);
+          asm volatile("st.shared.b32 [%0], %1;" ::"r"(mine + (uint32_t)(2 * i) * kGrpRowBytes), "r"(o) : "memory");
+        }
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(rows_bar(half));
+        // All four warps have written the buffer, and read the other one: each arrives for a chunk after it has read the one before.
+        if (!wait_all(rows_bar(half), chunks & 1u)) {
+          ok = false;
+          break;
+        }
+        ++chunks;
+        const int piece = lane & 15;
+        const bool col_ok = f_cta + piece * 8 < p.N_out;  // (N_out is a multiple of 8)
+        __nv_bfloat16* const dst = reinterpret_cast<__nv_bfloat16*>(p.C) + (long long)(w.t0 + c) * p.ldc + f_cta + piece * 8;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = q * 8 + 2 * i + (lane >> 4);
+          const uint4 o = ptx::ld_shared_v4(buf + (uint32_t)row * kGrpRowBytes + ((uint32_t)(piece ^ ((row & 1) << 2)) << 4));
+          if (col_ok && w.t0 + c + row < w.t_end) *reinterpret_cast<uint4*>(dst + (long long)row * p.ldc) = o;
+        }
+      }
+      if (!ok) break;
+      // hand the accumulator back to the issuer (relaxed, see fact_gemm_kernel)
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive_cluster_relaxed(ptx::mapa(acce_bar(acc), 0));
+      acc ^= 1;
+      if (acc == 0) acc_phase ^= 1u;
+    }
+    __syncwarp();
+  }
+
+  // ------------------------------------------------------------ teardown
+  ptx::grid_launch_dependents();
+  if (*abort_p) {  // a wait expired somewhere: give copies that may still be in flight time to land
+    const unsigned long long t0 = ptx::globaltimer_ns();
+    while (ptx::globaltimer_ns() - t0 < 200000ull) {
+    }
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    long long* stamp = reinterpret_cast<long long*>(p.status + 2);
+    stamp[0] = clock64() - t_clk0;
+    stamp[1] = (long long)(ptx::globaltimer_ns() - t_ns0);
+  }
+  ptx::cluster_arrive();  // neither CTA may free tensor memory or exit while its peer still uses it
+  ptx::cluster_wait();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc<2>(tmem_base, 512);
+  }
+}
+
+}  // namespace fact

@@ -232,3 +232,33 @@ def test_grouped_call_in_a_cuda_graph(h):
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("rows,N,K,epi,out", [
+    ([1, 15, 16, 17, 31, 33], 264, 200, "NONE", "bf16"),             # tiles of 16, 32 and 48 columns, the last features ragged
+    ([255, 256, 257, 0, 272, 500, 513], 520, 136, "BIAS", "bf16"),   # one, two and three even shares; 112 to 256 columns
+    ([96, 112, 144, 176, 208, 240], 256, 64, "BIAS_RELU", "bf16"),   # every split of half a tile into one or two boxes
+    ([60, 300, 7], 129, 72, "NONE", "f32"), ([130, 1], 8, 8, "BIAS", "f32"),
+    ([100, 0, 301], 392, 328, "BIAS_RESIDUAL", "bf16"), ([33, 70], 390, 64, "BIAS_RESIDUAL", "f32"),
+    ([5] * 40, 1032, 1096, "BIAS_GELU_TANH", "bf16"), ([2000], 256, 512, "NONE", "bf16"), ([90] * 256, 64, 64, "NONE", "bf16"),
+], ids=lambda v: "x".join(map(str, v[:4])) if isinstance(v, list) else str(v))
+def test_weights_as_the_wide_operand(h, rows, N, K, epi, out):
+    """Token tiles of every width, at the edges of their columns, boxes and features; both epilogue stores."""
+    run_and_check(h, rows, N, K, epilogue=epi, out_dtype=torch.float32 if out == "f32" else torch.bfloat16, seed=51)
+
+
+@pytest.mark.parametrize("ld,off,N", [(272, 0, 264), (266, 0, 264), (272, 3, 264), (203, 0, 203), (256, 8, 248)])
+def test_grouped_outputs_of_any_alignment(h, ld, off, N):
+    """Rows of whole 16-byte pieces are stored by the warps together; other outputs keep the path that stores any."""
+    rows, K = [70, 0, 150, 1], 96
+    M = sum(rows)
+    X, W = draw((M, K), 61), draw((4, N, K), 62, K ** -0.5)
+    buf = torch.full((M + 4, ld), 7.0, dtype=torch.bfloat16, device="cuda")
+    out = buf.view(-1)[off:off + M * ld].view(M, ld)[:, :N]
+    h.linear_grouped(X.cuda(), W.cuda(), rows, out=out)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    c, t = gates(oracle.linear_grouped(wl.bits(X), wl.bits(W), rows, layout="NK"), to_f64(out.contiguous()), "bf16", "NONE")
+    assert c <= 1.0 and t <= 1.0
+    out.fill_(7.0)
+    assert bool((buf == 7.0).all())
