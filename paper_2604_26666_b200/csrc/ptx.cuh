@@ -238,6 +238,13 @@ __device__ __forceinline__ void tma_load_3d_cg2_hint(uint32_t dst, const void* t
       : "memory");
 }
 
+// `bytes` contiguous bytes (a multiple of 16, both addresses on 16) into this CTA's shared memory.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
 // 4-D tiled load global -> this CTA's shared memory, completion on this CTA's mbarrier.
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2,
                                             int c3) {
