@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(kNormWarps * 32, norm_stream_ctas(CH, RMS)) fa
   if (threadIdx.x == 0) *abort_p = 0;
   __syncthreads();
   ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();  // (a short kernel: the next one's start overlaps all of it)
   const long long first = (long long)blockIdx.x * kNormWarps + warp, stride = (long long)gridDim.x * kNormWarps;
   const int chunks = p.C >> 3;
   const uint32_t bytes = (uint32_t)chunks * 16u;
@@ -234,6 +235,7 @@ __global__ void __launch_bounds__(T, (CH <= 2 ? 1536 : 768) / T) fact_norm_long_
   constexpr int kWarps = T / 32;
   __shared__ float red[2][kWarps];
   ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();  // (a short kernel: the next one's start overlaps all of it)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long row = blockIdx.x;
   const int chunks = p.C >> 3;
