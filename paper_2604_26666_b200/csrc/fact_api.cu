@@ -122,6 +122,7 @@ struct Plan {
   bool kcluster = false;    // the K slices of a tile run as one cluster and are added up through shared memory
   int smem_bytes;
   int grid;
+  int a_rows = kTileM;      // rows of A that one load brings in
   size_t ws_bytes;
   const GroupTable* groups = nullptr;  // grouped: the row groups of the call in flight
   GemmParams p;
@@ -771,7 +772,11 @@ fact_status_t make_plan(fact_handle_t h, const Problem& q, const fact_config_t* 
   }
   p.b_box_bytes = (uint32_t)p.b_box_n * kTileK * 2;
   p.stage_bytes = (uint32_t)stage_bytes_for(c.tile_n, cg);
-  p.tx_bytes = p.stage_bytes * (uint32_t)cg;
+  // Fewer rows than a tile: only they are loaded, not a box of 128 whose other rows are filled with zeros (what the stage
+  // holds there comes out in rows that nobody stores).  Boxes of more than about 100 such rows are slow: FP8, 20 x 4096 -> 6144 14.6 ->
+  // 9.6 us, 20 x 4096 -> 2 x 14336 gated 29.2 -> 23.1 (as 40 rows always were); 100 x 70 x 1000 x 1000 batched 47.5 -> 45.4.
+  plan->a_rows = cg == 1 && q.groups == 0 && q.M < kTileM ? round_up((int)q.M, 8) : kTileM;
+  p.tx_bytes = (p.stage_bytes - (uint32_t)(kTileM - plan->a_rows) * 128u) * (uint32_t)cg;
   // A and W[N x K]: K-major, rows of 128 bytes, 8-row swizzle atoms 1024 bytes apart; 16 K-elements = 32 bytes.
   p.a_desc = smem_desc_template(16, 1024);
   p.a_k_step = 32 >> 4;
@@ -1444,7 +1449,7 @@ fact_status_t run(fact_handle_t h, const Problem& q, const fact_config_t* user, 
     const uint64_t sA = q.batch > 1 ? (uint64_t)q.strideA : (uint64_t)q.lda * (uint64_t)q.M;
     const uint32_t kbox = (uint32_t)q.k_elems();  // 128 bytes of K
     st = encode_map(h, &tmA, q.A, (uint64_t)q.K, (uint64_t)q.M, batch_dim, (uint64_t)q.lda, std::max<uint64_t>(sA, 16),
-                    kbox, kTileM, false, q.fp8);
+                    kbox, (uint32_t)plan.a_rows, false, q.fp8);
     if (st != FACT_OK) return st;
     if (q.layout == FACT_B_KN) {
       const uint64_t sB = b_strided ? (uint64_t)q.strideB : (uint64_t)q.ldb * (uint64_t)q.K;
